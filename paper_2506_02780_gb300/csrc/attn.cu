@@ -707,50 +707,61 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
       }
     } else if (warp == kWarpMma) {
       // ---------- MMA issuer: Q.K^T(0..kSB-1), then P.V(t), Q.K^T(t+kSB) ----------
-      if (lane == 0) {
+      // the whole warp walks the loop (wait outcomes made warp-uniform) and one
+      // elected lane issues, with every descriptor an offset from a uniform base
+      tc_fence_after();
+      const uint32_t id_qk = idesc_f16(kRows, kKT, 1, 1, 0);
+      const uint32_t id_pv = idesc_f16(kRows, kD, 1, 1, 1);
+      const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+      const uint64_t dq = smem_desc_sw128(__shfl_sync(0xffffffffu, sbase + kOffQ, 0));
+      const uint64_t dk0 = smem_desc_sw128(__shfl_sync(0xffffffffu, sK, 0));
+      const uint64_t dv0 = smem_desc_sw128_mn(__shfl_sync(0xffffffffu, sV, 0), kKVHalf, 1024);
+      auto wait = [&](uint32_t bar, int use) -> bool {
+        return __all_sync(0xffffffffu, mbar_wait(bar, (uint32_t)(use & 1), &s_abort));
+      };
+      auto issue_qk = [&](int t) -> bool {
+        const int tg = tb + t;
+        const int st = tg % kKST, sb = tg % kSB;
+        if (!wait(k_full + 8 * st, tg / kKST)) return false;
         tc_fence_after();
-        const uint32_t id_qk = idesc_f16(kRows, kKT, 1, 1, 0);
-        const uint32_t sQ = sbase + kOffQ;
-        const uint32_t id_pv = idesc_f16(kRows, kD, 1, 1, 1);
-        auto issue_qk = [&](int t) -> bool {
-          const int tg = tb + t;
-          if (!mbar_wait(k_full + 8 * (tg % kKST), (uint32_t)((tg / kKST) & 1), &s_abort)) return false;
-          tc_fence_after();
-          const uint32_t kb = sK + (tg % kKST) * kKVBytes;
+        if (elect_one()) {
+          const uint64_t dk = dk0 + (uint64_t)(st * (kKVBytes >> 4));
 #pragma unroll
           for (int kk = 0; kk < kD / 16; ++kk) {
-            const uint32_t off = (kk & 3) * 32;
-            tc_mma(tmem + (tg % kSB) * kKT, smem_desc_sw128(sQ + (kk >> 2) * kKVHalf + off),
-                   smem_desc_sw128(kb + (kk >> 2) * kKVHalf + off), id_qk, kk > 0 ? 1u : 0u);
+            const uint64_t off = ((kk >> 2) * kKVHalf + (kk & 3) * 32) >> 4;
+            tc_mma(tm + sb * kKT, dq + off, dk + off, id_qk, kk > 0 ? 1u : 0u);
           }
-          tc_commit(k_empty + 8 * (tg % kKST));
-          tc_commit(s_full + 8 * (tg % kSB));
-          return true;
-        };
-        bool ok = mbar_wait(q_ready, (uint32_t)(nseg & 1), &s_abort);
-        for (int t = 0; t < kSB && t < n_tiles && ok; ++t) ok = issue_qk(t);
-        for (int t = 0; t < n_tiles && ok; ++t) {
-          const int tg = tb + t;
-          if (!mbar_wait(p_full + 8 * (tg % kSB), (uint32_t)((tg / kSB) & 1), &s_abort) ||
-              !mbar_wait(v_full + 8 * (tg % kVST), (uint32_t)((tg / kVST) & 1), &s_abort))
-            break;
-          tc_fence_after();
-          const uint32_t pa = tmem + (tg % kSB) * kKT;       // bf16 P head: cols 0..63, tail: 64..127
-          const uint32_t vb = sV + (tg % kVST) * kKVBytes;
+          tc_commit(k_empty + 8 * st);
+          tc_commit(s_full + 8 * sb);
+        }
+        __syncwarp();
+        return true;
+      };
+      bool ok = wait(q_ready, nseg);
+      for (int t = 0; t < kSB && t < n_tiles && ok; ++t) ok = issue_qk(t);
+      for (int t = 0; t < n_tiles && ok; ++t) {
+        const int tg = tb + t;
+        const int st = tg % kVST, sb = tg % kSB;
+        if (!wait(p_full + 8 * sb, tg / kSB) || !wait(v_full + 8 * st, tg / kVST)) break;
+        tc_fence_after();
+        if (elect_one()) {
+          const uint32_t pa = tm + sb * kKT;       // bf16 P head: cols 0..63, tail: 64..127
+          const uint64_t dv = dv0 + (uint64_t)(st * (kKVBytes >> 4));
 #pragma unroll
           for (int part = 0; part < 2; ++part)
 #pragma unroll
             for (int j = 0; j < kKT / 16; ++j)
-              tc_mma_ts(tmem + kColO, pa + 64 * part + 8 * j,
-                        smem_desc_sw128_mn(vb + j * 2048, kKVHalf, 1024), id_pv,
+              tc_mma_ts(tm + kColO, pa + 64 * part + 8 * j, dv + (uint64_t)(j * (2048 >> 4)), id_pv,
                         (t > 0 || part > 0 || j > 0) ? 1u : 0u);
-          tc_commit(v_empty + 8 * (tg % kVST));
+          tc_commit(v_empty + 8 * st);
           tc_commit(o_done + 8 * (tg & 1));
-          if (t + kSB < n_tiles) ok = issue_qk(t + kSB);
         }
-        // one phase per segment: every product of the segment is complete
-        if (n_tiles > 0) tc_commit(o_final);
+        __syncwarp();
+        if (t + kSB < n_tiles) ok = issue_qk(t + kSB);
       }
+      // one phase per segment: every product of the segment is complete
+      if (n_tiles > 0 && elect_one()) tc_commit(o_final);
+      __syncwarp();
     } else if (warp >= kWarpSoft0) {
       // ---------------- softmax: one query row and half of every tile per thread ----------------
       // Warps w and w + 4 share TMEM lane quarter w & 3 (32 query rows); half hf
@@ -1032,7 +1043,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
       if (s_vissued[st] >= 0) mbar_wait_plain(v_full + 8 * st, (uint32_t)(s_vissued[st] & 1));
   }
   if (warp == kWarpMma) {
-    if (aborted && lane == 0) {
+    if (aborted && elect_one()) {   // the lane that issued the MMAs
       tc_commit(drain);
       mbar_wait_plain(drain, 0);
     }

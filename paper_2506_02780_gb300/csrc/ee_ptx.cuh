@@ -96,6 +96,19 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// One lane of a converged warp (elect.sync picks the same lane every time for
+// the same mask).  An MMA loop that the whole warp runs, with only the MMAs and
+// commits under elect_one(), keeps its descriptors in uniform registers; under
+// `lane == 0` each operand of each MMA is moved there one by one, which is slower
+// than the tensor pipe once other warps take issue slots (24 MMAs of 128x128x16
+// beside eight softmax warps: 2169 cycles against 1807, 1536 of them pipe time).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok));
+  return ok != 0;
+}
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"

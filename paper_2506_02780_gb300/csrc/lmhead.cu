@@ -410,40 +410,46 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(BM, BN);
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      int lt = 0;
-      for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++lt) {
-        const int acc = lt & 1;
-        const uint32_t acc_phase = (lt >> 1) & 1;
-        if (!mbar_wait(tempty0 + 8 * acc, acc_phase ^ 1, &s_abort)) break;
+    // the whole warp walks the loop (wait outcomes made warp-uniform) and one
+    // elected lane issues the MMAs, every descriptor an offset from a uniform base
+    const uint32_t idesc = idesc_bf16(BM, BN);
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
+    const uint64_t ad0 = smem_desc_sw128(__shfl_sync(0xffffffffu, smem_u32(sA), 0));
+    const uint64_t bd0 = smem_desc_sw128(__shfl_sync(0xffffffffu, smem_u32(sB), 0));
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    int lt = 0, consumed = 0;
+    for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++lt) {
+      const int acc = lt & 1;
+      const uint32_t acc_phase = (lt >> 1) & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(tempty0 + 8 * acc, acc_phase ^ 1, &s_abort))) break;
+      tc_fence_after();
+      const uint32_t d_tmem = tm + (uint32_t)(acc * BN);
+      for (int kb = 0; kb < p.nkb; ++kb) {
+        if (!__all_sync(0xffffffffu, mbar_wait(full0 + 8 * stage, phase, &s_abort))) {
+          ok = false;
+          break;
+        }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-        for (int kb = 0; kb < p.nkb; ++kb) {
-          if (!mbar_wait(full0 + 8 * stage, phase, &s_abort)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint64_t ad = smem_desc_sw128(smem_u32(sA + (size_t)stage * kABytes));
-          const uint64_t bd = smem_desc_sw128(smem_u32(sB + (size_t)stage * bBytes));
+        if (elect_one()) {
+          const uint64_t ad = ad0 + (uint64_t)(stage * (kABytes >> 4));
+          const uint64_t bd = bd0 + (uint64_t)(stage * (bBytes >> 4));
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
-            tc_mma(d_tmem, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc,
-                   (kb | k) != 0 ? 1u : 0u);
+            tc_mma(d_tmem, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kb | k) != 0 ? 1u : 0u);
           tc_commit(empty0 + 8 * stage);
-          ++s_consumed;
-          if (++stage == S) {
-            stage = 0;
-            phase ^= 1;
-          }
+          if (kb == p.nkb - 1) tc_commit(tfull0 + 8 * acc);
         }
-        if (ok) tc_commit(tfull0 + 8 * acc);
+        __syncwarp();
+        ++consumed;
+        if (++stage == S) {
+          stage = 0;
+          phase ^= 1;
+        }
       }
     }
+    if (lane == 0) s_consumed = consumed;
   } else {
     // epilogue warps 2..5: TMEM lane quarter = warp % 4
     const int q = warp & 3;                 // TMEM lane quarter
@@ -687,7 +693,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
     }
   }
   if (warp == 1) {
-    if (aborted && lane == 0) {
+    if (aborted && elect_one()) {   // the lane that issued the MMAs
       tc_commit(drain);
       mbar_wait_plain(drain, 0);
     }
