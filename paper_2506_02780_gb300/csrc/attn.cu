@@ -90,13 +90,13 @@ constexpr int kVST = 2;                          // V ring depth
 constexpr int kSB = 3;                           // S buffers in TMEM (Q.K^T runs kSB tiles ahead)
 constexpr uint32_t kKVHalf = kKT * 128;          // 16 KB: one 64-dim half of a K or V tile
 constexpr uint32_t kKVBytes = 2 * kKVHalf;       // 32 KB
-constexpr int kMaxCtaPages = 2048;               // context pages one CTA can own (32768 keys)
+constexpr int kMaxCtaPages = 2048;               // context pages one CTA owns at most (32768 keys)
+constexpr int kMaskRing = 8;                     // page-validity masks in flight (K runs at most 6 tiles ahead)
 constexpr uint32_t kOffK = 0;
 constexpr uint32_t kOffV = kOffK + kKST * kKVBytes;
 constexpr uint32_t kOffQ = kOffV + kVST * kKVBytes;  // Q block, 128 rows x 128 bf16, SW128 K-major
-constexpr uint32_t kOffPages = kOffQ + kKVBytes;
-constexpr uint32_t kOffBar = kOffPages + 4 * kMaxCtaPages;
-constexpr uint32_t kNumBars = 2 * kKST + 2 * kVST + 2 * kSB + 2 + 3;
+constexpr uint32_t kOffBar = kOffQ + kKVBytes;
+constexpr uint32_t kNumBars = 2 * kKST + 2 * kVST + 3 * kSB + 5;
 constexpr uint32_t kSmemBytes = 1024 + kOffBar + 8 * kNumBars + 64;
 constexpr uint32_t kTmemCols = 512;              // S0 [0,128) S1 [128,256) S2 [256,384) O [384,512)
 constexpr uint32_t kColO = 384;
@@ -104,13 +104,12 @@ constexpr float kRescaleLog2 = 8.0f;
 constexpr int kMaxCluster = 8;                   // portable thread-block cluster size
 constexpr int kMaxSplits = ee::kAttnMaxSplits;   // chunks per row block (cooperative launch)
 constexpr int kMaxBalSeqs = 512;                 // sequences of a balanced launch
-// warp roles (warp 3 is idle after set-up); softmax warps 4..11, two per TMEM
-// lane quarter
-constexpr int kWarpK = 0, kWarpMma = 1, kWarpV = 2, kWarpSched = 3, kWarpSoft0 = 4;
-constexpr int kSoftThreads = 8 * 32;
+// warp roles; softmax warps 4..11, two per TMEM lane quarter
+constexpr int kWarpK = 0, kWarpPv = 1, kWarpV = 2, kWarpQk = 3, kWarpSoft0 = 4;
+constexpr int kSoftWarps = 8;
 
 static_assert(kRows == ee::kAttnRows, "row block size");
-static_assert(kThreads == 32 * kWarpSoft0 + kSoftThreads, "eight softmax warps, two per TMEM lane quarter");
+static_assert(kThreads == 32 * (kWarpSoft0 + kSoftWarps), "eight softmax warps, two per TMEM lane quarter");
 static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 static_assert(ee::kAttnMlOff == kRows * kD * 4, "partial slot: O rows, then (m, l), then counters");
 
@@ -126,6 +125,7 @@ struct AttnParams {
   int num_pages, max_pages, max_ctx, n_q, n_kv, g, total_nodes, max_T, nrb, chunk, S;
   int coop;                    // 1: cooperative launch, counters; 0: cluster barrier
   int B;                       // sequences (the balanced mode's work list)
+  uint32_t g_inv;              // ceil(2^32 / g) for g > 1 (row -> node without a division), 0 for g = 1
   float scale_log2;
 };
 
@@ -145,19 +145,6 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   float r;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
-}
-
-// Loaded-page mask of context tile t: bit i set when the tile's 16-row block i
-// holds keys below k_end in a valid page.  s_pages holds the CTA's page ids
-// (-1 for an out-of-range block-table entry).
-__device__ __forceinline__ unsigned tile_mask(const int32_t* s_pages, int t, int k_begin, int k_end) {
-  unsigned m = 0u;
-#pragma unroll
-  for (int i = 0; i < kKT / 16; ++i) {
-    const int pos = k_begin + t * kKT + 16 * i;
-    m |= (pos < k_end && s_pages[t * (kKT / 16) + i] >= 0) ? (1u << i) : 0u;
-  }
-  return m;
 }
 
 // Merge rows [r0, r0 + nown) of a row block (query rows row0, ...) from its S
@@ -204,7 +191,7 @@ __device__ __forceinline__ void merge_rows(const AttnParams& p, size_t slot_a, s
     w[s] = ml[s].x == -INFINITY ? 0.f : ex2(ml[s].x - M);
     L += w[s] * ml[s].y;
   }
-  const float il = L > 0.f ? 1.f / L : 0.f;
+  const float il = L == 0.f ? 0.f : 1.f / L;   // NaN scores stay NaN
   const int rrow = row0 + j;
   const int nd = rrow / p.g;
   float4* dst = reinterpret_cast<float4*>(p.out + ((size_t)(o + nd) * p.n_q + hk * p.g + (rrow - nd * p.g)) * kD);
@@ -259,6 +246,194 @@ __host__ __device__ inline int chain_rb_tiles(int ctx, int T, int g, int r) {
   return (ctx + n_hi + 1 + kKT - 1) / kKT;
 }
 
+// node of query row r, r / g by a multiplication: with g_inv = (2^32 + e) / g and
+// e < g it is exact while r * e < 2^32, and r < EE_MAX_CHAIN * g holds that for
+// g <= 1024
+__device__ __forceinline__ int row_node(const AttnParams& p, int r) {
+  if (p.g == 1) return r;
+  return p.g <= 1024 ? (int)__umulhi((uint32_t)r, p.g_inv) : r / p.g;
+}
+
+// One segment: a contiguous range of one row block's tiles, run in the order
+// rot, rot + 1, ..., n_tiles - 1, 0, ..., rot - 1.  Every role decodes the
+// CTA's segments by itself (same inputs, same result), so no CTA barrier
+// separates one segment from the next.
+struct Seg {
+  int b, hk, rb, o, T, ctx;    // sequence, KV head, row block, node offset, nodes, context length
+  int k_begin, k_end;          // paged keys
+  int n_ctx, n_tiles, rot;     // context tiles, all tiles (the tree tile last), first tile
+  bool alone;                  // the segment is its whole row block
+  int slot;                    // partial slot (alone: unused)
+  int y;                       // balanced: where the segment starts in the work list
+  int c0, c1, slot0;           // balanced: CTAs holding the unit's first and last tiles, piece 0's slot
+};
+
+// Shared state of a CTA's work: balanced mode, per sequence (node offset, T,
+// context length, tiles), the exclusive prefix of the sequences' work in
+// tiles, and (range start, range end, W, N).
+struct WorkList {
+  const int4* seq;
+  const int* wpre;
+  const int* sched;
+};
+
+// The segment of the balanced work list that ends at y (this CTA's range is
+// walked from its end); tb: tiles the CTA ran before it.  Whole warp.
+template <int kKV>
+__device__ __forceinline__ void bal_segment(const AttnParams& p, const WorkList& w, int y, int tb, int lane, Seg& s) {
+  constexpr bool kIP = kKV != kKVTree;
+  constexpr bool kChain = kKV == kKVChain;
+  const int g = p.g;
+  // The CTA walks its range from the end: its last segment (the head of a
+  // row block) first.  Within a segment the tiles run rotated so that the
+  // CTA reads tile x of a row block at about its local time x mod P (P =
+  // the share): the CTAs holding other row blocks of the same KV head then
+  // read the same K/V tiles at about the same time, and L2 serves the
+  // repeats (each KV head's tiles are read by all its row blocks).
+  const int x_begin = w.sched[0], W = w.sched[2], N = w.sched[3];
+  int lo = 0, hi = p.B;   // wpre[lo] <= y - 1 < wpre[hi]
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (w.wpre[mid] <= y - 1) lo = mid; else hi = mid;
+  }
+  s.b = lo;
+  const int4 sq = w.seq[lo];
+  s.o = sq.x;
+  s.T = sq.y;
+  s.ctx = sq.z;
+  int tiles = sq.w;
+  int U0;                                        // the unit's first tile in the work list
+  const int base_w = w.wpre[lo];
+  const int nrb_b = (s.T * g + kRows - 1) / kRows;
+  if constexpr (kChain) {
+    // sq.w = tiles of one KV head's row blocks; row block r has chain_rb_tiles
+    const int local = y - 1 - base_w;
+    s.hk = local / tiles;
+    const int rem = local - s.hk * tiles;
+    // the row block holding tile rem: a scan of the row blocks' tile counts, 32 at a time
+    int r = nrb_b - 1, cum = 0, tu = 0;
+    for (int r0 = 0, base = 0; r0 < nrb_b; r0 += 32) {
+      const int rr = r0 + lane;
+      const int t = rr < nrb_b ? chain_rb_tiles(s.ctx, s.T, g, rr) : 0;
+      int incl = t;
+#pragma unroll
+      for (int dd = 1; dd < 32; dd <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, dd);
+        if (lane >= dd) incl += v;
+      }
+      const int excl = base + incl - t;
+      const unsigned hit = __ballot_sync(0xffffffffu, rr < nrb_b && rem >= excl && rem < excl + t);
+      if (hit) {
+        const int src = __ffs(hit) - 1;
+        r = r0 + src;
+        cum = __shfl_sync(0xffffffffu, excl, src);
+        tu = __shfl_sync(0xffffffffu, t, src);
+        break;
+      }
+      base += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (tu == 0) {   // not reached for a consistent work list
+      cum = 0;
+      for (int q = 0; q < r; ++q) cum += chain_rb_tiles(s.ctx, s.T, g, q);
+      tu = chain_rb_tiles(s.ctx, s.T, g, r);
+    }
+    s.rb = r;
+    U0 = base_w + s.hk * tiles + cum;
+    tiles = tu;
+  } else {
+    const int u = (y - 1 - base_w) / tiles;
+    s.hk = u / nrb_b;
+    s.rb = u - s.hk * nrb_b;
+    U0 = base_w + u * tiles;
+  }
+  const int seg0 = max(U0, x_begin);
+  const int t0 = seg0 - U0;
+  const int len = y - seg0;
+  const int n_ctx_b = kIP ? tiles : tiles - 1;   // paged tiles of the unit
+  s.k_begin = min(t0, n_ctx_b) * kKT;
+  const int unit_span =
+      kChain ? s.ctx + min(s.T, ((s.rb + 1) * kRows - 1) / g + 1) : (kIP ? s.ctx + s.T : s.ctx);
+  s.k_end = t0 < n_ctx_b ? min(unit_span, min(t0 + len, n_ctx_b) * kKT) : s.k_begin;
+  s.n_ctx = s.k_end > s.k_begin ? (s.k_end - s.k_begin + kKT - 1) / kKT : 0;
+  s.n_tiles = s.n_ctx + (!kIP && t0 + len == tiles ? 1 : 0);
+  const int P = (W + N - 1) / N;
+  int ph = (tb - t0) % P;
+  ph += ph < 0 ? P : 0;
+  s.rot = ph < len ? ph : 0;
+  // the CTAs holding the unit's first and last tiles
+  s.c0 = ((U0 + 1) * N - 1) / W;
+  s.c1 = ((U0 + tiles) * N - 1) / W;
+  s.alone = s.c0 == s.c1;
+  s.slot0 = 2 * s.c0 + (U0 > s.c0 * W / N ? 1 : 0);
+  // a piece starts the CTA's range (slot 2c) or ends it (slot 2c + 1)
+  s.slot = 2 * (int)blockIdx.x + (seg0 > x_begin ? 1 : 0);
+  s.y = seg0;
+}
+
+// The one (row block, chunk) of a CTA of a uniform launch; false when the row
+// block has no work (uniform over the row block's CTAs).
+template <int kKV>
+__device__ __forceinline__ bool uni_segment(const AttnParams& p, bool report, Seg& s) {
+  constexpr bool kIP = kKV != kKVTree;
+  constexpr bool kChain = kKV == kKVChain;
+  constexpr int kMaxT = kChain ? EE_MAX_CHAIN : EE_MAX_TREE;
+  s.b = blockIdx.z;
+  s.hk = blockIdx.y;
+  s.rb = blockIdx.x / p.S;                     // the S chunks of a row block are consecutive
+  const int split = blockIdx.x - s.rb * p.S;
+  s.o = p.node_off[s.b];
+  s.T = p.node_off[s.b + 1] - s.o;
+  s.ctx = p.ctx_len[s.b];
+  const bool bad_tree = s.T < 1 || s.T > kMaxT || s.T > p.max_T || s.o < 0 || s.o + s.T > p.total_nodes;
+  report = report && blockIdx.x == 0 && s.hk == 0;
+  if (bad_tree && report) flag_error(p.err, EE_DEVERR_TREE);
+  if (bad_tree || s.rb * kRows >= s.T * p.g) return false;
+  if (s.ctx < 0 || s.ctx > p.max_ctx) {
+    if (report) flag_error(p.err, EE_DEVERR_CTX);
+    s.ctx = s.ctx < 0 ? 0 : p.max_ctx;
+  }
+  // everything above is uniform over the row block's CTAs; from here on every
+  // CTA reaches the merge synchronisation
+  // paged keys of the row block (chain: up to its last node's position)
+  const int span = kChain ? s.ctx + min(s.T, ((s.rb + 1) * kRows - 1) / p.g + 1) : (kIP ? s.ctx + s.T : s.ctx);
+  const int S = attn_splits_for(span, p.chunk);  // chunks this sequence uses, <= p.S
+  const bool active = split < S;
+  s.k_begin = split * p.chunk;
+  s.k_end = active ? min(span, s.k_begin + p.chunk) : s.k_begin;
+  s.n_ctx = s.k_end > s.k_begin ? (s.k_end - s.k_begin + kKT - 1) / kKT : 0;
+  s.n_tiles = s.n_ctx + (!kIP && active && split == S - 1 ? 1 : 0);
+  s.rot = 0;
+  s.alone = p.S == 1;
+  s.slot = (int)(((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
+  s.y = 0;
+  return true;
+}
+
+// Row block rows [2 * first, ...) of Q into shared memory as the A operand of
+// Q.K^T, by warps first, first + n, ... of n (a half-warp copies one 256-byte
+// row): 128 rows x 128 bf16 in two 64-column slabs, 128-byte swizzled K-major
+// (the layout TMA gives the K tiles): 16-byte chunk j of row r at slab (j / 8),
+// (r / 8) * 1024 + (r % 8) * 128 + ((j % 8) ^ (r % 8)) * 16; rows past R are
+// zero.  Asynchronous copies: every row is in flight before the first wait.
+template <int kN>
+__device__ __forceinline__ void load_q(const AttnParams& p, const Seg& s, uint32_t sQ, int first, int lane) {
+  const int R = s.T * p.g;
+  const int j = lane & 15;
+  const __nv_bfloat16* base = p.q + ((size_t)s.o * p.n_q + s.hk * p.g) * kD + 8 * j;
+#pragma unroll 8
+  for (int k = 0; k < kRows / 2 / kN; ++k) {
+    const int rq = 2 * (first + kN * k) + (lane >> 4);   // 0..127
+    const int rr = s.rb * kRows + rq;
+    const int rc = min(rr, R - 1);
+    const int nd = row_node(p, rc);
+    cp_async16(sQ + (j >> 3) * kKVHalf + (rq >> 3) * 1024 + (rq & 7) * 128 + (((j & 7) ^ (rq & 7)) << 4),
+               base + ((size_t)nd * p.n_q + (rc - nd * p.g)) * kD, rr < R ? 16u : 0u);
+  }
+  cp_async_wait_all();
+  fence_async_smem();   // generic-proxy writes, read by the tensor core
+  __syncwarp();
+}
+
 // kBal: balanced work list (else one (row block, chunk) per CTA).
 template <bool kBal, int kKV>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -274,24 +449,25 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ int s_kissued[kKST], s_vissued[kVST];
-  __shared__ float s_xmax[2][2][kRows];             // [tile parity][half][row]: softmax pair exchange
+  __shared__ uint32_t s_xmax[2][2][kRows];          // [tile parity][half][row]: softmax pair exchange
   __shared__ float s_xl[2][kRows];                  // [half][row]: final row sums
-  // balanced mode: per sequence (node offset, T, context length, tiles) and the
-  // exclusive prefix of the sequences' work in tiles
+  __shared__ int s_xok[2][4][2];                    // [tile parity][lane quarter][half]: "this half's wait ended well"
+  __shared__ uint32_t s_mask[kMaskRing];            // per tile: 16-row blocks with keys in a valid page
   __shared__ int4 s_seq[kBal ? kMaxBalSeqs : 1];
   __shared__ int s_wpre[kBal ? kMaxBalSeqs + 1 : 1];
-  __shared__ int s_sched[7];   // balanced: range start, range end, W, N, tiles done, segments done, next end
-  __shared__ BalPiece s_pc[2];                      // balanced: this CTA's pieces of split units
+  __shared__ int s_sched[4];                        // balanced: range start, range end, W, N
+  __shared__ BalPiece s_pc[2];                      // this CTA's pieces of split row blocks
   __shared__ int s_npc;
+  __shared__ int2 s_uni;                            // uniform: the row block's node offset and rows
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t sbase = smem_u32(smem);
-  const uint32_t sK = sbase + kOffK, sV = sbase + kOffV;
+  const uint32_t sK = sbase + kOffK, sV = sbase + kOffV, sQ = sbase + kOffQ;
   const uint32_t bar0 = sbase + kOffBar;
   const uint32_t k_full = bar0, k_empty = k_full + 8 * kKST;
   const uint32_t v_full = k_empty + 8 * kKST, v_empty = v_full + 8 * kVST;
-  const uint32_t s_full = v_empty + 8 * kVST, p_full = s_full + 8 * kSB, o_done = p_full + 8 * kSB;
-  const uint32_t drain = o_done + 16, q_ready = drain + 8, o_final = q_ready + 8;
+  const uint32_t s_full = v_empty + 8 * kVST, p_full = s_full + 8 * kSB, pv_done = p_full + 8 * kSB;
+  const uint32_t drain = pv_done + 8 * kSB, q_ready = drain + 16, q_empty = q_ready + 8, o_free = q_empty + 8;
 
   // on-chip set-up first: it touches no global memory, so it overlaps the end
   // of the previous kernel in the stream
@@ -302,6 +478,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmVt)) : "memory");
     s_abort = 0;
     s_npc = 0;
+    s_uni = make_int2(0, 0);
     for (int i = 0; i < kKST; ++i) {
       mbar_init(k_full + 8 * i, 1);
       mbar_init(k_empty + 8 * i, 1);
@@ -313,23 +490,29 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
       s_vissued[i] = -1;
     }
     for (int i = 0; i < kSB; ++i) {
-      mbar_init(s_full + 8 * i, 1);
-      mbar_init(p_full + 8 * i, 2 * kRows);
+      mbar_init(s_full + 8 * i, 2);
+      mbar_init(p_full + 8 * i, kSoftWarps);
+      mbar_init(pv_done + 8 * i, 1);
     }
-    for (int i = 0; i < 2; ++i) mbar_init(o_done + 8 * i, 1);
     mbar_init(drain, 1);
-    mbar_init(q_ready, 2 * kRows);
-    mbar_init(o_final, 1);
+    mbar_init(drain + 8, 1);
+    mbar_init(q_ready, kSoftWarps);
+    mbar_init(q_empty, 1);
+    mbar_init(o_free, kSoftWarps);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
-  if (warp == kWarpMma) {
+  if (warp == kWarpPv) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&s_tmem)),
                  "r"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
 
   pdl_wait();   // no global access before the previous kernel's writes are visible
   const int g = p.g;
@@ -342,9 +525,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   // start the next (at most two of its segments are pieces of split units).
   // N is capped so that every CTA gets at least m = max(2, ceil(t_max / 14))
   // tiles, which bounds the pieces of any unit by 15.
-  // Warp 3 (otherwise idle) builds it: lane l takes sequences [16 l, 16 l + 16).
+  // Warp kWarpQk builds it: lane l takes sequences [16 l, 16 l + 16).
   if constexpr (kBal) {
-    if (warp == kWarpSched) {
+    if (warp == kWarpQk) {
       constexpr int kPer = kMaxBalSeqs / 32;
       int wl[kPer];
       int wsum = 0, tmax = 0;
@@ -431,439 +614,315 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
         s_sched[1] = mine ? ((int)blockIdx.x + 1) * W / N : 0;
         s_sched[2] = W;
         s_sched[3] = N;
-        s_sched[4] = 0;
-        s_sched[5] = 0;
-        s_sched[6] = s_sched[1];
         s_wpre[p.B] = W;
       }
     }
     __syncthreads();
   }
 
-  const int qhalf = lane >> 4, qc = lane & 15;
-  int32_t* s_pages = reinterpret_cast<int32_t*>(smem + kOffPages);
-  uint32_t tmem = 0;
-  bool skip = false;          // uniform mode: the row block has no work
-  // uniform mode: the (row block, chunk) of this CTA, and the row block's node
-  // offset and rows for the merge
-  const int split = kBal ? 0 : (int)(blockIdx.x % p.S);   // == cluster rank in the cluster mode
-  int u_o = 0, u_R = 0;
-  // uniform cooperative mode, thread 0: the row block's count as read at the
-  // start (the target is the next multiple of kCountGen)
-  unsigned long long u_target = 0;
-
-  for (;;) {
-    // ---------------- the next segment of this CTA's work ----------------
-    constexpr int kPgPerThread = (kMaxCtaPages + kThreads - 1) / kThreads;
-    int b, hk, rb, o, T, ctx, k_begin, k_end;
-    bool with_tree, alone;
-    size_t slot;
-    int32_t pgr[kPgPerThread];
-    int x_next = 0;
-    int rot = 0;                // tiles run in the order rot, rot + 1, ..., n_tiles - 1, 0, ..., rot - 1
-    // tiles this CTA processed before this segment (ring slots and phases count
-    // over all segments), and the segments done; kept in shared memory so that
-    // no register carries them across the softmax loop
-    const int tb = kBal ? s_sched[4] : 0;
-    const int nseg = kBal ? s_sched[5] : 0;
+  const WorkList wlist{s_seq, s_wpre, s_sched};
+  // The CTA's segments, decoded by each role: `first` starts the walk, `next`
+  // moves to the following segment (tiles before it: tb, segments before it: nseg).
+  Seg sg;
+  int tb = 0, nseg = 0;
+  auto first = [&](bool report) -> bool {
     if constexpr (kBal) {
-      // The CTA walks its range from the end: its last segment (the head of a
-      // row block) first.  Within a segment the tiles run rotated so that the
-      // CTA reads tile x of a row block at about its local time x mod P (P =
-      // the share): the CTAs holding other row blocks of the same KV head then
-      // read the same K/V tiles at about the same time, and L2 serves the
-      // repeats (each KV head's tiles are read by all its row blocks).
-      const int x_begin = s_sched[0], y = s_sched[6], W = s_sched[2], N = s_sched[3];
-      if (y <= x_begin) break;
-      int lo = 0, hi = p.B;   // s_wpre[lo] <= y - 1 < s_wpre[hi]
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (s_wpre[mid] <= y - 1) lo = mid; else hi = mid;
-      }
-      b = lo;
-      const int4 sq = s_seq[b];
-      o = sq.x;
-      T = sq.y;
-      ctx = sq.z;
-      int tiles = sq.w;
-      int U0;                                        // the unit's first tile in the work list
-      if constexpr (kChain) {
-        // sq.w = tiles of one KV head's row blocks; row block r has chain_rb_tiles
-        const int local = y - 1 - s_wpre[b];
-        hk = local / tiles;
-        const int rem = local - hk * tiles;
-        // the row block holding tile rem: every warp scans the row blocks' tile
-        // counts 32 at a time (a warp prefix sum; all warps reach the same answer)
-        const int nrb_b = (T * g + kRows - 1) / kRows;
-        int r = nrb_b - 1, cum = 0, tu = 0;
-        for (int r0 = 0, base = 0; r0 < nrb_b; r0 += 32) {
-          const int rr = r0 + lane;
-          const int t = rr < nrb_b ? chain_rb_tiles(ctx, T, g, rr) : 0;
-          int incl = t;
-#pragma unroll
-          for (int dd = 1; dd < 32; dd <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, dd);
-            if (lane >= dd) incl += v;
-          }
-          const int excl = base + incl - t;
-          const unsigned hit = __ballot_sync(0xffffffffu, rr < nrb_b && rem >= excl && rem < excl + t);
-          if (hit) {
-            const int src = __ffs(hit) - 1;
-            r = r0 + src;
-            cum = __shfl_sync(0xffffffffu, excl, src);
-            tu = __shfl_sync(0xffffffffu, t, src);
-            break;
-          }
-          base += __shfl_sync(0xffffffffu, incl, 31);
-        }
-        if (tu == 0) {   // not reached for a consistent work list
-          cum = 0;
-          for (int q = 0; q < r; ++q) cum += chain_rb_tiles(ctx, T, g, q);
-          tu = chain_rb_tiles(ctx, T, g, r);
-        }
-        rb = r;
-        U0 = s_wpre[b] + hk * tiles + cum;
-        tiles = tu;
-      } else {
-        const int nrb_b = (T * g + kRows - 1) / kRows;
-        const int u = (y - 1 - s_wpre[b]) / tiles;
-        hk = u / nrb_b;
-        rb = u - hk * nrb_b;
-        U0 = s_wpre[b] + u * tiles;
-      }
-      const int seg0 = max(U0, x_begin);
-      const int t0 = seg0 - U0;
-      const int len = y - seg0;
-      const int n_ctx_b = kIP ? tiles : tiles - 1;   // paged tiles of the unit
-      k_begin = min(t0, n_ctx_b) * kKT;
-      const int unit_span = kChain ? ctx + min(T, ((rb + 1) * kRows - 1) / g + 1) : (kIP ? ctx + T : ctx);
-      k_end = t0 < n_ctx_b ? min(unit_span, min(t0 + len, n_ctx_b) * kKT) : k_begin;
-      with_tree = !kIP && t0 + len == tiles;
-      const int P = (W + N - 1) / N;
-      int ph = (tb - t0) % P;
-      ph += ph < 0 ? P : 0;
-      rot = ph < len ? ph : 0;
-      // the CTAs holding the unit's first and last tiles
-      const int c0 = ((U0 + 1) * N - 1) / W;
-      const int c1 = ((U0 + tiles) * N - 1) / W;
-      alone = c0 == c1;
-      // a piece starts the CTA's range (slot 2c) or ends it (slot 2c + 1)
-      slot = 2 * (size_t)blockIdx.x + (seg0 > x_begin ? 1 : 0);
-      if (!alone && threadIdx.x == 0 && s_npc < 2) {
-        const int start0 = c0 * W / N;
-        const int slot0 = 2 * c0 + (U0 > start0 ? 1 : 0);
-        const unsigned long long c = ld_acquire64(
-            reinterpret_cast<const unsigned long long*>(p.part + (size_t)slot0 * kAttnPartBytes + kAttnCntOff));
-        s_pc[s_npc] = BalPiece{hk, rb, o, T * g, c1 - c0 + 1, (int)blockIdx.x - c0, slot0, 2 * (c0 + 1),
-                               (c / kCountGen + 1) * kCountGen};
-        s_npc = s_npc + 1;
-      }
-      x_next = seg0;
-      const int pg_first = k_begin / EE_PAGE;
-      const int npg = (k_end - k_begin + EE_PAGE - 1) / EE_PAGE;   // <= kMaxCtaPages: see the plan
-#pragma unroll
-      for (int k = 0; k < kPgPerThread; ++k) {
-        const int i = threadIdx.x + k * kThreads;
-        pgr[k] = i < npg ? ld_nc_pinned(p.block_table + (size_t)b * p.max_pages + pg_first + i) : -1;
-      }
+      if (s_sched[1] <= s_sched[0]) return false;
+      bal_segment<kKV>(p, wlist, s_sched[1], 0, lane, sg);
+      return true;
     } else {
-      b = blockIdx.z;
-      hk = blockIdx.y;
-      rb = blockIdx.x / p.S;                     // the S chunks of a row block are consecutive
-      // the row block's count, read now beside the node range (any time before
-      // this CTA's own arrival will do: it is a multiple of kCountGen plus the
-      // arrivals of this launch so far, never all of them)
-      if (p.coop && p.S > 1 && threadIdx.x == 0) {
-        const size_t cta0 = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + (size_t)rb * p.S;
-        u_target = ld_relaxed64(
-            reinterpret_cast<const unsigned long long*>(p.part + cta0 * kAttnPartBytes + kAttnCntOff));
-      }
-      // this chunk's page ids, issued now beside the sequence's node range and
-      // context length so that the round trips overlap (validated below)
-      const int pg_first = split * (p.chunk / EE_PAGE);
-      const int npg_cap = max(0, min(p.chunk / EE_PAGE, p.max_pages - pg_first));
-#pragma unroll
-      for (int k = 0; k < kPgPerThread; ++k) {
-        const int i = threadIdx.x + k * kThreads;
-        pgr[k] = i < npg_cap ? ld_nc_pinned(p.block_table + (size_t)b * p.max_pages + pg_first + i) : -1;
-      }
-      o = p.node_off[b];
-      T = p.node_off[b + 1] - o;
-      ctx = p.ctx_len[b];
-      const bool bad_tree = T < 1 || T > kMaxT || T > p.max_T || o < 0 || o + T > p.total_nodes;
-      if (bad_tree && threadIdx.x == 0 && blockIdx.x == 0 && hk == 0) flag_error(p.err, EE_DEVERR_TREE);
-      if (bad_tree || rb * kRows >= T * g) {     // uniform over the CTA (and the row block)
-        skip = true;
-        break;
-      }
-      if (ctx < 0 || ctx > p.max_ctx) {
-        if (threadIdx.x == 0 && blockIdx.x == 0 && hk == 0) flag_error(p.err, EE_DEVERR_CTX);
-        ctx = ctx < 0 ? 0 : p.max_ctx;
-      }
-      // everything above is uniform over the row block's CTAs; from here on every
-      // CTA reaches the merge synchronisation
-      // paged keys of the row block (chain: up to its last node's position)
-      const int span = kChain ? ctx + min(T, ((rb + 1) * kRows - 1) / g + 1) : (kIP ? ctx + T : ctx);
-      const int S = attn_splits_for(span, p.chunk);  // chunks this sequence uses, <= p.S
-      const bool active = split < S;
-      k_begin = split * p.chunk;
-      k_end = active ? min(span, k_begin + p.chunk) : k_begin;
-      with_tree = !kIP && active && split == S - 1;
-      alone = p.S == 1;
-      slot = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-      u_o = o;
-      u_R = T * g;
-
+      return uni_segment<kKV>(p, report, sg);
     }
-    const int R = T * g;
-    const int n_ctx_tiles = k_end > k_begin ? (k_end - k_begin + kKT - 1) / kKT : 0;
-    const int n_tiles = n_ctx_tiles + (with_tree ? 1 : 0);
+  };
+  auto next = [&]() -> bool {
+    if constexpr (kBal) {
+      tb += sg.n_tiles;
+      ++nseg;
+      if (sg.y <= s_sched[0]) return false;
+      bal_segment<kKV>(p, wlist, sg.y, tb, lane, sg);
+      return true;
+    } else {
+      return false;
+    }
+  };
+  // wait outcomes are made warp-uniform: what follows is warp-collective
+  auto wait = [&](uint32_t bar, int use) -> bool {
+    return __all_sync(0xffffffffu, mbar_wait(bar, (uint32_t)(use & 1), &s_abort));
+  };
 
-    // softmax threads issue the coalesced loads of the block's Q rows now (a
-    // half-warp reads one 256-byte row; rows past R read row R - 1 and are
-    // zeroed later) so that they leave before the K/V stream starts; the values
-    // are consumed after the barrier below
-    bool pages_ok = true;
-    uint4 qv[kRows / 16];
-    if (warp >= kWarpSoft0) {
-#pragma unroll
-      for (int k = 0; k < kRows / 16; ++k) {
-        const int rq = 2 * ((warp - kWarpSoft0) + 8 * k) + qhalf;   // 0..127
-        const int rrq = min(rb * kRows + rq, R - 1);
-        const int nq = rrq / g;
-        qv[k] = __ldg(reinterpret_cast<const uint4*>(
-                          p.q + ((size_t)(o + nq) * p.n_q + hk * g + (rrq - nq * g)) * kD) +
-                      qc);
+  if (warp == kWarpK || warp == kWarpV) {
+    // ---------------- TMA producers: warp 0 streams K, warp 2 streams V ----------------
+    // Ring slots and phases count the CTA's tiles over all its segments.  Lane l
+    // holds the page id of 16-row block l % 8 of the (l / 8)-th of four
+    // consecutive tiles, loaded four tiles ahead; one elected lane issues the
+    // tile's 16 boxes (eight blocks, two 64-dim halves) from warp-uniform rows.
+    // Boxes issued by different lanes are serialised one by one: 1100 cycles a
+    // tile (and the K stream behind the tensor pipe), against about 300.
+    const bool isK = warp == kWarpK;
+    const int nst = isK ? kKST : kVST;
+    const uint32_t full0 = isK ? k_full : v_full, empty0 = isK ? k_empty : v_empty;
+    const uint32_t ring = isK ? sK : sV;
+    const CUtensorMap* mc = isK ? &tmKc : &tmVc;
+    const CUtensorMap* mt = isK ? &tmKt : &tmVt;
+    int* issued = isK ? s_kissued : s_vissued;
+    int32_t early = -1;
+    unsigned long long u_count = 0;
+    if constexpr (!kBal) {
+      // the chunk's first page ids (and the row block's count), issued beside the
+      // node range and context length so that the round trips overlap
+      const int split = (int)(blockIdx.x % p.S);
+      const int pg = split * (p.chunk / EE_PAGE) + lane;
+      if (pg < p.max_pages) early = ld_nc_pinned(p.block_table + (size_t)blockIdx.z * p.max_pages + pg);
+      if (!isK && lane == 0 && p.coop && p.S > 1)
+        u_count = ld_relaxed64(reinterpret_cast<const unsigned long long*>(
+            p.part + (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x - split) * kAttnPartBytes +
+            kAttnCntOff));
+    }
+    bool more = first(isK && lane == 0);
+    if constexpr (!kBal) {
+      // the count any time before this CTA's own arrival is a multiple of
+      // kCountGen plus the arrivals of this launch so far, never all of them
+      if (!isK && lane == 0 && more) {
+        s_uni = make_int2(sg.o, sg.T * g);
+        s_pc[0].target = (u_count / kCountGen + 1) * kCountGen;
       }
     }
-    {
-      // pages that hold keys of this segment (k_end <= ctx <= max_pages * 16);
-      // the previous segment's readers are past the barrier that ended it
-      const int npg = (k_end - k_begin + EE_PAGE - 1) / EE_PAGE;
-#pragma unroll
-      for (int k = 0; k < kPgPerThread; ++k) {
-        const int i = threadIdx.x + k * kThreads;
-        if (i < npg) {
-          const int pg = pgr[k];
-          const bool ok = pg >= 0 && pg < p.num_pages;
-          if (!ok) flag_error(p.err, EE_DEVERR_PAGE);
-          s_pages[i] = ok ? pg : -1;
-          pages_ok &= ok;
+    bool go = true;
+    for (; more && go; more = next()) {
+      // page ids of tiles 4 c .. 4 c + 3 of the segment's order; INT_MIN: no keys there
+      auto fetch = [&](int c) -> int32_t {
+        const int t = 4 * c + (lane >> 3);
+        if (t >= sg.n_tiles) return INT32_MIN;
+        const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;
+        const int pos = sg.k_begin + i * kKT + 16 * (lane & 7);
+        if (i >= sg.n_ctx || pos >= sg.k_end) return INT32_MIN;
+        if (!kBal && c == 0) return max(early, -1);
+        return max(ld_nc_pinned(p.block_table + (size_t)sg.b * p.max_pages + pos / EE_PAGE), -1);
+      };
+      int32_t ids = fetch(0), ids_next = INT32_MIN;
+      for (int t = 0; t < sg.n_tiles; ++t) {
+        if ((t & 3) == 0) {
+          if (t > 0) ids = ids_next;
+          ids_next = fetch((t >> 2) + 1);
         }
-      }
-    }
-    tc_fence_before();
-    // every page of the segment valid: whole context tiles need no mask
-    const bool seg_pages_ok = __syncthreads_and(pages_ok) != 0;
-    tc_fence_after();
-    tmem = s_tmem;
-    // every thread has read the schedule position: advance it for the next segment
-    if (kBal && threadIdx.x == 0) {
-      s_sched[6] = x_next;
-      s_sched[4] = tb + n_tiles;
-      s_sched[5] = nseg + 1;
-    }
-
-    if (warp == kWarpK || warp == kWarpV) {
-      // ---------------- TMA producers: warp 0 streams K, warp 2 streams V ----------------
-      // lane 0 waits for the slot and posts the byte count; lane i < 8 then issues
-      // the two boxes of the tile's 16-row block i.  Ring slots and phases count
-      // the CTA's tiles over all its segments.
-      const bool isK = warp == kWarpK;
-      const int nst = isK ? kKST : kVST;
-      const uint32_t full0 = isK ? k_full : v_full, empty0 = isK ? k_empty : v_empty;
-      const uint32_t ring = isK ? sK : sV;
-      const CUtensorMap* mc = isK ? &tmKc : &tmVc;
-      const CUtensorMap* mt = isK ? &tmKt : &tmVt;
-      int* issued = isK ? s_kissued : s_vissued;
-      for (int t = 0; t < n_tiles; ++t) {
         const int tg = tb + t;
         const int st = tg % nst, use = tg / nst;
-        bool go = true;
-        if (lane == 0) go = mbar_wait(empty0 + 8 * st, (uint32_t)(use & 1) ^ 1u, &s_abort);
-        if (!__shfl_sync(0xffffffffu, go, 0)) break;
+        // the tile's eight blocks, the same in every lane: first cache row, -EE_PAGE
+        // without a page
+        int row[kKT / 16];
+        unsigned okm = 0u;      // bit i: block i has keys in a valid page
+        bool bad = false;
+#pragma unroll
+        for (int q = 0; q < kKT / 16; ++q) {
+          const int32_t id = __shfl_sync(0xffffffffu, ids, 8 * (t & 3) + q);
+          const bool ok = id >= 0 && id < p.num_pages;
+          row[q] = ok ? (id * p.n_kv + sg.hk) * EE_PAGE : -EE_PAGE;
+          okm |= ok ? 1u << q : 0u;
+          bad |= !ok && id != INT32_MIN;
+        }
+        if (isK && bad && lane == 0) flag_error(p.err, EE_DEVERR_PAGE);
+        go = wait(empty0 + 8 * st, use + 1);
+        if (!go) break;
         const uint32_t full = full0 + 8 * st;
         const uint32_t dst = ring + st * kKVBytes;
-        if (lane == 0) mbar_expect_tx(full, 2 * kKVHalf);
-        __syncwarp();
-        const int i = t + rot < n_tiles ? t + rot : t + rot - n_tiles;   // the segment's tile
-        if (i < n_ctx_tiles) {
-          // every 16-row block is written: blocks without a loaded page are read at
-          // row -16, wholly out of range, which the TMA unit fills with zeros (a
-          // stale V row would turn 0 * P into NaN)
-          if (lane < kKT / 16) {
-            const int pos = k_begin + i * kKT + 16 * lane;
-            const int pg = pos < k_end ? s_pages[i * (kKT / 16) + lane] : -1;
-            const int row0 = pg >= 0 ? (pg * p.n_kv + hk) * EE_PAGE : -EE_PAGE;
-            tma_load_2d(dst + lane * 2048, mc, full, 0, row0);
-            tma_load_2d(dst + kKVHalf + lane * 2048, mc, full, 64, row0);
+        const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;   // the segment's tile
+        if (elect_one()) {
+          if (isK) s_mask[tg % kMaskRing] = okm;
+          mbar_expect_tx(full, 2 * kKVHalf);
+          if (i < sg.n_ctx) {
+            // every 16-row block is written: blocks without a loaded page are read at
+            // row -16, wholly out of range, which the TMA unit fills with zeros (a
+            // stale V row would turn 0 * P into NaN)
+#pragma unroll
+            for (int q = 0; q < kKT / 16; ++q) {
+              tma_load_2d(dst + q * 2048, mc, full, 0, row[q]);
+              tma_load_2d(dst + kKVHalf + q * 2048, mc, full, 64, row[q]);
+            }
+          } else {
+            tma_load_3d(dst, mt, full, 0, sg.hk, sg.o);
+            tma_load_3d(dst + kKVHalf, mt, full, 64, sg.hk, sg.o);
           }
-        } else if (lane == 0) {
-          tma_load_3d(dst, mt, full, 0, hk, o);
-          tma_load_3d(dst + kKVHalf, mt, full, 64, hk, o);
         }
         __syncwarp();
         if (lane == 0) issued[st] = use;
+        if constexpr (kBal) {
+          // the piece of a split row block, and its count as read before this
+          // CTA's own arrival
+          if (!isK && t == min(1, sg.n_tiles - 1) && !sg.alone && lane == 0 && s_npc < 2) {
+            const unsigned long long c = ld_relaxed64(
+                reinterpret_cast<const unsigned long long*>(p.part + (size_t)sg.slot0 * kAttnPartBytes + kAttnCntOff));
+            s_pc[s_npc] = BalPiece{sg.hk, sg.rb, sg.o, sg.T * g, sg.c1 - sg.c0 + 1, (int)blockIdx.x - sg.c0,
+                                   sg.slot0, 2 * (sg.c0 + 1), (c / kCountGen + 1) * kCountGen};
+            s_npc = s_npc + 1;
+          }
+        }
       }
-    } else if (warp == kWarpMma) {
-      // ---------- MMA issuer: Q.K^T(0..kSB-1), then P.V(t), Q.K^T(t+kSB) ----------
-      // the whole warp walks the loop (wait outcomes made warp-uniform) and one
-      // elected lane issues, with every descriptor an offset from a uniform base
+    }
+  } else if (warp == kWarpQk) {
+    // ---------------- S = Q K^T, up to kSB tiles ahead of P.V ----------------
+    // One warp issues Q.K^T and another P.V: while one waits for its operands (a
+    // ready mbarrier still costs about 100 cycles to see), the other's MMAs keep
+    // the tensor pipe busy.  The whole warp walks the loop and one elected lane
+    // issues, every descriptor an offset from a uniform base.
+    const uint32_t id_qk = idesc_f16(kRows, kKT, 1, 1, 0);
+    const uint64_t dq = smem_desc_sw128(__shfl_sync(0xffffffffu, sQ, 0));
+    const uint64_t dk0 = smem_desc_sw128(__shfl_sync(0xffffffffu, sK, 0));
+    bool go = true;
+    for (bool more = first(false); more && go; more = next()) {
+      if (sg.n_tiles == 0) continue;
+      if (nseg == 0) {
+        go = wait(q_ready, 0);       // the softmax warps load the first row block
+      } else {
+        // the previous segment's last Q.K^T has read its rows; the load runs while
+        // its last kSB tiles are in the softmax
+        go = wait(q_empty, nseg - 1);
+        if (go) load_q<1>(p, sg, sQ, 0, lane);
+      }
       tc_fence_after();
-      const uint32_t id_qk = idesc_f16(kRows, kKT, 1, 1, 0);
-      const uint32_t id_pv = idesc_f16(kRows, kD, 1, 1, 1);
-      const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-      const uint64_t dq = smem_desc_sw128(__shfl_sync(0xffffffffu, sbase + kOffQ, 0));
-      const uint64_t dk0 = smem_desc_sw128(__shfl_sync(0xffffffffu, sK, 0));
-      const uint64_t dv0 = smem_desc_sw128_mn(__shfl_sync(0xffffffffu, sV, 0), kKVHalf, 1024);
-      auto wait = [&](uint32_t bar, int use) -> bool {
-        return __all_sync(0xffffffffu, mbar_wait(bar, (uint32_t)(use & 1), &s_abort));
-      };
-      auto issue_qk = [&](int t) -> bool {
+      for (int t = 0; t < sg.n_tiles && go; ++t) {
         const int tg = tb + t;
         const int st = tg % kKST, sb = tg % kSB;
-        if (!wait(k_full + 8 * st, tg / kKST)) return false;
+        if (tg >= kSB) go = wait(pv_done + 8 * sb, tg / kSB - 1);   // S buffer's P consumed
+        go = go && wait(k_full + 8 * st, tg / kKST);
+        if (!go) break;
         tc_fence_after();
         if (elect_one()) {
           const uint64_t dk = dk0 + (uint64_t)(st * (kKVBytes >> 4));
 #pragma unroll
           for (int kk = 0; kk < kD / 16; ++kk) {
             const uint64_t off = ((kk >> 2) * kKVHalf + (kk & 3) * 32) >> 4;
-            tc_mma(tm + sb * kKT, dq + off, dk + off, id_qk, kk > 0 ? 1u : 0u);
+            tc_mma(tmem + sb * kKT, dq + off, dk + off, id_qk, kk > 0 ? 1u : 0u);
           }
-          tc_commit(k_empty + 8 * st);
           tc_commit(s_full + 8 * sb);
+          tc_commit(k_empty + 8 * st);
+          if (t == sg.n_tiles - 1) tc_commit(q_empty);
+          mbar_arrive(s_full + 8 * sb);   // releases the tile's page mask (acquired with k_full)
         }
         __syncwarp();
-        return true;
-      };
-      bool ok = wait(q_ready, nseg);
-      for (int t = 0; t < kSB && t < n_tiles && ok; ++t) ok = issue_qk(t);
-      for (int t = 0; t < n_tiles && ok; ++t) {
+      }
+    }
+  } else if (warp == kWarpPv) {
+    // ---------------- O += P V ----------------
+    const uint32_t id_pv = idesc_f16(kRows, kD, 1, 1, 1);
+    const uint64_t dv0 = smem_desc_sw128_mn(__shfl_sync(0xffffffffu, sV, 0), kKVHalf, 1024);
+    bool go = true;
+    int filled = 0;    // segments with tiles so far
+    for (bool more = first(false); more && go; more = next()) {
+      if (sg.n_tiles == 0) continue;
+      // the softmax has read the previous segment's O
+      if (filled > 0) go = wait(o_free, filled - 1);
+      ++filled;
+      for (int t = 0; t < sg.n_tiles && go; ++t) {
         const int tg = tb + t;
         const int st = tg % kVST, sb = tg % kSB;
-        if (!wait(p_full + 8 * sb, tg / kSB) || !wait(v_full + 8 * st, tg / kVST)) break;
+        go = wait(v_full + 8 * st, tg / kVST) && wait(p_full + 8 * sb, tg / kSB);
+        if (!go) break;
         tc_fence_after();
         if (elect_one()) {
-          const uint32_t pa = tm + sb * kKT;       // bf16 P head: cols 0..63, tail: 64..127
+          const uint32_t pa = tmem + sb * kKT;       // bf16 P head: cols 0..63, tail: 64..127
           const uint64_t dv = dv0 + (uint64_t)(st * (kKVBytes >> 4));
 #pragma unroll
           for (int part = 0; part < 2; ++part)
 #pragma unroll
             for (int j = 0; j < kKT / 16; ++j)
-              tc_mma_ts(tm + kColO, pa + 64 * part + 8 * j, dv + (uint64_t)(j * (2048 >> 4)), id_pv,
+              tc_mma_ts(tmem + kColO, pa + 64 * part + 8 * j, dv + (uint64_t)(j * (2048 >> 4)), id_pv,
                         (t > 0 || part > 0 || j > 0) ? 1u : 0u);
+          tc_commit(pv_done + 8 * sb);
           tc_commit(v_empty + 8 * st);
-          tc_commit(o_done + 8 * (tg & 1));
         }
         __syncwarp();
-        if (t + kSB < n_tiles) ok = issue_qk(t + kSB);
       }
-      // one phase per segment: every product of the segment is complete
-      if (n_tiles > 0 && elect_one()) tc_commit(o_final);
-      __syncwarp();
-    } else if (warp >= kWarpSoft0) {
-      // ---------------- softmax: one query row and half of every tile per thread ----------------
-      // Warps w and w + 4 share TMEM lane quarter w & 3 (32 query rows); half hf
-      // of the pair takes keys [64 hf, 64 hf + 64) of every tile and O columns
-      // [64 hf, 64 hf + 64).  The pair agrees on each tile's row maximum through
-      // shared memory at a 64-thread named barrier, so both halves take the same
-      // rescale decisions; each keeps the sum over its own keys, and the two sums
-      // are added (half 0 first) at the end.  Two warps per sub-partition hide
-      // each other's latencies.  Every exit from the tile loop happens right
-      // after the pair barrier and on a decision both warps share.
-      const int qd = warp & 3;
-      const int hf = (warp - kWarpSoft0) >> 2;
-      const uint32_t pair_bar = 2 + qd;
-      const int r = qd * 32 + lane;                     // == TMEM lane of this quarter
-      const int rr = rb * kRows + r;
+    }
+  } else {
+    // ---------------- softmax: one query row and half of every tile per thread ----------------
+    // Warps w and w + 4 share TMEM lane quarter w & 3 (32 query rows); half hf
+    // of the pair takes keys [64 hf, 64 hf + 64) of every tile and O columns
+    // [64 hf, 64 hf + 64).  The pair agrees on each tile's row maximum through
+    // shared memory at a 64-thread named barrier, so both halves take the same
+    // rescale decisions; each keeps the sum over its own keys, and the two sums
+    // are added (half 0 first) at the end.  Two warps per sub-partition hide
+    // each other's latencies.  Every exit from the tile loop happens right
+    // after the pair barrier and on a decision both warps share.
+    const int qd = warp & 3;
+    const int hf = (warp - kWarpSoft0) >> 2;
+    const uint32_t pair_bar = 2 + qd;
+    const int r = qd * 32 + lane;                     // == TMEM lane of this quarter
+    const uint32_t tl = tmem + ((uint32_t)(qd * 32) << 16);
+    const float sl2 = p.scale_log2;
+    bool ok = true;
+    bool loaded = false;
+    for (bool more = first(false); more && ok; more = next()) {
+      const int R = sg.T * g;
+      const int rr = sg.rb * kRows + r;
       const bool vrow = rr < R;
-      const int node = vrow ? rr / g : 0;
+      const int node = vrow ? row_node(p, rr) : 0;
+      if (!loaded) {   // the first row block's Q: each softmax warp copies 16 rows
+        load_q<kSoftWarps>(p, sg, sQ, warp - kWarpSoft0, lane);
+        if (lane == 0) mbar_arrive(q_ready);
+        loaded = true;
+      }
       // this half's tree keys (separate tree tile), or the row's whole ancestor
       // mask (in place: tree keys at any offset from a half's first key)
-      const uint64_t ancw = (!kChain && vrow) ? p.anc[2 * (size_t)(o + node) + (kIP ? 0 : hf)] : 0ull;
-      const uint64_t anc_hi = (kKV == kKVInPlace && vrow) ? p.anc[2 * (size_t)(o + node) + 1] : 0ull;
-      const uint32_t tl = tmem + ((uint32_t)(qd * 32) << 16);
-      // the block's Q rows into shared memory as the A operand of Q.K^T: 128 rows
-      // x 128 bf16 in two 64-column slabs, 128-byte swizzled K-major (the layout
-      // TMA gives the K tiles): 16-byte chunk j of row r at slab (j / 8),
-      // (r / 8) * 1024 + (r % 8) * 128 + ((j % 8) ^ (r % 8)) * 16; rows past R are
-      // zero.  The rows were loaded (coalesced) before the set-up barrier; the
-      // previous segment's Q.K^T products completed before its last P.V did.
-      {
-        uint8_t* qs = smem + kOffQ;
-#pragma unroll
-        for (int k = 0; k < kRows / 16; ++k) {
-          const int rq = 2 * ((warp - kWarpSoft0) + 8 * k) + qhalf;
-          const int j = qc & 7;
-          *reinterpret_cast<uint4*>(qs + (qc >> 3) * kKVHalf + (rq >> 3) * 1024 + (rq & 7) * 128 +
-                                    ((j ^ (rq & 7)) << 4)) =
-              rb * kRows + rq < R ? qv[k] : make_uint4(0u, 0u, 0u, 0u);
-        }
-        fence_async_smem();   // generic-proxy writes, read by the tensor core
-        mbar_arrive(q_ready);
-      }
+      const uint64_t ancw = (!kChain && vrow) ? p.anc[2 * (size_t)(sg.o + node) + (kIP ? 0 : hf)] : 0ull;
+      const uint64_t anc_hi = (kKV == kKVInPlace && vrow) ? p.anc[2 * (size_t)(sg.o + node) + 1] : 0ull;
       // m_used is kept in raw score units (scale > 0, so the max commutes with it)
       float m_used = -INFINITY, l = 0.f;
-      const float sl2 = p.scale_log2;
-      const float kFail = __int_as_float(0x7fffffff);   // NaN: "this half's wait failed"
-      bool ok = true;
-      // the loop runs over the CTA's tile count tg (ring phases), with the
-      // segment's first tile at tg = tb; step tg processes the segment's tile
-      // tg + d (mod n_tiles)
-      const int tg_end = tb + n_tiles;
-      const int d = rot - tb;
-      for (int tg = tb; tg < tg_end; ++tg) {
+      // keys below full_end: every row sees all of them (when their pages are valid)
+      const int full_end = kIP ? min(sg.k_end, sg.ctx) : sg.k_end;
+      // step tg processes the segment's tile tg - tb + rot (mod n_tiles)
+      for (int t = 0; t < sg.n_tiles; ++t) {
+        const int tg = tb + t;
         const int sb = tg % kSB;    // S buffer of this tile
         const int xb = tg & 1;      // pair-exchange slot
-        // wait outcomes are warp-uniform: the TMEM accesses that follow are
-        // warp-collective (.sync.aligned)
-        const bool got =
-            __all_sync(0xffffffffu, mbar_wait(s_full + 8 * sb, (uint32_t)((tg / kSB) & 1), &s_abort));
+        const bool got = wait(s_full + 8 * sb, tg / kSB);
         uint32_t sr[64];
         float tmax = -INFINITY;
         if (got) {
           tc_fence_after();
-          tc_ld32(tl + sb * kKT + 64 * hf, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
-          tc_ld32(tl + sb * kKT + 64 * hf + 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
-          // visibility of this half's 64 keys as one 64-bit word
-          uint64_t kw;
-          const int i = tg + d < n_tiles ? tg + d : tg + d - n_tiles;
-          if (seg_pages_ok && k_begin + (i + 1) * kKT <= (kIP ? min(k_end, ctx) : k_end)) {
-            kw = ~0ull;   // a whole tile of context keys in valid pages: every row sees all of it
-          } else if (i < n_ctx_tiles) {
-            const unsigned m = tile_mask(s_pages, i, k_begin, k_end);
-            const int nv = min(max(k_end - (k_begin + i * kKT) - 64 * hf, 0), 64);
-            uint64_t pgw = 0ull;
+          tc_ld32_nowait(tl + sb * kKT + 64 * hf, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
+          tc_ld32_nowait(tl + sb * kKT + 64 * hf + 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
+          const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;
+          const unsigned pm = s_mask[tg % kMaskRing];     // bit j: 16-row block j has a valid page
+          const int p0 = sg.k_begin + i * kKT;            // the tile's first key
+          // a whole tile of context keys in valid pages needs no mask: every row
+          // sees all of it (rows past R hold zero queries and are never stored)
+          const bool whole = i < sg.n_ctx && pm == 0xFFu && p0 + kKT <= full_end;
+          tc_wait_ld32(*reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
+          tc_pin32(*reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
+          if (!whole) {
+            // visibility of this half's 64 keys as one 64-bit word
+            uint64_t kw;
+            const int h0 = p0 + 64 * hf;
+            if (i < sg.n_ctx) {
+              const int nv = min(max(sg.k_end - h0, 0), 64);
+              uint64_t pgw = 0ull;
 #pragma unroll
-            for (int pb = 0; pb < 4; ++pb) pgw |= ((m >> (4 * hf + pb)) & 1u) ? (0xFFFFull << (16 * pb)) : 0ull;
-            kw = pgw & (nv >= 64 ? ~0ull : ((1ull << nv) - 1ull));
-            if constexpr (kChain) {
-              // causal: node sees positions up to ctx + node
-              const int p0 = k_begin + i * kKT + 64 * hf;
-              const int nvis = min(max(ctx + node + 1 - p0, 0), 64);
-              kw &= nvis >= 64 ? ~0ull : ((1ull << nvis) - 1ull);
-            } else if constexpr (kIP) {
-              // keys below ctx are context; key p >= ctx is tree node p - ctx
-              const int p0 = k_begin + i * kKT + 64 * hf;
-              const int nc = min(max(ctx - p0, 0), 64);
-              const int sh = p0 - ctx;    // ancestor bit of this half's first key
-              uint64_t tm;
-              if (sh >= 0)
-                tm = sh >= 128 ? 0ull
-                     : sh >= 64 ? (anc_hi >> (sh - 64))
-                     : sh == 0  ? ancw
-                                : ((ancw >> sh) | (anc_hi << (64 - sh)));
-              else
-                tm = sh <= -64 ? 0ull : (ancw << (-sh));
-              kw &= (nc >= 64 ? ~0ull : ((1ull << nc) - 1ull)) | tm;
+              for (int pb = 0; pb < 4; ++pb)
+                pgw |= ((pm >> (4 * hf + pb)) & 1u) ? (0xFFFFull << (16 * pb)) : 0ull;
+              kw = pgw & (nv >= 64 ? ~0ull : ((1ull << nv) - 1ull));
+              if constexpr (kChain) {
+                // causal: node sees positions up to ctx + node
+                const int nvis = min(max(sg.ctx + node + 1 - h0, 0), 64);
+                kw &= nvis >= 64 ? ~0ull : ((1ull << nvis) - 1ull);
+              } else if constexpr (kIP) {
+                // keys below ctx are context; key p >= ctx is tree node p - ctx
+                const int nc = min(max(sg.ctx - h0, 0), 64);
+                const int sh = h0 - sg.ctx;    // ancestor bit of this half's first key
+                uint64_t tm;
+                if (sh >= 0)
+                  tm = sh >= 128 ? 0ull
+                       : sh >= 64 ? (anc_hi >> (sh - 64))
+                       : sh == 0  ? ancw
+                                  : ((ancw >> sh) | (anc_hi << (64 - sh)));
+                else
+                  tm = sh <= -64 ? 0ull : (ancw << (-sh));
+                kw &= (nc >= 64 ? ~0ull : ((1ull << nc) - 1ull)) | tm;
+              }
+            } else {
+              const int th = min(max(sg.T - 64 * hf, 0), 64);
+              kw = ancw & (th >= 64 ? ~0ull : ((1ull << th) - 1ull));
             }
-          } else {
-            const int th = min(max(T - 64 * hf, 0), 64);
-            kw = ancw & (th >= 64 ? ~0ull : ((1ull << th) - 1ull));
-          }
-          if (!vrow) kw = 0ull;
-          if (!__all_sync(0xffffffffu, kw == ~0ull)) {
+            if (!vrow) kw = 0ull;
 #pragma unroll
             for (int c = 0; c < 64; ++c)
               if (!((kw >> c) & 1ull)) sr[c] = __float_as_uint(-INFINITY);
@@ -882,27 +941,25 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
           tmax = fmax3(fmax3(mx[0], mx[1], mx[2]), fmax3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7]));
         }
         // the pair swaps its halves' maxima; both S halves are in registers before
-        // either warp overwrites S with P
-        s_xmax[xb][hf][r] = got ? tmax : kFail;
+        // either warp overwrites S with P.  kFail (a NaN no maximum yields: theirs is
+        // 0x7fffffff) says that this half's wait failed
+        constexpr uint32_t kFail = 0xffffffffu;
+        s_xmax[xb][hf][r] = got ? __float_as_uint(tmax) : kFail;
         tc_fence_before();
         asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
         tc_fence_after();
-        const float other = s_xmax[xb][hf ^ 1][r];
-        if (!__all_sync(0xffffffffu, got && other == other)) {
+        const uint32_t other = s_xmax[xb][hf ^ 1][r];
+        if (!__all_sync(0xffffffffu, got && other != kFail)) {
           ok = false;
           break;
         }
-        tmax = fmaxf(tmax, other);
+        tmax = fmaxf(tmax, __uint_as_float(other));
         const float m_new = fmaxf(m_used, tmax);
         const bool need = (m_new - m_used) * sl2 > kRescaleLog2;   // true when m_used = -inf < m_new
-        if (tg > 0 && __any_sync(0xffffffffu, need)) {
+        if (t > 0 && __any_sync(0xffffffffu, need)) {
           // O must hold P.V(tg-1) before this half's columns are rescaled; a failed
-          // wait sets the abort flag, and the pair stops at the next barrier.  At a
-          // segment's first tile that product belongs to the previous segment (its
-          // completion was already waited for) and the rescale is harmless: the
-          // segment's first P.V overwrites O.
-          if (__all_sync(0xffffffffu,
-                         mbar_wait(o_done + 8 * ((tg - 1) & 1), (uint32_t)(((tg - 1) >> 1) & 1), &s_abort))) {
+          // wait sets the abort flag, and the pair stops at the next barrier
+          if (wait(pv_done + 8 * ((tg - 1) % kSB), (tg - 1) / kSB)) {
             tc_fence_after();
             const float f = need ? ex2((m_used - m_new) * sl2) : 1.f;
 #pragma unroll 1
@@ -957,6 +1014,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
           tc_st16_nowait(tl + sb * kKT + 64 + 32 * hf + 16 * hh, tw);
         }
         tc_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(p_full + 8 * sb);
         {
           uint32_t a0, a1, b0, b1, c0, c1, d0, d1;
           f2_unpack(ls2[0], a0, a1);
@@ -966,44 +1026,47 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
           l += ((__uint_as_float(a0) + __uint_as_float(a1)) + (__uint_as_float(b0) + __uint_as_float(b1))) +
                ((__uint_as_float(c0) + __uint_as_float(c1)) + (__uint_as_float(d0) + __uint_as_float(d1)));
         }
-        tc_fence_before();
-        mbar_arrive(p_full + 8 * sb);
       }
-      // wait for the last P.V; the pair adds its two sums, then each half writes
-      // its 64 columns out: O / l itself when the segment is a whole row block,
-      // else the partial (O, m, l) to the segment's slot.  The wait is on a
-      // barrier of its own: here the tensor pipe may still owe P.V(n-3) and
-      // P.V(n-1), two phases of the same o_done barrier, which a parity wait
-      // cannot tell apart (inside the loop at most one phase is pending, since
-      // S(t) completes after P.V(t-3))
-      const bool fin = ok && n_tiles > 0 && mbar_wait(o_final, (uint32_t)(nseg & 1), &s_abort);
-      const bool have = __all_sync(0xffffffffu, fin);
-      s_xl[hf][r] = have ? l : kFail;
+      // wait for the last P.V (products complete in order, and this barrier's
+      // previous phase, P.V three tiles before, was over before the last S
+      // existed); the pair adds its two sums, then each half writes its 64
+      // columns out: O / l itself when the segment is a whole row block, else the
+      // partial (O, m, l) to the segment's slot
+      const int tl_g = tb + sg.n_tiles - 1;
+      const bool have = ok && sg.n_tiles > 0 && wait(pv_done + 8 * (tl_g % kSB), tl_g / kSB);
+      s_xl[hf][r] = l;
+      if (lane == 0) s_xok[nseg & 1][qd][hf] = have;
       asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-      const float l_sum = s_xl[0][r] + s_xl[1][r];     // NaN when either half failed
-      const bool both = have && l_sum == l_sum;
-      const float row_m = (both && vrow && m_used != -INFINITY) ? m_used * sl2 : -INFINITY;
-      const float row_l = (both && vrow && m_used != -INFINITY) ? l_sum : 0.f;
+      const float l_sum = s_xl[0][r] + s_xl[1][r];
+      const bool both = s_xok[nseg & 1][qd][0] && s_xok[nseg & 1][qd][1];
+      const bool nan_row = both && vrow && l_sum != l_sum;   // NaN scores: the output is NaN
+      const float row_m =
+          nan_row ? 0.f : ((both && vrow && m_used != -INFINITY) ? m_used * sl2 : -INFINITY);
+      const float row_l = (both && vrow && (m_used != -INFINITY || nan_row)) ? l_sum : 0.f;
       float4* dst;
       size_t dstride;                                   // float4 between column chunks
       float inv = 1.f;
-      if (alone) {
-        const size_t orow = (size_t)(o + node) * p.n_q + hk * g + (rr - node * g);
+      if (sg.alone) {
+        const size_t orow = (size_t)(sg.o + node) * p.n_q + sg.hk * g + (rr - node * g);
         dst = reinterpret_cast<float4*>(p.out + orow * kD);
         dstride = 1;
-        inv = row_l > 0.f ? 1.f / row_l : 0.f;
+        inv = row_l == 0.f ? 0.f : 1.f / row_l;
       } else {
-        dst = reinterpret_cast<float4*>(p.part + slot * kAttnPartBytes) + r;
+        dst = reinterpret_cast<float4*>(p.part + (size_t)sg.slot * kAttnPartBytes) + r;
         dstride = kRows;
       }
-      const bool store = alone ? vrow : row_l > 0.f;
-      // the TMEM read is warp-collective: the whole warp reads when any lane stores
-      if (__any_sync(0xffffffffu, store)) {
+      const bool store = sg.alone ? vrow : (row_l > 0.f || nan_row);
+      if (sg.n_tiles > 0) {
         tc_fence_after();
 #pragma unroll 1
         for (int c4 = 0; c4 < 2; ++c4) {
           uint32_t ov[32];
           tc_ld32(tl + kColO + 64 * hf + 32 * c4, ov);
+          if (c4 == 1) {   // O is in registers: the next segment's P.V may overwrite it
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(o_free);
+          }
           if (store) {
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -1015,20 +1078,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
           }
         }
       }
-      if (!alone) {
+      if (!sg.alone) {
         if (hf == 0)
-          __stcg(reinterpret_cast<float2*>(p.part + slot * kAttnPartBytes + kAttnMlOff) + r,
+          __stcg(reinterpret_cast<float2*>(p.part + (size_t)sg.slot * kAttnPartBytes + kAttnMlOff) + r,
                  make_float2(row_m, row_l));
       }
+      if (!both) ok = false;
     }
-    if constexpr (!kBal) break;
-    // end of the segment: every role is done with its pages, Q, S buffers and O
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (s_abort) break;
   }
-
   // ---- CTA teardown: drain on abort, free TMEM --------------------------------
   tc_fence_before();
   __syncthreads();
@@ -1042,12 +1099,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
     for (int st = 0; st < kVST; ++st)
       if (s_vissued[st] >= 0) mbar_wait_plain(v_full + 8 * st, (uint32_t)(s_vissued[st] & 1));
   }
-  if (warp == kWarpMma) {
-    if (aborted && elect_one()) {   // the lane that issued the MMAs
-      tc_commit(drain);
-      mbar_wait_plain(drain, 0);
+  if (aborted) {
+    // MMAs still in flight: each issuing warp's elected lane commits and waits
+    if ((warp == kWarpPv || warp == kWarpQk) && elect_one()) {
+      const uint32_t dr = drain + (warp == kWarpQk ? 8 : 0);
+      tc_commit(dr);
+      mbar_wait_plain(dr, 0);
     }
-    __syncwarp();
+    __syncthreads();
+  }
+  if (warp == kWarpPv) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(kTmemCols)
                  : "memory");
@@ -1099,12 +1160,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
     }
     return;
   } else {
-    if (skip || p.S == 1) return;
+    if (s_uni.y == 0 || p.S == 1) return;   // (y == 0: the row block has no work)
+    const int split = (int)(blockIdx.x % p.S);   // == cluster rank in the cluster mode
 
     // ---- merge (uniform modes) -------------------------------------------------------
     // once every slot of the row block is complete and visible, chunk `split`
     // merges rows [r0, r0 + nown) of the row block
-    const int R = u_R, o = u_o;
+    const int R = s_uni.y, o = s_uni.x;
     const int rb = blockIdx.x / p.S;
     const size_t cta0 = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + (size_t)rb * p.S;
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(p.part + cta0 * kAttnPartBytes + kAttnCntOff);
@@ -1112,7 +1174,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
       if (threadIdx.x == 0) {
         // this CTA's partial (every thread's stores precede the teardown barrier)
         red_add_release64(cnt, kCountGen / (unsigned)p.S);
-        const bool ready = wait_count64_geq(cnt, (u_target / kCountGen + 1) * kCountGen);
+        const bool ready = wait_count64_geq(cnt, s_pc[0].target);
         if (!ready) flag_error(p.err, EE_DEVERR_TIMEOUT);
         s_ready[0] = ready;
       }
@@ -1406,6 +1468,7 @@ ee_status verify_attn(const ee_bf16* q, const ee_bf16* k_tree, const ee_bf16* v_
   p.S = S;
   p.coop = (S > 1 && sp.coop) || sp.bal ? 1 : 0;
   p.B = B;
+  p.g_inv = g > 1 ? (uint32_t)(((1ull << 32) + g - 1) / g) : 0u;
   p.scale_log2 = scale * 1.4426950408889634f;
 
   cudaLaunchConfig_t cfg = {};
