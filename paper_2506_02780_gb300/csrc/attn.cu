@@ -96,7 +96,7 @@ constexpr uint32_t kOffK = 0;
 constexpr uint32_t kOffV = kOffK + kKST * kKVBytes;
 constexpr uint32_t kOffQ = kOffV + kVST * kKVBytes;  // Q block, 128 rows x 128 bf16, SW128 K-major
 constexpr uint32_t kOffBar = kOffQ + kKVBytes;
-constexpr uint32_t kNumBars = 2 * kKST + 2 * kVST + 3 * kSB + 5;
+constexpr uint32_t kNumBars = 2 * kKST + 2 * kVST + 3 * kSB + 6;
 constexpr uint32_t kSmemBytes = 1024 + kOffBar + 8 * kNumBars + 64;
 constexpr uint32_t kTmemCols = 512;              // S0 [0,128) S1 [128,256) S2 [256,384) O [384,512)
 constexpr uint32_t kColO = 384;
@@ -265,12 +265,12 @@ struct Seg {
   bool alone;                  // the segment is its whole row block
   int slot;                    // partial slot (alone: unused)
   int y;                       // balanced: where the segment starts in the work list
-  int c0, c1, slot0;           // balanced: CTAs holding the unit's first and last tiles, piece 0's slot
+  int U0, tiles;               // balanced: the unit's first tile in the work list and its tiles
 };
 
 // Shared state of a CTA's work: balanced mode, per sequence (node offset, T,
 // context length, tiles), the exclusive prefix of the sequences' work in
-// tiles, and (range start, range end, W, N).
+// tiles, and (range start, range end, W, N, the share ceil(W / N)).
 struct WorkList {
   const int4* seq;
   const int* wpre;
@@ -290,7 +290,7 @@ __device__ __forceinline__ void bal_segment(const AttnParams& p, const WorkList&
   // the share): the CTAs holding other row blocks of the same KV head then
   // read the same K/V tiles at about the same time, and L2 serves the
   // repeats (each KV head's tiles are read by all its row blocks).
-  const int x_begin = w.sched[0], W = w.sched[2], N = w.sched[3];
+  const int x_begin = w.sched[0], x_end = w.sched[1], P = w.sched[4];
   int lo = 0, hi = p.B;   // wpre[lo] <= y - 1 < wpre[hi]
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -304,11 +304,11 @@ __device__ __forceinline__ void bal_segment(const AttnParams& p, const WorkList&
   int tiles = sq.w;
   int U0;                                        // the unit's first tile in the work list
   const int base_w = w.wpre[lo];
-  const int nrb_b = (s.T * g + kRows - 1) / kRows;
+  const int nrb_b = (int)((unsigned)(s.T * g + kRows - 1) / kRows);
   if constexpr (kChain) {
     // sq.w = tiles of one KV head's row blocks; row block r has chain_rb_tiles
     const int local = y - 1 - base_w;
-    s.hk = local / tiles;
+    s.hk = (int)((unsigned)local / (unsigned)tiles);
     const int rem = local - s.hk * tiles;
     // the row block holding tile rem: a scan of the row blocks' tile counts, 32 at a time
     int r = nrb_b - 1, cum = 0, tu = 0;
@@ -341,8 +341,8 @@ __device__ __forceinline__ void bal_segment(const AttnParams& p, const WorkList&
     U0 = base_w + s.hk * tiles + cum;
     tiles = tu;
   } else {
-    const int u = (y - 1 - base_w) / tiles;
-    s.hk = u / nrb_b;
+    const int u = (int)((unsigned)(y - 1 - base_w) / (unsigned)tiles);
+    s.hk = (int)((unsigned)u / (unsigned)nrb_b);
     s.rb = u - s.hk * nrb_b;
     U0 = base_w + u * tiles;
   }
@@ -356,15 +356,12 @@ __device__ __forceinline__ void bal_segment(const AttnParams& p, const WorkList&
   s.k_end = t0 < n_ctx_b ? min(unit_span, min(t0 + len, n_ctx_b) * kKT) : s.k_begin;
   s.n_ctx = s.k_end > s.k_begin ? (s.k_end - s.k_begin + kKT - 1) / kKT : 0;
   s.n_tiles = s.n_ctx + (!kIP && t0 + len == tiles ? 1 : 0);
-  const int P = (W + N - 1) / N;
   int ph = (tb - t0) % P;
   ph += ph < 0 ? P : 0;
   s.rot = ph < len ? ph : 0;
-  // the CTAs holding the unit's first and last tiles
-  s.c0 = ((U0 + 1) * N - 1) / W;
-  s.c1 = ((U0 + tiles) * N - 1) / W;
-  s.alone = s.c0 == s.c1;
-  s.slot0 = 2 * s.c0 + (U0 > s.c0 * W / N ? 1 : 0);
+  s.alone = U0 >= x_begin && U0 + tiles <= x_end;
+  s.U0 = U0;
+  s.tiles = tiles;
   // a piece starts the CTA's range (slot 2c) or ends it (slot 2c + 1)
   s.slot = 2 * (int)blockIdx.x + (seg0 > x_begin ? 1 : 0);
   s.y = seg0;
@@ -409,25 +406,41 @@ __device__ __forceinline__ bool uni_segment(const AttnParams& p, bool report, Se
   return true;
 }
 
-// Row block rows [2 * first, ...) of Q into shared memory as the A operand of
-// Q.K^T, by warps first, first + n, ... of n (a half-warp copies one 256-byte
-// row): 128 rows x 128 bf16 in two 64-column slabs, 128-byte swizzled K-major
+// Query rows of the segment's row block into shared memory as the A operand of
+// Q.K^T: 128 rows x 128 bf16 in two 64-column slabs, 128-byte swizzled K-major
 // (the layout TMA gives the K tiles): 16-byte chunk j of row r at slab (j / 8),
 // (r / 8) * 1024 + (r % 8) * 128 + ((j % 8) ^ (r % 8)) * 16; rows past R are
-// zero.  Asynchronous copies: every row is in flight before the first wait.
-template <int kN>
-__device__ __forceinline__ void load_q(const AttnParams& p, const Seg& s, uint32_t sQ, int first, int lane) {
-  const int R = s.T * p.g;
+// zero.  Rows r0, r0 + kStep, ... (kCount of them; a half-warp copies one
+// 256-byte row, so kStep counts rows from one copy of a lane to its next), as
+// asynchronous copies, all in flight before the wait.  The (node, head) of a row
+// advances by additions: one warp's instruction chain sets the time of the load.
+template <int kStep, int kCount>
+__device__ __forceinline__ void load_q(const AttnParams& p, const Seg& s, uint32_t sQ, int r0, int lane) {
+  const int g = p.g;
   const int j = lane & 15;
-  const __nv_bfloat16* base = p.q + ((size_t)s.o * p.n_q + s.hk * p.g) * kD + 8 * j;
-#pragma unroll 8
-  for (int k = 0; k < kRows / 2 / kN; ++k) {
-    const int rq = 2 * (first + kN * k) + (lane >> 4);   // 0..127
-    const int rr = s.rb * kRows + rq;
-    const int rc = min(rr, R - 1);
-    const int nd = row_node(p, rc);
-    cp_async16(sQ + (j >> 3) * kKVHalf + (rq >> 3) * 1024 + (rq & 7) * 128 + (((j & 7) ^ (rq & 7)) << 4),
-               base + ((size_t)nd * p.n_q + (rc - nd * p.g)) * kD, rr < R ? 16u : 0u);
+  int rq = r0 + (lane >> 4);                     // 0..127
+  const int left = s.T * g - s.rb * kRows;       // rows of the block that exist
+  const int rr = s.rb * kRows + rq;
+  const int nd = row_node(p, rr);
+  int h = rr - nd * g;
+  const char* base =
+      reinterpret_cast<const char*>(p.q + ((size_t)s.o * p.n_q + s.hk * g) * kD + 8 * j);
+  uint32_t off = ((uint32_t)nd * p.n_q + h) * (kD * 2);   // bytes; below 2048 * n_q * 256
+  const int dn = kStep / g, dh = kStep - dn * g;          // kStep rows = dn nodes and dh heads
+  const uint32_t step = ((uint32_t)dn * p.n_q + dh) * (kD * 2), wrap = (uint32_t)(p.n_q - g) * (kD * 2);
+  const uint32_t dst = sQ + (j >> 3) * kKVHalf;
+#pragma unroll
+  for (int k = 0; k < kCount; ++k) {
+    const bool in = rq < left;
+    cp_async16(dst + (rq >> 3) * 1024 + (rq & 7) * 128 + (((j & 7) ^ (rq & 7)) << 4), base + (in ? off : 0u),
+               in ? 16u : 0u);
+    rq += kStep;
+    off += step;
+    h += dh;
+    if (h >= g) {
+      h -= g;
+      off += wrap;
+    }
   }
   cp_async_wait_all();
   fence_async_smem();   // generic-proxy writes, read by the tensor core
@@ -455,7 +468,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   __shared__ uint32_t s_mask[kMaskRing];            // per tile: 16-row blocks with keys in a valid page
   __shared__ int4 s_seq[kBal ? kMaxBalSeqs : 1];
   __shared__ int s_wpre[kBal ? kMaxBalSeqs + 1 : 1];
-  __shared__ int s_sched[4];                        // balanced: range start, range end, W, N
+  __shared__ int s_sched[5];                        // balanced: range start, range end, W, N, ceil(W / N)
   __shared__ BalPiece s_pc[2];                      // this CTA's pieces of split row blocks
   __shared__ int s_npc;
   __shared__ int2 s_uni;                            // uniform: the row block's node offset and rows
@@ -468,6 +481,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   const uint32_t v_full = k_empty + 8 * kKST, v_empty = v_full + 8 * kVST;
   const uint32_t s_full = v_empty + 8 * kVST, p_full = s_full + 8 * kSB, pv_done = p_full + 8 * kSB;
   const uint32_t drain = pv_done + 8 * kSB, q_ready = drain + 16, q_empty = q_ready + 8, o_free = q_empty + 8;
+  const uint32_t q_half = o_free + 8;
 
   // on-chip set-up first: it touches no global memory, so it overlaps the end
   // of the previous kernel in the stream
@@ -499,6 +513,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
     mbar_init(q_ready, kSoftWarps);
     mbar_init(q_empty, 1);
     mbar_init(o_free, kSoftWarps);
+    mbar_init(q_half, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
@@ -525,16 +540,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   // start the next (at most two of its segments are pieces of split units).
   // N is capped so that every CTA gets at least m = max(2, ceil(t_max / 14))
   // tiles, which bounds the pieces of any unit by 15.
-  // Warp kWarpQk builds it: lane l takes sequences [16 l, 16 l + 16).
+  // Warp kWarpQk builds it: lane l takes sequences [per l, per l + per), per = ceil(B / 32).
   if constexpr (kBal) {
     if (warp == kWarpQk) {
-      constexpr int kPer = kMaxBalSeqs / 32;
-      int wl[kPer];
+      const int per = (p.B + 31) >> 5;     // sequences of a lane
       int wsum = 0, tmax = 0;
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {   // loads first (clamped indices), all in flight
-        const int bb = min(lane * kPer + k, p.B - 1);
-        s_seq[lane * kPer + k] = make_int4(p.node_off[bb], p.node_off[bb + 1], p.ctx_len[bb], 0);
+      for (int k = 0; k < per; ++k) {      // (clamped indices)
+        const int bb = min(lane * per + k, p.B - 1);
+        s_seq[lane * per + k] = make_int4(p.node_off[bb], p.node_off[bb + 1], p.ctx_len[bb], 0);
       }
       __syncwarp();
       // chain drafts: one KV head's tiles are a sum over its row blocks; for a
@@ -556,11 +569,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
         }
         __syncwarp();
       }
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {
-        const int bb = lane * kPer + k;
-        wl[k] = 0;
+      for (int k = 0; k < per; ++k) {
+        const int bb = lane * per + k;
         if (bb < p.B) {
+          int wl = 0;
           const int4 sq = s_seq[bb];
           const int Tb = sq.y - sq.x;
           const bool bad = Tb < 1 || Tb > kMaxT || Tb > p.max_T || sq.x < 0 || sq.x + Tb > p.total_nodes;
@@ -583,12 +595,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
             unit_max = bad ? 1 : chain_rb_tiles(c, Tb, g, nrb_b - 1);
           }
           if (!bad) {
-            wl[k] = p.n_kv * (kChain ? 1 : nrb_b) * tiles;
+            wl = p.n_kv * (kChain ? 1 : nrb_b) * tiles;
             tmax = max(tmax, unit_max);
           }
           s_seq[bb] = make_int4(sq.x, bad ? 0 : Tb, c, tiles);
+          s_wpre[bb] = wsum;               // within the lane
+          wsum += wl;
         }
-        wsum += wl[k];
       }
       // warp-wide exclusive scan of the lanes' sums (lane order is sequence order)
       int incl = wsum;
@@ -599,12 +612,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
       }
       const int W = __shfl_sync(0xffffffffu, incl, 31);
       const int tmax_all = __reduce_max_sync(0xffffffffu, tmax);
-      int run = incl - wsum;
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {
-        const int bb = lane * kPer + k;
-        if (bb < p.B) s_wpre[bb] = run;
-        run += wl[k];
+      for (int k = 0; k < per; ++k) {
+        const int bb = lane * per + k;
+        if (bb < p.B) s_wpre[bb] += incl - wsum;
       }
       if (lane == 0) {
         const int m = max(2, (tmax_all + 13) / 14);
@@ -614,6 +624,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
         s_sched[1] = mine ? ((int)blockIdx.x + 1) * W / N : 0;
         s_sched[2] = W;
         s_sched[3] = N;
+        s_sched[4] = N > 0 ? (W + N - 1) / N : 1;
         s_wpre[p.B] = W;
       }
     }
@@ -746,13 +757,25 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
         __syncwarp();
         if (lane == 0) issued[st] = use;
         if constexpr (kBal) {
+          // a later segment's Q rows 64 .. 127, once its first tiles are in the ring
+          // (the next slot frees only after this segment's first Q.K^T)
+          if (isK && nseg > 0 && t == min(kKST - 1, sg.n_tiles - 1)) {
+            go = wait(q_empty, nseg - 1);
+            if (!go) break;
+            load_q<2, kRows / 4>(p, sg, sQ, kRows / 2, lane);
+            if (lane == 0) mbar_arrive(q_half);
+          }
           // the piece of a split row block, and its count as read before this
           // CTA's own arrival
           if (!isK && t == min(1, sg.n_tiles - 1) && !sg.alone && lane == 0 && s_npc < 2) {
+            // the CTAs holding the unit's first and last tiles, piece 0's slot
+            const int W = s_sched[2], N = s_sched[3];
+            const int c0 = ((sg.U0 + 1) * N - 1) / W, c1 = ((sg.U0 + sg.tiles) * N - 1) / W;
+            const int slot0 = 2 * c0 + (sg.U0 > c0 * W / N ? 1 : 0);
             const unsigned long long c = ld_relaxed64(
-                reinterpret_cast<const unsigned long long*>(p.part + (size_t)sg.slot0 * kAttnPartBytes + kAttnCntOff));
-            s_pc[s_npc] = BalPiece{sg.hk, sg.rb, sg.o, sg.T * g, sg.c1 - sg.c0 + 1, (int)blockIdx.x - sg.c0,
-                                   sg.slot0, 2 * (sg.c0 + 1), (c / kCountGen + 1) * kCountGen};
+                reinterpret_cast<const unsigned long long*>(p.part + (size_t)slot0 * kAttnPartBytes + kAttnCntOff));
+            s_pc[s_npc] = BalPiece{sg.hk, sg.rb, sg.o, sg.T * g, c1 - c0 + 1, (int)blockIdx.x - c0,
+                                   slot0, 2 * (c0 + 1), (c / kCountGen + 1) * kCountGen};
             s_npc = s_npc + 1;
           }
         }
@@ -776,7 +799,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
         // the previous segment's last Q.K^T has read its rows; the load runs while
         // its last kSB tiles are in the softmax
         go = wait(q_empty, nseg - 1);
-        if (go) load_q<1>(p, sg, sQ, 0, lane);
+        if (go) load_q<2, kRows / 4>(p, sg, sQ, 0, lane);
+        go = go && wait(q_half, nseg - 1);   // the K warp loads the other half
       }
       tc_fence_after();
       for (int t = 0; t < sg.n_tiles && go; ++t) {
@@ -857,7 +881,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
       const bool vrow = rr < R;
       const int node = vrow ? row_node(p, rr) : 0;
       if (!loaded) {   // the first row block's Q: each softmax warp copies 16 rows
-        load_q<kSoftWarps>(p, sg, sQ, warp - kWarpSoft0, lane);
+        load_q<2 * kSoftWarps, kRows / 2 / kSoftWarps>(p, sg, sQ, 2 * (warp - kWarpSoft0), lane);
         if (lane == 0) mbar_arrive(q_ready);
         loaded = true;
       }
