@@ -849,7 +849,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
           for (int part = 0; part < 2; ++part)
 #pragma unroll
             for (int j = 0; j < kKT / 16; ++j)
-              tc_mma_ts(tmem + kColO, pa + 64 * part + 8 * j, dv + (uint64_t)(j * (2048 >> 4)), id_pv,
+              tc_mma_ts(tmem + kColO, pa + 64 * part + 8 * j, dv + (uint64_t)(j * (2048 >> 4)), part ? (id_pv | kIdescNegA) : id_pv,
                         (t > 0 || part > 0 || j > 0) ? 1u : 0u);
           tc_commit(pv_done + 8 * sb);
           tc_commit(v_empty + 8 * st);
@@ -1029,10 +1029,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
             // head = p rounded to bf16; tail = the remainder p - head (exact
             // in fp32) rounded to bf16
             const uint32_t hb = bf16x2_rn(__uint_as_float(p1), __uint_as_float(p0));
-            uint32_t t0, t1;
-            f2_unpack(f2_sub(pp, f2_pack(hb << 16, hb & 0xFFFF0000u)), t0, t1);
+            float t0, t1;
+            sub_bf16x2(hb, __uint_as_float(p0), __uint_as_float(p1), t0, t1);
             hw[e2] = hb;
-            tw[e2] = bf16x2_rn(__uint_as_float(t1), __uint_as_float(t0));
+            tw[e2] = bf16x2_rn(t1, t0);
           }
           tc_st16_nowait(tl + sb * kKT + 32 * hf + 16 * hh, hw);
           tc_st16_nowait(tl + sb * kKT + 64 + 32 * hf + 16 * hh, tw);

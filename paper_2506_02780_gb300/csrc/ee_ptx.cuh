@@ -292,6 +292,13 @@ __device__ __forceinline__ bool wait_count64_geq(const unsigned long long* c, un
 __device__ __forceinline__ void prefetch_l2_bulk(const void* a, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(bytes) : "memory");
 }
+// bf16 pair minus fp32 values (mixed-precision subtraction, sm_100 family): d0 =
+// lo half of h - a, d1 = hi half of h - b, in fp32.
+__device__ __forceinline__ void sub_bf16x2(uint32_t h, float a, float b, float& d0, float& d1) {
+  asm("{\n .reg .b16 l, u;\n mov.b32 {l, u}, %2;\n sub.rn.f32.bf16 %0, l, %3;\n sub.rn.f32.bf16 %1, u, %4;\n}\n"
+      : "=f"(d0), "=f"(d1)
+      : "r"(h), "f"(a), "f"(b));
+}
 // Packed fp32 pairs (sm_100 family): two lanes of fp32 arithmetic per instruction.
 __device__ __forceinline__ uint64_t f2_pack(uint32_t lo, uint32_t hi) {
   uint64_t d;
@@ -383,6 +390,8 @@ __device__ __forceinline__ uint64_t smem_desc_sw128_mn(uint32_t addr, uint32_t l
   d |= (uint64_t)2 << 61;
   return d;
 }
+// A operand negated (instruction descriptor bit)
+constexpr uint32_t kIdescNegA = 1u << 13;
 // Instruction descriptor of kind::f16 with fp32 accumulation.  a_bf16/b_bf16:
 // 1 = bf16, 0 = fp16 operand; b_mn: B is MN-major.
 __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, int a_bf16, int b_bf16, int b_mn) {
