@@ -214,6 +214,26 @@ __device__ void accept_sequences(const AcceptArgs& a, const int32_t* am, const i
       a0[c] = in ? a.anc[2 * (size_t)(o + i)] : 0ull;
       a1[c] = in ? a.anc[2 * (size_t)(o + i) + 1] : 0ull;
     }
+    // then what the rule needs of each node's parent: argmax, ranked ids, top_tau
+    // (again one round trip; verification reads them through L2)
+    int am_[4], tau_[4], tk_[4][kVerify ? ee::kLmMaxK : 1];
+    bool gen_[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int i = c * 32 + lane;
+      const int par = par_[c];
+      const bool use = i < T && i > 0 && par >= 0 && par < i;
+      am_[c] = use ? ld_i(am + o + par) : 0;
+      gen_[c] = false;
+      if constexpr (kVerify) {
+        gen_[c] = use && (!a.gen_mask || a.gen_mask[o + i]);
+        tau_[c] = use && a.mode == EE_VERIFY_ENTROPY ? ld_i(tau + o + par)
+                                                    : (a.mode == EE_VERIFY_TOPK ? a.K : 1);
+#pragma unroll
+        for (int rr = 0; rr < ee::kLmMaxK; ++rr)
+          tk_[c][rr] = use && rr < a.K && a.mode != EE_VERIFY_DIRECT ? ld_i(tk + (size_t)(o + par) * a.K + rr) : 0;
+      }
+    }
     int key_best = -1;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
@@ -221,20 +241,17 @@ __device__ void accept_sequences(const AcceptArgs& a, const int32_t* am, const i
       bool bad = false;
       if (i < T && i > 0) {
         const int par = par_[c];
+        const int tok = tok_[c];
         if (par < 0 || par >= i) {
           bad = true;
-        } else {
-          const int tok = tok_[c];
-          if (!kVerify || (a.gen_mask && !a.gen_mask[o + i])) {
-            bad = tok != ld_i(am + o + par);               // reused code: greedy
-          } else if (a.mode == EE_VERIFY_DIRECT) {
-            bad = false;
-          } else {
-            const int lim = a.mode == EE_VERIFY_GREEDY ? 1
-                          : (a.mode == EE_VERIFY_TOPK ? a.K : ld_i(tau + o + par));
+        } else if (!kVerify || !gen_[c]) {
+          bad = tok != am_[c];               // reused code: greedy
+        } else if constexpr (kVerify) {
+          if (a.mode != EE_VERIFY_DIRECT) {
             bad = true;
-            for (int rr = 0; rr < lim; ++rr)
-              if (ld_i(tk + (size_t)(o + par) * a.K + rr) == tok) bad = false;
+#pragma unroll
+            for (int rr = 0; rr < ee::kLmMaxK; ++rr)
+              if (rr < a.K && rr < tau_[c] && tk_[c][rr] == tok) bad = false;
           }
         }
       }
@@ -550,66 +567,58 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
           }
           __syncwarp();
           // (2) top-K per node column: a row is a candidate when its key beats the
-          //     CTA's shared threshold; up to four candidates are inserted into
-          //     the warp's sorted list by lane 0, more re-select the K best of
-          //     list + candidates with K rounds of a warp argmax
+          //     CTA's shared threshold.  Lane k holds entry k of the warp's sorted
+          //     list; a candidate's place is the number of better entries (one
+          //     ballot) and the worse ones move down one lane.  An empty list (the
+          //     first tile, where every row is a candidate) takes its K best by K
+          //     warp maxima, the lowest lane, i.e. row, first among equals.  (With
+          //     lane 0 inserting in shared memory and two warp reductions per pick
+          //     the first tile's epilogue outlasted two tiles' weight streams.)
           const int row0 = vt * p.BMr + q * 32;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            float* lv = s_lv + (size_t)(ew * BN + c0 + j) * K;
-            int* li = s_li + (size_t)(ew * BN + c0 + j) * K;
             const bool cand = row_ok && make_key(v0[j], row) > s_thr[c0 + j];
             unsigned mask = __ballot_sync(0xffffffffu, cand);
             if (mask == 0u) continue;
-            if (__popc(mask) <= 4) {
+            float* lv = s_lv + (size_t)(ew * BN + c0 + j) * K;
+            int* li = s_li + (size_t)(ew * BN + c0 + j) * K;
+            float av = lane < K ? lv[lane] : -INFINITY;
+            int ai = lane < K ? li[lane] : 0x7fffffff;
+            if (__shfl_sync(0xffffffffu, ai, 0) == 0x7fffffff) {
+              uint32_t key = cand ? ordered(v0[j]) : 0u;
+              for (int rr = 0; rr < K; ++rr) {
+                const uint32_t mx = __reduce_max_sync(0xffffffffu, key);
+                if (mx == 0u) break;   // fewer candidates than K
+                const int src = __ffs(__ballot_sync(0xffffffffu, key == mx)) - 1;
+                if (lane == src) key = 0u;
+                if (lane == rr) {
+                  av = unordered(mx);
+                  ai = row0 + src;
+                }
+              }
+            } else {
               while (mask) {
                 const int src = __ffs(mask) - 1;
                 mask &= mask - 1;
                 const float cv = __shfl_sync(0xffffffffu, v0[j], src);
                 const int ci = row0 + src;
-                if (lane == 0 && better(cv, ci, lv[K - 1], li[K - 1])) {
-                  int pos = K - 1;
-                  while (pos > 0 && better(cv, ci, lv[pos - 1], li[pos - 1])) {
-                    lv[pos] = lv[pos - 1];
-                    li[pos] = li[pos - 1];
-                    --pos;
-                  }
-                  lv[pos] = cv;
-                  li[pos] = ci;
-                }
-                __syncwarp();
-              }
-            } else {
-              float av = lane < K ? lv[lane] : -INFINITY;
-              int ai = lane < K ? li[lane] : 0x7fffffff;
-              float bv = cand ? v0[j] : -INFINITY;
-              int bi = cand ? row : 0x7fffffff;
-              __syncwarp();
-              for (int rr = 0; rr < K; ++rr) {
-                const bool useA = better(av, ai, bv, bi);
-                const float mv = useA ? av : bv;
-                const int mi = useA ? ai : bi;
-                float xv;
-                int xi;
-                warp_best(mv, mi, &xv, &xi);
-                if (mi == xi && mv == xv) {   // (value, id) pairs are unique: this lane held it
-                  if (useA) {
-                    av = -INFINITY;
-                    ai = 0x7fffffff;
-                  } else {
-                    bv = -INFINITY;
-                    bi = 0x7fffffff;
-                  }
-                }
-                if (lane == 0) {
-                  lv[rr] = xv;
-                  li[rr] = xi;
+                const int pos = __popc(__ballot_sync(0xffffffffu, lane < K && better(av, ai, cv, ci)));
+                const float uv = __shfl_up_sync(0xffffffffu, av, 1);
+                const int ui = __shfl_up_sync(0xffffffffu, ai, 1);
+                if (lane > pos) {
+                  av = uv;
+                  ai = ui;
+                } else if (lane == pos) {
+                  av = cv;
+                  ai = ci;
                 }
               }
-              __syncwarp();
             }
-            if (lane == 0 && li[K - 1] != 0x7fffffff)
-              atomicMax(&s_thr[c0 + j], make_key(lv[K - 1], li[K - 1]));
+            if (lane < K) {
+              lv[lane] = av;
+              li[lane] = ai;
+            }
+            if (lane == K - 1 && ai != 0x7fffffff) atomicMax(&s_thr[c0 + j], make_key(av, ai));
             __syncwarp();
           }
         }
@@ -818,7 +827,8 @@ __global__ void __launch_bounds__(32 * kFinWarps, 1) lm_verify_finalize_kernel(c
 #pragma unroll
     for (int u = 0; u < kMaxU; ++u) {
       const bool valid = lane + 32 * u < p.n_src;
-      if (valid) lse_add(m, sm, xs[u].x, xs[u].y);
+      if (!valid) xs[u] = make_float2(-INFINITY, 0.f);
+      m = fmaxf(m, xs[u].x);
 #pragma unroll
       for (int rr = 0; rr < K; ++rr)
         if (!valid) {
@@ -826,12 +836,11 @@ __global__ void __launch_bounds__(32 * kFinWarps, 1) lm_verify_finalize_kernel(c
           ci[u][rr] = 0x7fffffff;
         }
     }
+    m = unordered(__reduce_max_sync(0xffffffffu, ordered(m)));
 #pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-      const float mo = __shfl_xor_sync(0xffffffffu, m, d);
-      const float so = __shfl_xor_sync(0xffffffffu, sm, d);
-      lse_add(m, sm, mo, so);
-    }
+    for (int u = 0; u < kMaxU; ++u) sm += xs[u].x == -INFINITY ? 0.f : xs[u].y * ex2f((xs[u].x - m) * kLog2e);
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) sm += __shfl_xor_sync(0xffffffffu, sm, d);
     const float lse = m + logf(sm);
     // survivors into the warp's buffer
     float* sv = s_sv[warp];
