@@ -91,12 +91,13 @@ constexpr int kSB = 3;                           // S buffers in TMEM (Q.K^T run
 constexpr uint32_t kKVHalf = kKT * 128;          // 16 KB: one 64-dim half of a K or V tile
 constexpr uint32_t kKVBytes = 2 * kKVHalf;       // 32 KB
 constexpr int kMaxCtaPages = 2048;               // context pages one CTA owns at most (32768 keys)
+constexpr int kSegRing = 16;                     // published segments (K runs at most 8 ahead of the softmax)
 constexpr int kMaskRing = 8;                     // page-validity masks in flight (K runs at most 6 tiles ahead)
 constexpr uint32_t kOffK = 0;
 constexpr uint32_t kOffV = kOffK + kKST * kKVBytes;
 constexpr uint32_t kOffQ = kOffV + kVST * kKVBytes;  // Q block, 128 rows x 128 bf16, SW128 K-major
 constexpr uint32_t kOffBar = kOffQ + kKVBytes;
-constexpr uint32_t kNumBars = 2 * kKST + 2 * kVST + 3 * kSB + 6;
+constexpr uint32_t kNumBars = 2 * kKST + 2 * kVST + 3 * kSB + 5 + kSegRing;
 constexpr uint32_t kSmemBytes = 1024 + kOffBar + 8 * kNumBars + 64;
 constexpr uint32_t kTmemCols = 512;              // S0 [0,128) S1 [128,256) S2 [256,384) O [384,512)
 constexpr uint32_t kColO = 384;
@@ -106,7 +107,10 @@ constexpr int kMaxSplits = ee::kAttnMaxSplits;   // chunks per row block (cooper
 constexpr int kMaxBalSeqs = 512;                 // sequences of a balanced launch
 // warp roles; softmax warps 4..11, two per TMEM lane quarter
 constexpr int kWarpK = 0, kWarpPv = 1, kWarpV = 2, kWarpQk = 3, kWarpSoft0 = 4;
-constexpr int kSoftWarps = 8;
+constexpr int kSoftWarps = 8, kSoftThreads = 32 * kSoftWarps;
+// registers per thread: at launch (__launch_bounds__(384, 1)), then by role in a uniform launch
+constexpr int kRegsLaunch = 168, kRegsSoft = 208, kRegsOther = 88;
+static_assert(kSoftThreads * kRegsSoft + 32 * kWarpSoft0 * kRegsOther <= kThreads * kRegsLaunch, "register split");
 
 static_assert(kRows == ee::kAttnRows, "row block size");
 static_assert(kThreads == 32 * (kWarpSoft0 + kSoftWarps), "eight softmax warps, two per TMEM lane quarter");
@@ -147,69 +151,80 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return r;
 }
 
-// Merge rows [r0, r0 + nown) of a row block (query rows row0, ...) from its S
+// Merge rows [r0, r0 + nown) of a row block (query rows row0, ...) from its K
 // partial slots with log-sum-exp weights (Sec. III-A: the scores of one row
-// are normalised over all keys it sees) and write the fp32 output.  Thread t
-// takes row t % nown and the 16-byte column chunks t / nown + k * tpr, where
-// tpr = 256 / nown threads share a row: the loads of a warp for one chunk are
-// contiguous, and every load is issued before the first one is used.  Rows
-// without keys have (m, l) = (-inf, 0) and weight 0; their O words, never
-// written, are not used.
-template <int S>
-__device__ __forceinline__ void merge_rows(const AttnParams& p, size_t slot_a, size_t slot_b, int stride,
-                                           int row0, int r0, int nown, int o, int hk) {
+// are normalised over all keys it sees) and write the fp32 output.  The softmax
+// threads do it (nthr of them): thread t takes row t % nown and the 16-byte
+// column chunks t / nown + k * tpr, where tpr = nthr / nown threads share a row:
+// the loads of a warp for one chunk are contiguous, and up to kOut chunks' loads
+// from all slots (K <= kMax) are issued before the first is used.  Rows without keys have
+// (m, l) = (-inf, 0) and weight 0; their O words, never written, are not used.
+template <int kMax, int kOut>
+__device__ __forceinline__ void merge_rows(const AttnParams& p, size_t slot_a, size_t slot_b, int stride, int K,
+                                           int row0, int r0, int nown, int o, int hk, int tid, int nthr) {
   // partial s lives in slot slot_a (s = 0) or slot_b + (s - 1) * stride
   auto slot = [&](int s) -> const uint8_t* {
     return p.part + (s == 0 ? slot_a : slot_b + (size_t)(s - 1) * stride) * kAttnPartBytes;
   };
-  constexpr int kRpc = (kRows + S - 1) / S;
-  constexpr int kTprMin = kThreads / kRpc;
-  constexpr int kCh = (kD / 4 + kTprMin - 1) / kTprMin;   // chunks per thread, at most
-  const int tpr = kThreads / nown;                        // >= kTprMin, as nown <= kRpc
-  const int j = threadIdx.x % nown, cg = threadIdx.x / nown;
+  const int tpr = nthr / nown;
+  const int cg = tid / nown, j = tid - cg * nown;
   if (cg >= tpr) return;
-  float2 ml[S];
+  float2 ml[kMax];
 #pragma unroll
-  for (int s = 0; s < S; ++s)
-    ml[s] = __ldcg(reinterpret_cast<const float2*>(slot(s) + kAttnMlOff) + r0 + j);
-  float4 v[kCh][S];
-#pragma unroll
-  for (int k = 0; k < kCh; ++k) {
-    const int c = cg + k * tpr;
-#pragma unroll
-    for (int s = 0; s < S; ++s)
-      v[k][s] = c < kD / 4 ? __ldcg(reinterpret_cast<const float4*>(slot(s)) +
-                                    (size_t)c * kRows + r0 + j)
-                           : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  float M = -INFINITY;
-#pragma unroll
-  for (int s = 0; s < S; ++s) M = fmaxf(M, ml[s].x);
-  float w[S], L = 0.f;
-#pragma unroll
-  for (int s = 0; s < S; ++s) {
-    w[s] = ml[s].x == -INFINITY ? 0.f : ex2(ml[s].x - M);
-    L += w[s] * ml[s].y;
-  }
-  const float il = L == 0.f ? 0.f : 1.f / L;   // NaN scores stay NaN
+  for (int s = 0; s < kMax; ++s)
+    ml[s] = s < K ? __ldcg(reinterpret_cast<const float2*>(slot(s) + kAttnMlOff) + r0 + j)
+                  : make_float2(-INFINITY, 0.f);
   const int rrow = row0 + j;
   const int nd = rrow / p.g;
   float4* dst = reinterpret_cast<float4*>(p.out + ((size_t)(o + nd) * p.n_q + hk * p.g + (rrow - nd * p.g)) * kD);
+  float M = -INFINITY, il = 0.f, w[kMax];
+  for (int c0 = cg; c0 < kD / 4; c0 += kOut * tpr) {
+    float4 v[kOut][kMax];
 #pragma unroll
-  for (int k = 0; k < kCh; ++k) {
-    const int c = cg + k * tpr;
-    if (c >= kD / 4) break;
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < kOut; ++k) {
+      const int c = c0 + k * tpr;
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      if (w[s] == 0.f) continue;
-      a.x = fmaf(w[s], v[k][s].x, a.x);
-      a.y = fmaf(w[s], v[k][s].y, a.y);
-      a.z = fmaf(w[s], v[k][s].z, a.z);
-      a.w = fmaf(w[s], v[k][s].w, a.w);
+      for (int s = 0; s < kMax; ++s)
+        v[k][s] = (c < kD / 4 && s < K)
+                      ? __ldcg(reinterpret_cast<const float4*>(slot(s)) + (size_t)c * kRows + r0 + j)
+                      : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    dst[c] = make_float4(a.x * il, a.y * il, a.z * il, a.w * il);
+    if (c0 == cg) {   // the weights, while the first chunks are in flight
+#pragma unroll
+      for (int s = 0; s < kMax; ++s) M = fmaxf(M, ml[s].x);
+      float L = 0.f;
+#pragma unroll
+      for (int s = 0; s < kMax; ++s) {
+        w[s] = ml[s].x == -INFINITY ? 0.f : ex2(ml[s].x - M);
+        L += w[s] * ml[s].y;
+      }
+      il = L == 0.f ? 0.f : 1.f / L;   // NaN scores stay NaN
+    }
+#pragma unroll
+    for (int k = 0; k < kOut; ++k) {
+      const int c = c0 + k * tpr;
+      if (c >= kD / 4) break;
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int s = 0; s < kMax; ++s) {
+        if (w[s] == 0.f) continue;
+        a.x = fmaf(w[s], v[k][s].x, a.x);
+        a.y = fmaf(w[s], v[k][s].y, a.y);
+        a.z = fmaf(w[s], v[k][s].z, a.z);
+        a.w = fmaf(w[s], v[k][s].w, a.w);
+      }
+      dst[c] = make_float4(a.x * il, a.y * il, a.z * il, a.w * il);
+    }
   }
+}
+// kX: 16 kX loads per thread in flight
+template <int kX>
+__device__ __forceinline__ void merge_pieces(const AttnParams& p, size_t slot_a, size_t slot_b, int stride, int K,
+                                             int row0, int r0, int nown, int o, int hk, int tid, int nthr) {
+  if (K <= 2) merge_rows<2, 8 * kX>(p, slot_a, slot_b, stride, K, row0, r0, nown, o, hk, tid, nthr);
+  else if (K <= 4) merge_rows<4, 4 * kX>(p, slot_a, slot_b, stride, K, row0, r0, nown, o, hk, tid, nthr);
+  else if (K <= 8) merge_rows<8, 2 * kX>(p, slot_a, slot_b, stride, K, row0, r0, nown, o, hk, tid, nthr);
+  else merge_rows<16, kX>(p, slot_a, slot_b, stride, K, row0, r0, nown, o, hk, tid, nthr);
 }
 
 // A row block's partial that this CTA merges with the other pieces of the same
@@ -254,10 +269,17 @@ __device__ __forceinline__ int row_node(const AttnParams& p, int r) {
   return p.g <= 1024 ? (int)__umulhi((uint32_t)r, p.g_inv) : r / p.g;
 }
 
+// chain_rb_tiles without the division
+__device__ __forceinline__ int chain_tiles(const AttnParams& p, int ctx, int T, int r) {
+  return (ctx + min(T - 1, row_node(p, (r + 1) * kRows - 1)) + kKT) / kKT;
+}
+
 // One segment: a contiguous range of one row block's tiles, run in the order
-// rot, rot + 1, ..., n_tiles - 1, 0, ..., rot - 1.  Every role decodes the
-// CTA's segments by itself (same inputs, same result), so no CTA barrier
-// separates one segment from the next.
+// rot, rot + 1, ..., n_tiles - 1, 0, ..., rot - 1.  In a balanced launch the K
+// producer, which runs ahead of every other role, decodes the CTA's segments and
+// publishes them in a ring in shared memory (one mbarrier each): no CTA barrier
+// separates one segment from the next, and the decode (about 2,000 cycles of
+// dependent integer work) is off the other roles' path.
 struct Seg {
   int b, hk, rb, o, T, ctx;    // sequence, KV head, row block, node offset, nodes, context length
   int k_begin, k_end;          // paged keys
@@ -310,32 +332,41 @@ __device__ __forceinline__ void bal_segment(const AttnParams& p, const WorkList&
     const int local = y - 1 - base_w;
     s.hk = (int)((unsigned)local / (unsigned)tiles);
     const int rem = local - s.hk * tiles;
-    // the row block holding tile rem: a scan of the row blocks' tile counts, 32 at a time
-    int r = nrb_b - 1, cum = 0, tu = 0;
-    for (int r0 = 0, base = 0; r0 < nrb_b; r0 += 32) {
-      const int rr = r0 + lane;
-      const int t = rr < nrb_b ? chain_rb_tiles(s.ctx, s.T, g, rr) : 0;
-      int incl = t;
+    // the row block holding tile rem: a scan of the row blocks' tile counts, four
+    // consecutive ones per lane
+    int r = nrb_b - 1, cum = 0, tu = 1;
+    for (int r0 = 0, base = 0; r0 < nrb_b; r0 += 128) {
+      int t[4], sum = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int rr = r0 + 4 * lane + q;
+        t[q] = rr < nrb_b ? chain_tiles(p, s.ctx, s.T, rr) : 0;
+        sum += t[q];
+      }
+      int incl = sum;
 #pragma unroll
       for (int dd = 1; dd < 32; dd <<= 1) {
         const int v = __shfl_up_sync(0xffffffffu, incl, dd);
         if (lane >= dd) incl += v;
       }
-      const int excl = base + incl - t;
-      const unsigned hit = __ballot_sync(0xffffffffu, rr < nrb_b && rem >= excl && rem < excl + t);
+      int excl = base + incl - sum;
+      const unsigned hit = __ballot_sync(0xffffffffu, rem >= excl && rem < excl + sum);
       if (hit) {
         const int src = __ffs(hit) - 1;
-        r = r0 + src;
+        int q = 0;      // (the owner lane's)
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+          if (q == k && rem >= excl + t[k]) {
+            excl += t[k];
+            q = k + 1;
+          }
+        const int tq = q == 0 ? t[0] : q == 1 ? t[1] : q == 2 ? t[2] : t[3];
+        r = r0 + 4 * src + __shfl_sync(0xffffffffu, q, src);
         cum = __shfl_sync(0xffffffffu, excl, src);
-        tu = __shfl_sync(0xffffffffu, t, src);
+        tu = __shfl_sync(0xffffffffu, tq, src);
         break;
       }
       base += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (tu == 0) {   // not reached for a consistent work list
-      cum = 0;
-      for (int q = 0; q < r; ++q) cum += chain_rb_tiles(s.ctx, s.T, g, q);
-      tu = chain_rb_tiles(s.ctx, s.T, g, r);
     }
     s.rb = r;
     U0 = base_w + s.hk * tiles + cum;
@@ -352,7 +383,7 @@ __device__ __forceinline__ void bal_segment(const AttnParams& p, const WorkList&
   const int n_ctx_b = kIP ? tiles : tiles - 1;   // paged tiles of the unit
   s.k_begin = min(t0, n_ctx_b) * kKT;
   const int unit_span =
-      kChain ? s.ctx + min(s.T, ((s.rb + 1) * kRows - 1) / g + 1) : (kIP ? s.ctx + s.T : s.ctx);
+      kChain ? s.ctx + min(s.T, row_node(p, (s.rb + 1) * kRows - 1) + 1) : (kIP ? s.ctx + s.T : s.ctx);
   s.k_end = t0 < n_ctx_b ? min(unit_span, min(t0 + len, n_ctx_b) * kKT) : s.k_begin;
   s.n_ctx = s.k_end > s.k_begin ? (s.k_end - s.k_begin + kKT - 1) / kKT : 0;
   s.n_tiles = s.n_ctx + (!kIP && t0 + len == tiles ? 1 : 0);
@@ -392,7 +423,7 @@ __device__ __forceinline__ bool uni_segment(const AttnParams& p, bool report, Se
   // everything above is uniform over the row block's CTAs; from here on every
   // CTA reaches the merge synchronisation
   // paged keys of the row block (chain: up to its last node's position)
-  const int span = kChain ? s.ctx + min(s.T, ((s.rb + 1) * kRows - 1) / p.g + 1) : (kIP ? s.ctx + s.T : s.ctx);
+  const int span = kChain ? s.ctx + min(s.T, row_node(p, (s.rb + 1) * kRows - 1) + 1) : (kIP ? s.ctx + s.T : s.ctx);
   const int S = attn_splits_for(span, p.chunk);  // chunks this sequence uses, <= p.S
   const bool active = split < S;
   s.k_begin = split * p.chunk;
@@ -469,6 +500,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   __shared__ int4 s_seq[kBal ? kMaxBalSeqs : 1];
   __shared__ int s_wpre[kBal ? kMaxBalSeqs + 1 : 1];
   __shared__ int s_sched[5];                        // balanced: range start, range end, W, N, ceil(W / N)
+  __shared__ Seg s_seg[kBal ? kSegRing : 1];        // balanced: published segments (n_tiles 0: no more)
   __shared__ BalPiece s_pc[2];                      // this CTA's pieces of split row blocks
   __shared__ int s_npc;
   __shared__ int2 s_uni;                            // uniform: the row block's node offset and rows
@@ -481,7 +513,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   const uint32_t v_full = k_empty + 8 * kKST, v_empty = v_full + 8 * kVST;
   const uint32_t s_full = v_empty + 8 * kVST, p_full = s_full + 8 * kSB, pv_done = p_full + 8 * kSB;
   const uint32_t drain = pv_done + 8 * kSB, q_ready = drain + 16, q_empty = q_ready + 8, o_free = q_empty + 8;
-  const uint32_t q_half = o_free + 8;
+  const uint32_t seg_full = o_free + 8;
 
   // on-chip set-up first: it touches no global memory, so it overlaps the end
   // of the previous kernel in the stream
@@ -513,7 +545,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
     mbar_init(q_ready, kSoftWarps);
     mbar_init(q_empty, 1);
     mbar_init(o_free, kSoftWarps);
-    mbar_init(q_half, 1);
+    for (int i = 0; i < kSegRing; ++i) mbar_init(seg_full + 8 * i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
@@ -540,9 +572,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   // start the next (at most two of its segments are pieces of split units).
   // N is capped so that every CTA gets at least m = max(2, ceil(t_max / 14))
   // tiles, which bounds the pieces of any unit by 15.
-  // Warp kWarpQk builds it: lane l takes sequences [per l, per l + per), per = ceil(B / 32).
+  // The K producer builds it: lane l takes sequences [per l, per l + per), per = ceil(B / 32).
   if constexpr (kBal) {
-    if (warp == kWarpQk) {
+    if (warp == kWarpK) {
       const int per = (p.B + 31) >> 5;     // sequences of a lane
       int wsum = 0, tmax = 0;
       for (int k = 0; k < per; ++k) {      // (clamped indices)
@@ -562,7 +594,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
           const int c = min(max(sq.z, 0), p.max_ctx);
           int acc = 0;
           if (!bad)
-            for (int r = lane; r < (Tb * g + kRows - 1) / kRows; r += 32) acc += chain_rb_tiles(c, Tb, g, r);
+            for (int r = lane; r < (Tb * g + kRows - 1) / kRows; r += 32) acc += chain_tiles(p, c, Tb, r);
           acc = __reduce_add_sync(0xffffffffu, acc);
           __syncwarp();
           if (lane == 0) s_seq[bb].w = acc;
@@ -590,9 +622,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
             tiles = sq.w;
             if (!coop) {
               tiles = 0;
-              for (int r = 0; r < nrb_b && !bad; ++r) tiles += chain_rb_tiles(c, Tb, g, r);
+              for (int r = 0; r < nrb_b && !bad; ++r) tiles += chain_tiles(p, c, Tb, r);
             }
-            unit_max = bad ? 1 : chain_rb_tiles(c, Tb, g, nrb_b - 1);
+            unit_max = bad ? 1 : chain_tiles(p, c, Tb, nrb_b - 1);
           }
           if (!bad) {
             wl = p.n_kv * (kChain ? 1 : nrb_b) * tiles;
@@ -627,20 +659,46 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
         s_sched[4] = N > 0 ? (W + N - 1) / N : 1;
         s_wpre[p.B] = W;
       }
+      __syncwarp();
     }
-    __syncthreads();
   }
 
   const WorkList wlist{s_seq, s_wpre, s_sched};
-  // The CTA's segments, decoded by each role: `first` starts the walk, `next`
-  // moves to the following segment (tiles before it: tb, segments before it: nseg).
+  // wait outcomes are made warp-uniform: what follows is warp-collective
+  auto wait = [&](uint32_t bar, int use) -> bool {
+    return __all_sync(0xffffffffu, mbar_wait(bar, (uint32_t)(use & 1), &s_abort));
+  };
+  // The CTA's segments: `first` starts the walk, `next` moves to the following
+  // segment (tiles before it: tb, segments before it: nseg).
   Seg sg;
   int tb = 0, nseg = 0;
+  // balanced, the K producer: segment n (ending at y, tb0 tiles before it),
+  // decoded and published
+  auto publish = [&](int n, int y, int tb0, Seg& o) {
+    o.n_tiles = 0;
+    if (y > s_sched[0]) bal_segment<kKV>(p, wlist, y, tb0, lane, o);
+    if (lane == 0) {
+      s_seg[kBal ? n % kSegRing : 0] = o;
+      mbar_arrive(seg_full + 8 * (n % kSegRing));
+    }
+    __syncwarp();
+  };
+  // the other roles: segment nseg, received
+  auto receive = [&]() -> bool {
+    if (!wait(seg_full + 8 * (nseg % kSegRing), nseg / kSegRing)) return false;
+    sg = s_seg[kBal ? nseg % kSegRing : 0];
+    return sg.n_tiles > 0;
+  };
+  if constexpr (kBal) {
+    // the first segment meets a CTA barrier: eleven warps polling an mbarrier would
+    // take the issue slots the K warp builds and decodes with
+    if (warp == kWarpK) publish(0, s_sched[1], 0, sg);
+    __syncthreads();
+  }
   auto first = [&](bool report) -> bool {
     if constexpr (kBal) {
-      if (s_sched[1] <= s_sched[0]) return false;
-      bal_segment<kKV>(p, wlist, s_sched[1], 0, lane, sg);
-      return true;
+      if (warp != kWarpK) sg = s_seg[0];
+      return sg.n_tiles > 0;
     } else {
       return uni_segment<kKV>(p, report, sg);
     }
@@ -649,18 +707,18 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
     if constexpr (kBal) {
       tb += sg.n_tiles;
       ++nseg;
-      if (sg.y <= s_sched[0]) return false;
-      bal_segment<kKV>(p, wlist, sg.y, tb, lane, sg);
-      return true;
+      return receive();
     } else {
       return false;
     }
   };
-  // wait outcomes are made warp-uniform: what follows is warp-collective
-  auto wait = [&](uint32_t bar, int use) -> bool {
-    return __all_sync(0xffffffffu, mbar_wait(bar, (uint32_t)(use & 1), &s_abort));
-  };
 
+  // Uniform launches: the merge keeps 32 loads a thread in flight, so the softmax
+  // warps, which run it, take registers from the others (the shares add up to the
+  // launch's).  A balanced launch's producers need theirs: with 88 registers the K
+  // warp spills and the tile period grows (33B-shaped layer 129.5 -> 134 us).
+  if (warp < kWarpSoft0) {
+  if constexpr (!kBal) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
   if (warp == kWarpK || warp == kWarpV) {
     // ---------------- TMA producers: warp 0 streams K, warp 2 streams V ----------------
     // Ring slots and phases count the CTA's tiles over all its segments.  Lane l
@@ -699,27 +757,35 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
       }
     }
     bool go = true;
-    for (; more && go; more = next()) {
-      // page ids of tiles 4 c .. 4 c + 3 of the segment's order; INT_MIN: no keys there
-      auto fetch = [&](int c) -> int32_t {
-        const int t = 4 * c + (lane >> 3);
-        if (t >= sg.n_tiles) return INT32_MIN;
-        const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;
-        const int pos = sg.k_begin + i * kKT + 16 * (lane & 7);
-        if (i >= sg.n_ctx || pos >= sg.k_end) return INT32_MIN;
-        if (!kBal && c == 0) return max(early, -1);
-        return max(ld_nc_pinned(p.block_table + (size_t)sg.b * p.max_pages + pos / EE_PAGE), -1);
-      };
-      int32_t ids = fetch(0), ids_next = INT32_MIN;
+    // page ids of tiles 4 c .. 4 c + 3 of the segment's order (INT_MIN: no keys
+    // there), one predicated load that nothing waits for before the ids are used
+    auto fetch = [&](const Seg& sg, int c) -> int32_t {
+      const int t = 4 * c + (lane >> 3);
+      const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;
+      const int pos = sg.k_begin + i * kKT + 16 * (lane & 7);
+      const bool need = t < sg.n_tiles && i < sg.n_ctx && pos < sg.k_end;
+      if (!kBal && c == 0) return need ? early : INT32_MIN;
+      int32_t v = INT32_MIN;
+      if (need) v = ld_nc_pinned(p.block_table + (size_t)sg.b * p.max_pages + pos / EE_PAGE);
+      return v;
+    };
+    // balanced, the K producer: the next segment (decoded and published, its first
+    // page ids on the way, while this one's tiles wait for ring slots)
+    int32_t nx_ids = INT32_MIN;
+    while (more && go) {
+      int32_t ids = kBal && isK && nseg > 0 ? nx_ids : fetch(sg, 0), ids_next = INT32_MIN;
       for (int t = 0; t < sg.n_tiles; ++t) {
         if ((t & 3) == 0) {
           if (t > 0) ids = ids_next;
-          ids_next = fetch((t >> 2) + 1);
+          ids_next = fetch(sg, (t >> 2) + 1);
         }
         const int tg = tb + t;
         const int st = tg % nst, use = tg / nst;
         // the tile's eight blocks, the same in every lane: first cache row, -EE_PAGE
-        // without a page
+        // without a page; need8: the blocks that hold keys
+        const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;   // the segment's tile
+        const int left = sg.k_end - (sg.k_begin + i * kKT);
+        const unsigned need8 = i >= sg.n_ctx ? 0u : left >= kKT ? 0xFFu : (1u << ((left + 15) >> 4)) - 1u;
         int row[kKT / 16];
         unsigned okm = 0u;      // bit i: block i has keys in a valid page
         bool bad = false;
@@ -729,14 +795,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
           const bool ok = id >= 0 && id < p.num_pages;
           row[q] = ok ? (id * p.n_kv + sg.hk) * EE_PAGE : -EE_PAGE;
           okm |= ok ? 1u << q : 0u;
-          bad |= !ok && id != INT32_MIN;
+          bad |= !ok && (need8 >> q & 1u);
         }
         if (isK && bad && lane == 0) flag_error(p.err, EE_DEVERR_PAGE);
         go = wait(empty0 + 8 * st, use + 1);
         if (!go) break;
         const uint32_t full = full0 + 8 * st;
         const uint32_t dst = ring + st * kKVBytes;
-        const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;   // the segment's tile
         if (elect_one()) {
           if (isK) s_mask[tg % kMaskRing] = okm;
           mbar_expect_tx(full, 2 * kKVHalf);
@@ -757,13 +822,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
         __syncwarp();
         if (lane == 0) issued[st] = use;
         if constexpr (kBal) {
-          // a later segment's Q rows 64 .. 127, once its first tiles are in the ring
-          // (the next slot frees only after this segment's first Q.K^T)
-          if (isK && nseg > 0 && t == min(kKST - 1, sg.n_tiles - 1)) {
-            go = wait(q_empty, nseg - 1);
-            if (!go) break;
-            load_q<2, kRows / 4>(p, sg, sQ, kRows / 2, lane);
-            if (lane == 0) mbar_arrive(q_half);
+          if (isK && t == min(kKST - 1, sg.n_tiles - 1)) {
+            Seg nx;
+            publish(nseg + 1, sg.y, tb + sg.n_tiles, nx);
+            nx_ids = fetch(nx, 0);
           }
           // the piece of a split row block, and its count as read before this
           // CTA's own arrival
@@ -779,6 +841,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
             s_npc = s_npc + 1;
           }
         }
+      }
+      if (kBal && isK) {
+        tb += sg.n_tiles;
+        ++nseg;
+        sg = s_seg[kBal ? nseg % kSegRing : 0];
+        more = sg.n_tiles > 0;
+      } else {
+        more = next();
       }
     }
   } else if (warp == kWarpQk) {
@@ -799,8 +869,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
         // the previous segment's last Q.K^T has read its rows; the load runs while
         // its last kSB tiles are in the softmax
         go = wait(q_empty, nseg - 1);
-        if (go) load_q<2, kRows / 4>(p, sg, sQ, 0, lane);
-        go = go && wait(q_half, nseg - 1);   // the K warp loads the other half
+        if (go) load_q<2, kRows / 2>(p, sg, sQ, 0, lane);
       }
       tc_fence_after();
       for (int t = 0; t < sg.n_tiles && go; ++t) {
@@ -857,375 +926,347 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
         __syncwarp();
       }
     }
-  } else {
-    // ---------------- softmax: one query row and half of every tile per thread ----------------
-    // Warps w and w + 4 share TMEM lane quarter w & 3 (32 query rows); half hf
-    // of the pair takes keys [64 hf, 64 hf + 64) of every tile and O columns
-    // [64 hf, 64 hf + 64).  The pair agrees on each tile's row maximum through
-    // shared memory at a 64-thread named barrier, so both halves take the same
-    // rescale decisions; each keeps the sum over its own keys, and the two sums
-    // are added (half 0 first) at the end.  Two warps per sub-partition hide
-    // each other's latencies.  Every exit from the tile loop happens right
-    // after the pair barrier and on a decision both warps share.
-    const int qd = warp & 3;
-    const int hf = (warp - kWarpSoft0) >> 2;
-    const uint32_t pair_bar = 2 + qd;
-    const int r = qd * 32 + lane;                     // == TMEM lane of this quarter
-    const uint32_t tl = tmem + ((uint32_t)(qd * 32) << 16);
-    const float sl2 = p.scale_log2;
-    bool ok = true;
-    bool loaded = false;
-    for (bool more = first(false); more && ok; more = next()) {
-      const int R = sg.T * g;
-      const int rr = sg.rb * kRows + r;
-      const bool vrow = rr < R;
-      const int node = vrow ? row_node(p, rr) : 0;
-      if (!loaded) {   // the first row block's Q: each softmax warp copies 16 rows
-        load_q<2 * kSoftWarps, kRows / 2 / kSoftWarps>(p, sg, sQ, 2 * (warp - kWarpSoft0), lane);
-        if (lane == 0) mbar_arrive(q_ready);
-        loaded = true;
-      }
-      // this half's tree keys (separate tree tile), or the row's whole ancestor
-      // mask (in place: tree keys at any offset from a half's first key)
-      const uint64_t ancw = (!kChain && vrow) ? p.anc[2 * (size_t)(sg.o + node) + (kIP ? 0 : hf)] : 0ull;
-      const uint64_t anc_hi = (kKV == kKVInPlace && vrow) ? p.anc[2 * (size_t)(sg.o + node) + 1] : 0ull;
-      // m_used is kept in raw score units (scale > 0, so the max commutes with it)
-      float m_used = -INFINITY, l = 0.f;
-      // keys below full_end: every row sees all of them (when their pages are valid)
-      const int full_end = kIP ? min(sg.k_end, sg.ctx) : sg.k_end;
-      // step tg processes the segment's tile tg - tb + rot (mod n_tiles)
-      for (int t = 0; t < sg.n_tiles; ++t) {
-        const int tg = tb + t;
-        const int sb = tg % kSB;    // S buffer of this tile
-        const int xb = tg & 1;      // pair-exchange slot
-        const bool got = wait(s_full + 8 * sb, tg / kSB);
-        uint32_t sr[64];
-        float tmax = -INFINITY;
-        if (got) {
-          tc_fence_after();
-          tc_ld32_nowait(tl + sb * kKT + 64 * hf, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
-          tc_ld32_nowait(tl + sb * kKT + 64 * hf + 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
-          const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;
-          const unsigned pm = s_mask[tg % kMaskRing];     // bit j: 16-row block j has a valid page
-          const int p0 = sg.k_begin + i * kKT;            // the tile's first key
-          // a whole tile of context keys in valid pages needs no mask: every row
-          // sees all of it (rows past R hold zero queries and are never stored)
-          const bool whole = i < sg.n_ctx && pm == 0xFFu && p0 + kKT <= full_end;
-          tc_wait_ld32(*reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
-          tc_pin32(*reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
-          if (!whole) {
-            // visibility of this half's 64 keys as one 64-bit word
-            uint64_t kw;
-            const int h0 = p0 + 64 * hf;
-            if (i < sg.n_ctx) {
-              const int nv = min(max(sg.k_end - h0, 0), 64);
-              uint64_t pgw = 0ull;
-#pragma unroll
-              for (int pb = 0; pb < 4; ++pb)
-                pgw |= ((pm >> (4 * hf + pb)) & 1u) ? (0xFFFFull << (16 * pb)) : 0ull;
-              kw = pgw & (nv >= 64 ? ~0ull : ((1ull << nv) - 1ull));
-              if constexpr (kChain) {
-                // causal: node sees positions up to ctx + node
-                const int nvis = min(max(sg.ctx + node + 1 - h0, 0), 64);
-                kw &= nvis >= 64 ? ~0ull : ((1ull << nvis) - 1ull);
-              } else if constexpr (kIP) {
-                // keys below ctx are context; key p >= ctx is tree node p - ctx
-                const int nc = min(max(sg.ctx - h0, 0), 64);
-                const int sh = h0 - sg.ctx;    // ancestor bit of this half's first key
-                uint64_t tm;
-                if (sh >= 0)
-                  tm = sh >= 128 ? 0ull
-                       : sh >= 64 ? (anc_hi >> (sh - 64))
-                       : sh == 0  ? ancw
-                                  : ((ancw >> sh) | (anc_hi << (64 - sh)));
-                else
-                  tm = sh <= -64 ? 0ull : (ancw << (-sh));
-                kw &= (nc >= 64 ? ~0ull : ((1ull << nc) - 1ull)) | tm;
-              }
-            } else {
-              const int th = min(max(sg.T - 64 * hf, 0), 64);
-              kw = ancw & (th >= 64 ? ~0ull : ((1ull << th) - 1ull));
-            }
-            if (!vrow) kw = 0ull;
-#pragma unroll
-            for (int c = 0; c < 64; ++c)
-              if (!((kw >> c) & 1ull)) sr[c] = __float_as_uint(-INFINITY);
-          }
-          // 8 independent chains of three-input maxima over the 64 values
-          float mx[8];
-#pragma unroll
-          for (int c = 0; c < 8; ++c) mx[c] = __uint_as_float(sr[c]);
-#pragma unroll
-          for (int c = 8; c < 56; c += 16)         // values 8 .. 55, two per instruction
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-              mx[k] = fmax3(mx[k], __uint_as_float(sr[c + k]), __uint_as_float(sr[c + 8 + k]));
-#pragma unroll
-          for (int k = 0; k < 8; ++k) mx[k] = fmaxf(mx[k], __uint_as_float(sr[56 + k]));   // values 56 .. 63
-          tmax = fmax3(fmax3(mx[0], mx[1], mx[2]), fmax3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7]));
-        }
-        // the pair swaps its halves' maxima; both S halves are in registers before
-        // either warp overwrites S with P.  kFail (a NaN no maximum yields: theirs is
-        // 0x7fffffff) says that this half's wait failed
-        constexpr uint32_t kFail = 0xffffffffu;
-        s_xmax[xb][hf][r] = got ? __float_as_uint(tmax) : kFail;
-        tc_fence_before();
-        asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-        tc_fence_after();
-        const uint32_t other = s_xmax[xb][hf ^ 1][r];
-        if (!__all_sync(0xffffffffu, got && other != kFail)) {
-          ok = false;
-          break;
-        }
-        tmax = fmaxf(tmax, __uint_as_float(other));
-        const float m_new = fmaxf(m_used, tmax);
-        const bool need = (m_new - m_used) * sl2 > kRescaleLog2;   // true when m_used = -inf < m_new
-        if (t > 0 && __any_sync(0xffffffffu, need)) {
-          // O must hold P.V(tg-1) before this half's columns are rescaled; a failed
-          // wait sets the abort flag, and the pair stops at the next barrier
-          if (wait(pv_done + 8 * ((tg - 1) % kSB), (tg - 1) / kSB)) {
-            tc_fence_after();
-            const float f = need ? ex2((m_used - m_new) * sl2) : 1.f;
-#pragma unroll 1
-            for (int c4 = 0; c4 < 4; ++c4) {
-              uint32_t ov[16];
-              tc_ld16(tl + kColO + 64 * hf + 16 * c4, ov);
-#pragma unroll
-              for (int e = 0; e < 16; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * f);
-              tc_st16_nowait(tl + kColO + 64 * hf + 16 * c4, ov);
-            }
-            tc_wait_st();
-          } else {
-            ok = false;
-          }
-        }
-        if (need) {
-          l *= ex2((m_used - m_new) * sl2);
-          m_used = m_new;
-        }
-        const float nms = m_used == -INFINITY ? 0.f : -m_used * sl2;
-        // p = 2^(s*scale_log2 - m); P = head + tail, both bf16: this
-        // half's head pairs go to columns 32 hf.. of the S buffer, its tail pairs
-        // to 64 + 32 hf..
-        // (pairs of columns run on packed fp32x2 arithmetic: the scale-and-shift,
-        // the running sums and the tail subtraction take one instruction per pair)
-        const uint64_t sl2x2 = f2_pack(__float_as_uint(sl2), __float_as_uint(sl2));
-        const uint64_t nmsx2 = f2_pack(__float_as_uint(nms), __float_as_uint(nms));
-        uint64_t ls2[4];
-        // two halves of 16 column pairs: each half's head and tail words go
-        // out before the next half is computed (fewer live registers)
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          uint32_t hw[16], tw[16];
-#pragma unroll
-          for (int e2 = 0; e2 < 16; ++e2) {
-            const int e = 16 * hh + e2;
-            uint32_t y0, y1;
-            f2_unpack(f2_fma(f2_pack(sr[2 * e], sr[2 * e + 1]), sl2x2, nmsx2), y0, y1);
-            const uint32_t p0 = __float_as_uint(ex2(__uint_as_float(y0)));
-            const uint32_t p1 = __float_as_uint(ex2(__uint_as_float(y1)));
-            const uint64_t pp = f2_pack(p0, p1);
-            ls2[e & 3] = e < 4 ? pp : f2_add(ls2[e & 3], pp);
-            // head = p rounded to bf16; tail = the remainder p - head (exact
-            // in fp32) rounded to bf16
-            const uint32_t hb = bf16x2_rn(__uint_as_float(p1), __uint_as_float(p0));
-            float t0, t1;
-            sub_bf16x2(hb, __uint_as_float(p0), __uint_as_float(p1), t0, t1);
-            hw[e2] = hb;
-            tw[e2] = bf16x2_rn(t1, t0);
-          }
-          tc_st16_nowait(tl + sb * kKT + 32 * hf + 16 * hh, hw);
-          tc_st16_nowait(tl + sb * kKT + 64 + 32 * hf + 16 * hh, tw);
-        }
-        tc_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(p_full + 8 * sb);
-        {
-          uint32_t a0, a1, b0, b1, c0, c1, d0, d1;
-          f2_unpack(ls2[0], a0, a1);
-          f2_unpack(ls2[1], b0, b1);
-          f2_unpack(ls2[2], c0, c1);
-          f2_unpack(ls2[3], d0, d1);
-          l += ((__uint_as_float(a0) + __uint_as_float(a1)) + (__uint_as_float(b0) + __uint_as_float(b1))) +
-               ((__uint_as_float(c0) + __uint_as_float(c1)) + (__uint_as_float(d0) + __uint_as_float(d1)));
-        }
-      }
-      // wait for the last P.V (products complete in order, and this barrier's
-      // previous phase, P.V three tiles before, was over before the last S
-      // existed); the pair adds its two sums, then each half writes its 64
-      // columns out: O / l itself when the segment is a whole row block, else the
-      // partial (O, m, l) to the segment's slot
-      const int tl_g = tb + sg.n_tiles - 1;
-      const bool have = ok && sg.n_tiles > 0 && wait(pv_done + 8 * (tl_g % kSB), tl_g / kSB);
-      s_xl[hf][r] = l;
-      if (lane == 0) s_xok[nseg & 1][qd][hf] = have;
-      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-      const float l_sum = s_xl[0][r] + s_xl[1][r];
-      const bool both = s_xok[nseg & 1][qd][0] && s_xok[nseg & 1][qd][1];
-      const bool nan_row = both && vrow && l_sum != l_sum;   // NaN scores: the output is NaN
-      const float row_m =
-          nan_row ? 0.f : ((both && vrow && m_used != -INFINITY) ? m_used * sl2 : -INFINITY);
-      const float row_l = (both && vrow && (m_used != -INFINITY || nan_row)) ? l_sum : 0.f;
-      float4* dst;
-      size_t dstride;                                   // float4 between column chunks
-      float inv = 1.f;
-      if (sg.alone) {
-        const size_t orow = (size_t)(sg.o + node) * p.n_q + sg.hk * g + (rr - node * g);
-        dst = reinterpret_cast<float4*>(p.out + orow * kD);
-        dstride = 1;
-        inv = row_l == 0.f ? 0.f : 1.f / row_l;
-      } else {
-        dst = reinterpret_cast<float4*>(p.part + (size_t)sg.slot * kAttnPartBytes) + r;
-        dstride = kRows;
-      }
-      const bool store = sg.alone ? vrow : (row_l > 0.f || nan_row);
-      if (sg.n_tiles > 0) {
-        tc_fence_after();
-#pragma unroll 1
-        for (int c4 = 0; c4 < 2; ++c4) {
-          uint32_t ov[32];
-          tc_ld32(tl + kColO + 64 * hf + 32 * c4, ov);
-          if (c4 == 1) {   // O is in registers: the next segment's P.V may overwrite it
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(o_free);
-          }
-          if (store) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const float4 v = make_float4(__uint_as_float(ov[4 * e]) * inv, __uint_as_float(ov[4 * e + 1]) * inv,
-                                           __uint_as_float(ov[4 * e + 2]) * inv,
-                                           __uint_as_float(ov[4 * e + 3]) * inv);
-              __stcg(dst + (size_t)(16 * hf + 8 * c4 + e) * dstride, v);
-            }
-          }
-        }
-      }
-      if (!sg.alone) {
-        if (hf == 0)
-          __stcg(reinterpret_cast<float2*>(p.part + (size_t)sg.slot * kAttnPartBytes + kAttnMlOff) + r,
-                 make_float2(row_m, row_l));
-      }
-      if (!both) ok = false;
-    }
-  }
-  // ---- CTA teardown: drain on abort, free TMEM --------------------------------
-  tc_fence_before();
-  __syncthreads();
-  pdl_allow_next();   // this grid's pipeline is done: the next kernel may take SMs as they free
-  const bool aborted = s_abort != 0;
-  if (aborted && threadIdx.x == 0) {
-    flag_error(p.err, EE_DEVERR_TIMEOUT);
-    // TMA copies still in flight land before the rings are reused
-    for (int st = 0; st < kKST; ++st)
-      if (s_kissued[st] >= 0) mbar_wait_plain(k_full + 8 * st, (uint32_t)(s_kissued[st] & 1));
-    for (int st = 0; st < kVST; ++st)
-      if (s_vissued[st] >= 0) mbar_wait_plain(v_full + 8 * st, (uint32_t)(s_vissued[st] & 1));
-  }
-  if (aborted) {
-    // MMAs still in flight: each issuing warp's elected lane commits and waits
-    if ((warp == kWarpPv || warp == kWarpQk) && elect_one()) {
-      const uint32_t dr = drain + (warp == kWarpQk ? 8 : 0);
-      tc_commit(dr);
-      mbar_wait_plain(dr, 0);
-    }
-    __syncthreads();
-  }
-  if (warp == kWarpPv) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(kTmemCols)
-                 : "memory");
   }
 
+    // ---- producers and MMA issuers: drain on abort, free TMEM ----------------------
+    tc_fence_before();
+    __syncthreads();
+    pdl_allow_next();   // this grid's pipeline is done: the next kernel may take SMs as they free
+    if (s_abort) {
+      if (threadIdx.x == 0) {
+        flag_error(p.err, EE_DEVERR_TIMEOUT);
+        // TMA copies still in flight land before the rings are reused
+        for (int st = 0; st < kKST; ++st)
+          if (s_kissued[st] >= 0) mbar_wait_plain(k_full + 8 * st, (uint32_t)(s_kissued[st] & 1));
+        for (int st = 0; st < kVST; ++st)
+          if (s_vissued[st] >= 0) mbar_wait_plain(v_full + 8 * st, (uint32_t)(s_vissued[st] & 1));
+      }
+      // MMAs still in flight: each issuing warp's elected lane commits and waits
+      if ((warp == kWarpPv || warp == kWarpQk) && elect_one()) {
+        const uint32_t dr = drain + (warp == kWarpQk ? 8 : 0);
+        tc_commit(dr);
+        mbar_wait_plain(dr, 0);
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * kWarpSoft0) : "memory");
+    }
+    if (warp == kWarpPv) {
+      tc_fence_after();
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(kTmemCols)
+                   : "memory");
+    }
+    if (!kBal && s_uni.y > 0 && p.S > 1 && !p.coop) cluster_sync();   // with the softmax warps' below
+    return;
+  }
+if constexpr (!kBal) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoft));
+  // ---------------- softmax: one query row and half of every tile per thread ----------------
+  // Warps w and w + 4 share TMEM lane quarter w & 3 (32 query rows); half hf
+  // of the pair takes keys [64 hf, 64 hf + 64) of every tile and O columns
+  // [64 hf, 64 hf + 64).  The pair agrees on each tile's row maximum through
+  // shared memory at a 64-thread named barrier, so both halves take the same
+  // rescale decisions; each keeps the sum over its own keys, and the two sums
+  // are added (half 0 first) at the end.  Two warps per sub-partition hide
+  // each other's latencies.  Every exit from the tile loop happens right
+  // after the pair barrier and on a decision both warps share.
+  const int qd = warp & 3;
+  const int hf = (warp - kWarpSoft0) >> 2;
+  const uint32_t pair_bar = 2 + qd;
+  const int r = qd * 32 + lane;                     // == TMEM lane of this quarter
+  const uint32_t tl = tmem + ((uint32_t)(qd * 32) << 16);
+  const float sl2 = p.scale_log2;
+  bool ok = true;
+  bool loaded = false;
+  for (bool more = first(false); more && ok; more = next()) {
+    const int R = sg.T * g;
+    const int rr = sg.rb * kRows + r;
+    const bool vrow = rr < R;
+    const int node = vrow ? row_node(p, rr) : 0;
+    if (!loaded) {   // the first row block's Q: each softmax warp copies 16 rows
+      load_q<2 * kSoftWarps, kRows / 2 / kSoftWarps>(p, sg, sQ, 2 * (warp - kWarpSoft0), lane);
+      if (lane == 0) mbar_arrive(q_ready);
+      loaded = true;
+    }
+    // this half's tree keys (separate tree tile), or the row's whole ancestor
+    // mask (in place: tree keys at any offset from a half's first key)
+    const uint64_t ancw = (!kChain && vrow) ? p.anc[2 * (size_t)(sg.o + node) + (kIP ? 0 : hf)] : 0ull;
+    const uint64_t anc_hi = (kKV == kKVInPlace && vrow) ? p.anc[2 * (size_t)(sg.o + node) + 1] : 0ull;
+    // m_used is kept in raw score units (scale > 0, so the max commutes with it)
+    float m_used = -INFINITY, l = 0.f;
+    // keys below full_end: every row sees all of them (when their pages are valid)
+    const int full_end = kIP ? min(sg.k_end, sg.ctx) : sg.k_end;
+    // step tg processes the segment's tile tg - tb + rot (mod n_tiles)
+    for (int t = 0; t < sg.n_tiles; ++t) {
+      const int tg = tb + t;
+      const int sb = tg % kSB;    // S buffer of this tile
+      const int xb = tg & 1;      // pair-exchange slot
+      const bool got = wait(s_full + 8 * sb, tg / kSB);
+      uint32_t sr[64];
+      float tmax = -INFINITY;
+      if (got) {
+        tc_fence_after();
+        tc_ld32_nowait(tl + sb * kKT + 64 * hf, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
+        tc_ld32_nowait(tl + sb * kKT + 64 * hf + 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
+        const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;
+        const unsigned pm = s_mask[tg % kMaskRing];     // bit j: 16-row block j has a valid page
+        const int p0 = sg.k_begin + i * kKT;            // the tile's first key
+        // a whole tile of context keys in valid pages needs no mask: every row
+        // sees all of it (rows past R hold zero queries and are never stored)
+        const bool whole = i < sg.n_ctx && pm == 0xFFu && p0 + kKT <= full_end;
+        tc_wait_ld32(*reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
+        tc_pin32(*reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
+        if (!whole) {
+          // visibility of this half's 64 keys as one 64-bit word
+          uint64_t kw;
+          const int h0 = p0 + 64 * hf;
+          if (i < sg.n_ctx) {
+            const int nv = min(max(sg.k_end - h0, 0), 64);
+            uint64_t pgw = 0ull;
+#pragma unroll
+            for (int pb = 0; pb < 4; ++pb)
+              pgw |= ((pm >> (4 * hf + pb)) & 1u) ? (0xFFFFull << (16 * pb)) : 0ull;
+            kw = pgw & (nv >= 64 ? ~0ull : ((1ull << nv) - 1ull));
+            if constexpr (kChain) {
+              // causal: node sees positions up to ctx + node
+              const int nvis = min(max(sg.ctx + node + 1 - h0, 0), 64);
+              kw &= nvis >= 64 ? ~0ull : ((1ull << nvis) - 1ull);
+            } else if constexpr (kIP) {
+              // keys below ctx are context; key p >= ctx is tree node p - ctx
+              const int nc = min(max(sg.ctx - h0, 0), 64);
+              const int sh = h0 - sg.ctx;    // ancestor bit of this half's first key
+              uint64_t tm;
+              if (sh >= 0)
+                tm = sh >= 128 ? 0ull
+                     : sh >= 64 ? (anc_hi >> (sh - 64))
+                     : sh == 0  ? ancw
+                                : ((ancw >> sh) | (anc_hi << (64 - sh)));
+              else
+                tm = sh <= -64 ? 0ull : (ancw << (-sh));
+              kw &= (nc >= 64 ? ~0ull : ((1ull << nc) - 1ull)) | tm;
+            }
+          } else {
+            const int th = min(max(sg.T - 64 * hf, 0), 64);
+            kw = ancw & (th >= 64 ? ~0ull : ((1ull << th) - 1ull));
+          }
+          if (!vrow) kw = 0ull;
+#pragma unroll
+          for (int c = 0; c < 64; ++c)
+            if (!((kw >> c) & 1ull)) sr[c] = __float_as_uint(-INFINITY);
+        }
+        // 8 independent chains of three-input maxima over the 64 values
+        float mx[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) mx[c] = __uint_as_float(sr[c]);
+#pragma unroll
+        for (int c = 8; c < 56; c += 16)         // values 8 .. 55, two per instruction
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            mx[k] = fmax3(mx[k], __uint_as_float(sr[c + k]), __uint_as_float(sr[c + 8 + k]));
+#pragma unroll
+        for (int k = 0; k < 8; ++k) mx[k] = fmaxf(mx[k], __uint_as_float(sr[56 + k]));   // values 56 .. 63
+        tmax = fmax3(fmax3(mx[0], mx[1], mx[2]), fmax3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7]));
+      }
+      // the pair swaps its halves' maxima; both S halves are in registers before
+      // either warp overwrites S with P.  kFail (a NaN no maximum yields: theirs is
+      // 0x7fffffff) says that this half's wait failed
+      constexpr uint32_t kFail = 0xffffffffu;
+      s_xmax[xb][hf][r] = got ? __float_as_uint(tmax) : kFail;
+      tc_fence_before();
+      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
+      tc_fence_after();
+      const uint32_t other = s_xmax[xb][hf ^ 1][r];
+      if (!__all_sync(0xffffffffu, got && other != kFail)) {
+        ok = false;
+        break;
+      }
+      tmax = fmaxf(tmax, __uint_as_float(other));
+      const float m_new = fmaxf(m_used, tmax);
+      const bool need = (m_new - m_used) * sl2 > kRescaleLog2;   // true when m_used = -inf < m_new
+      if (t > 0 && __any_sync(0xffffffffu, need)) {
+        // O must hold P.V(tg-1) before this half's columns are rescaled; a failed
+        // wait sets the abort flag, and the pair stops at the next barrier
+        if (wait(pv_done + 8 * ((tg - 1) % kSB), (tg - 1) / kSB)) {
+          tc_fence_after();
+          const float f = need ? ex2((m_used - m_new) * sl2) : 1.f;
+#pragma unroll 1
+          for (int c4 = 0; c4 < 4; ++c4) {
+            uint32_t ov[16];
+            tc_ld16(tl + kColO + 64 * hf + 16 * c4, ov);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * f);
+            tc_st16_nowait(tl + kColO + 64 * hf + 16 * c4, ov);
+          }
+          tc_wait_st();
+        } else {
+          ok = false;
+        }
+      }
+      if (need) {
+        l *= ex2((m_used - m_new) * sl2);
+        m_used = m_new;
+      }
+      const float nms = m_used == -INFINITY ? 0.f : -m_used * sl2;
+      // p = 2^(s*scale_log2 - m); P = head + tail, both bf16: this
+      // half's head pairs go to columns 32 hf.. of the S buffer, its tail pairs
+      // to 64 + 32 hf..
+      // (pairs of columns run on packed fp32x2 arithmetic: the scale-and-shift,
+      // the running sums and the tail subtraction take one instruction per pair)
+      const uint64_t sl2x2 = f2_pack(__float_as_uint(sl2), __float_as_uint(sl2));
+      const uint64_t nmsx2 = f2_pack(__float_as_uint(nms), __float_as_uint(nms));
+      uint64_t ls2[4];
+      // two halves of 16 column pairs: each half's head and tail words go
+      // out before the next half is computed (fewer live registers)
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh) {
+        uint32_t hw[16], tw[16];
+#pragma unroll
+        for (int e2 = 0; e2 < 16; ++e2) {
+          const int e = 16 * hh + e2;
+          uint32_t y0, y1;
+          f2_unpack(f2_fma(f2_pack(sr[2 * e], sr[2 * e + 1]), sl2x2, nmsx2), y0, y1);
+          const uint32_t p0 = __float_as_uint(ex2(__uint_as_float(y0)));
+          const uint32_t p1 = __float_as_uint(ex2(__uint_as_float(y1)));
+          const uint64_t pp = f2_pack(p0, p1);
+          ls2[e & 3] = e < 4 ? pp : f2_add(ls2[e & 3], pp);
+          // head = p rounded to bf16; tail = the remainder p - head (exact
+          // in fp32) rounded to bf16
+          const uint32_t hb = bf16x2_rn(__uint_as_float(p1), __uint_as_float(p0));
+          float t0, t1;
+          sub_bf16x2(hb, __uint_as_float(p0), __uint_as_float(p1), t0, t1);
+          hw[e2] = hb;
+          tw[e2] = bf16x2_rn(t1, t0);
+        }
+        tc_st16_nowait(tl + sb * kKT + 32 * hf + 16 * hh, hw);
+        tc_st16_nowait(tl + sb * kKT + 64 + 32 * hf + 16 * hh, tw);
+      }
+      tc_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_full + 8 * sb);
+      {
+        uint32_t a0, a1, b0, b1, c0, c1, d0, d1;
+        f2_unpack(ls2[0], a0, a1);
+        f2_unpack(ls2[1], b0, b1);
+        f2_unpack(ls2[2], c0, c1);
+        f2_unpack(ls2[3], d0, d1);
+        l += ((__uint_as_float(a0) + __uint_as_float(a1)) + (__uint_as_float(b0) + __uint_as_float(b1))) +
+             ((__uint_as_float(c0) + __uint_as_float(c1)) + (__uint_as_float(d0) + __uint_as_float(d1)));
+      }
+    }
+    // wait for the last P.V (products complete in order, and this barrier's
+    // previous phase, P.V three tiles before, was over before the last S
+    // existed); the pair adds its two sums, then each half writes its 64
+    // columns out: O / l itself when the segment is a whole row block, else the
+    // partial (O, m, l) to the segment's slot
+    const int tl_g = tb + sg.n_tiles - 1;
+    const bool have = ok && sg.n_tiles > 0 && wait(pv_done + 8 * (tl_g % kSB), tl_g / kSB);
+    s_xl[hf][r] = l;
+    if (lane == 0) s_xok[nseg & 1][qd][hf] = have;
+    asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
+    const float l_sum = s_xl[0][r] + s_xl[1][r];
+    const bool both = s_xok[nseg & 1][qd][0] && s_xok[nseg & 1][qd][1];
+    const bool nan_row = both && vrow && l_sum != l_sum;   // NaN scores: the output is NaN
+    const float row_m =
+        nan_row ? 0.f : ((both && vrow && m_used != -INFINITY) ? m_used * sl2 : -INFINITY);
+    const float row_l = (both && vrow && (m_used != -INFINITY || nan_row)) ? l_sum : 0.f;
+    float4* dst;
+    size_t dstride;                                   // float4 between column chunks
+    float inv = 1.f;
+    if (sg.alone) {
+      const size_t orow = (size_t)(sg.o + node) * p.n_q + sg.hk * g + (rr - node * g);
+      dst = reinterpret_cast<float4*>(p.out + orow * kD);
+      dstride = 1;
+      inv = row_l == 0.f ? 0.f : 1.f / row_l;
+    } else {
+      dst = reinterpret_cast<float4*>(p.part + (size_t)sg.slot * kAttnPartBytes) + r;
+      dstride = kRows;
+    }
+    const bool store = sg.alone ? vrow : (row_l > 0.f || nan_row);
+    if (sg.n_tiles > 0) {
+      tc_fence_after();
+      uint32_t ov[64];
+      tc_ld32_nowait(tl + kColO + 64 * hf, *reinterpret_cast<uint32_t(*)[32]>(&ov[0]));
+      tc_ld32_nowait(tl + kColO + 64 * hf + 32, *reinterpret_cast<uint32_t(*)[32]>(&ov[32]));
+      tc_wait_ld32(*reinterpret_cast<uint32_t(*)[32]>(&ov[0]));
+      tc_pin32(*reinterpret_cast<uint32_t(*)[32]>(&ov[32]));
+      tc_fence_before();   // O is in registers: the next segment's P.V may overwrite it
+      __syncwarp();
+      if (lane == 0) mbar_arrive(o_free);
+      if (store) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e)
+          __stcg(dst + (size_t)(16 * hf + e) * dstride,
+                 make_float4(__uint_as_float(ov[4 * e]) * inv, __uint_as_float(ov[4 * e + 1]) * inv,
+                             __uint_as_float(ov[4 * e + 2]) * inv, __uint_as_float(ov[4 * e + 3]) * inv));
+      }
+    }
+    if (!sg.alone) {
+      if (hf == 0)
+        __stcg(reinterpret_cast<float2*>(p.part + (size_t)sg.slot * kAttnPartBytes + kAttnMlOff) + r,
+               make_float2(row_m, row_l));
+    }
+    if (!both) ok = false;
+  }
+
+  // ---- merge of split row blocks: the softmax warps' (they hold the registers) ------
+  tc_fence_before();
+  __syncthreads();
+  pdl_allow_next();
+  const int tid = threadIdx.x - 32 * kWarpSoft0;
   __shared__ int s_ready[2];
   if constexpr (kBal) {
     // ---- merge of split row blocks (balanced mode) ----------------------------------
-    // every CTA counts all its pieces before it waits for any (the launch is
-    // cooperative, so all CTAs are resident and every count arrives)
-    const int npieces = s_npc;     // written by thread 0 before the teardown barrier
+    // a CTA's pieces are counted and waited for independently, each by a thread of
+    // its own (the launch is cooperative: all CTAs are resident and every count arrives)
+    const int npieces = s_npc;     // written before the teardown barrier
     if (npieces == 0) return;
-    unsigned long long* cnt[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-      cnt[i] = reinterpret_cast<unsigned long long*>(
-          p.part + (size_t)s_pc[i < npieces ? i : 0].slot0 * kAttnPartBytes + kAttnCntOff);
-    if (threadIdx.x == 0) {
+    // two pieces: each group of four warps takes one
+    const int nthr = npieces == 2 ? kSoftThreads / 2 : kSoftThreads;
+    const int i = tid / nthr;
+    const int t = tid - i * nthr;
+    const BalPiece q = s_pc[i];
+    if (t == 0) {
       // the partials of this CTA's pieces (every thread's stores precede the
       // teardown barrier) are released with the count
-      for (int i = 0; i < npieces; ++i) red_add_release64(cnt[i], kCountGen / (unsigned)s_pc[i].K);
-      for (int i = 0; i < npieces; ++i) {
-        const bool ready = wait_count64_geq(cnt[i], s_pc[i].target);
-        if (!ready) flag_error(p.err, EE_DEVERR_TIMEOUT);
-        s_ready[i] = ready;
-      }
+      unsigned long long* cnt =
+          reinterpret_cast<unsigned long long*>(p.part + (size_t)q.slot0 * kAttnPartBytes + kAttnCntOff);
+      red_add_release64(cnt, kCountGen / (unsigned)q.K);
+      const bool ready = wait_count64_geq(cnt, q.target);
+      if (!ready) flag_error(p.err, EE_DEVERR_TIMEOUT);
+      s_ready[i] = ready;
     }
-    __syncthreads();
-    for (int i = 0; i < npieces; ++i) {
-      const BalPiece q = s_pc[i];
-      const int rpc = (kRows + q.K - 1) / q.K;
-      const int r0 = q.k * rpc;
-      const int nown = s_ready[i] ? max(0, min(rpc, min(kRows, q.R - q.rb * kRows) - r0)) : 0;
-      if (nown > 0) {
-        const int row0 = q.rb * kRows + r0;
-        switch (q.K) {
-#define EE_MERGE_CASE(n)                                                                   \
-  case n:                                                                                  \
-    merge_rows<n>(p, (size_t)q.slot0, (size_t)q.slot1, 2, row0, r0, nown, q.o, q.hk); \
-    break;
-          EE_MERGE_CASE(2) EE_MERGE_CASE(3) EE_MERGE_CASE(4) EE_MERGE_CASE(5) EE_MERGE_CASE(6)
-          EE_MERGE_CASE(7) EE_MERGE_CASE(8) EE_MERGE_CASE(9) EE_MERGE_CASE(10) EE_MERGE_CASE(11)
-          EE_MERGE_CASE(12) EE_MERGE_CASE(13) EE_MERGE_CASE(14) EE_MERGE_CASE(15) EE_MERGE_CASE(16)
-#undef EE_MERGE_CASE
-          default:
-            break;
-        }
-      }
-    }
-    return;
+    asm volatile("bar.sync %0, %1;" ::"r"(2 + i), "r"(nthr) : "memory");
+    const int rpc = (kRows + q.K - 1) / q.K;
+    const int r0 = q.k * rpc;
+    const int nown = s_ready[i] ? max(0, min(rpc, min(kRows, q.R - q.rb * kRows) - r0)) : 0;
+    if (nown > 0)
+      merge_pieces<1>(p, (size_t)q.slot0, (size_t)q.slot1, 2, q.K, q.rb * kRows + r0, r0, nown, q.o, q.hk, t, nthr);
   } else {
     if (s_uni.y == 0 || p.S == 1) return;   // (y == 0: the row block has no work)
-    const int split = (int)(blockIdx.x % p.S);   // == cluster rank in the cluster mode
-
     // ---- merge (uniform modes) -------------------------------------------------------
     // once every slot of the row block is complete and visible, chunk `split`
     // merges rows [r0, r0 + nown) of the row block
+    const int split = (int)(blockIdx.x % p.S);   // == cluster rank in the cluster mode
     const int R = s_uni.y, o = s_uni.x;
     const int rb = blockIdx.x / p.S;
     const size_t cta0 = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + (size_t)rb * p.S;
-    unsigned long long* cnt = reinterpret_cast<unsigned long long*>(p.part + cta0 * kAttnPartBytes + kAttnCntOff);
     if (p.coop) {
-      if (threadIdx.x == 0) {
+      if (tid == 0) {
         // this CTA's partial (every thread's stores precede the teardown barrier)
+        unsigned long long* cnt = reinterpret_cast<unsigned long long*>(p.part + cta0 * kAttnPartBytes + kAttnCntOff);
         red_add_release64(cnt, kCountGen / (unsigned)p.S);
         const bool ready = wait_count64_geq(cnt, s_pc[0].target);
         if (!ready) flag_error(p.err, EE_DEVERR_TIMEOUT);
         s_ready[0] = ready;
       }
-      __syncthreads();
     } else {
       cluster_sync();
-      if (threadIdx.x == 0) s_ready[0] = 1;
-      __syncthreads();
+      if (tid == 0) s_ready[0] = 1;
     }
+    asm volatile("bar.sync 2, %0;" ::"n"(kSoftThreads) : "memory");
     const int rpc = (kRows + p.S - 1) / p.S;
     const int r0 = split * rpc;
     const int nown = s_ready[0] ? max(0, min(rpc, min(kRows, R - rb * kRows) - r0)) : 0;
-    if (nown > 0) {
-      const int row0 = rb * kRows + r0;
-      switch (p.S) {
-#define EE_MERGE_CASE(n)                                                                  \
-  case n:                                                                                 \
-    merge_rows<n>(p, cta0, cta0 + 1, 1, row0, r0, nown, o, (int)blockIdx.y); \
-    break;
-        EE_MERGE_CASE(2) EE_MERGE_CASE(3) EE_MERGE_CASE(4) EE_MERGE_CASE(5) EE_MERGE_CASE(6)
-        EE_MERGE_CASE(7) EE_MERGE_CASE(8) EE_MERGE_CASE(9) EE_MERGE_CASE(10) EE_MERGE_CASE(11)
-        EE_MERGE_CASE(12) EE_MERGE_CASE(13) EE_MERGE_CASE(14) EE_MERGE_CASE(15) EE_MERGE_CASE(16)
-#undef EE_MERGE_CASE
-        default:
-          break;
-      }
-    }
+    if (nown > 0)
+      merge_pieces<2>(p, cta0, cta0 + 1, 1, p.S, rb * kRows + r0, r0, nown, o, (int)blockIdx.y, tid, kSoftThreads);
   }
 }
 
