@@ -151,45 +151,49 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return r;
 }
 
-// Merge rows [r0, r0 + nown) of a row block (query rows row0, ...) from its K
-// partial slots with log-sum-exp weights (Sec. III-A: the scores of one row
-// are normalised over all keys it sees) and write the fp32 output.  The softmax
-// threads do it (nthr of them): thread t takes row t % nown and the 16-byte
-// column chunks t / nown + k * tpr, where tpr = nthr / nown threads share a row:
-// the loads of a warp for one chunk are contiguous, and up to kOut chunks' loads
-// from all slots (K <= kMax) are issued before the first is used.  Rows without keys have
-// (m, l) = (-inf, 0) and weight 0; their O words, never written, are not used.
+// Merge the 16-byte column chunks [c_lo, c_hi) of a row block's rows (query rows
+// row0, ..., `rows` of them) from its K partial slots with log-sum-exp weights
+// (Sec. III-A: the scores of one row are normalised over all keys it sees) and
+// write the fp32 output.  A piece takes 32 / K chunks of every row, not 128 / K
+// rows of every chunk: a block with few rows (a root alone has g of them) then
+// keeps all its pieces busy.  The softmax threads do it (nthr of them): thread t
+// takes row t % rows and the chunks c_lo + t / rows + k * tpr, where tpr = nthr /
+// rows threads share a row: the loads of a warp for one chunk are contiguous, and
+// up to kOut chunks' loads from all slots (K <= kMax) are issued before the first
+// is used.  Rows without keys have (m, l) = (-inf, 0) and weight 0; their O
+// words, never written, are not used.
 template <int kMax, int kOut>
 __device__ __forceinline__ void merge_rows(const AttnParams& p, size_t slot_a, size_t slot_b, int stride, int K,
-                                           int row0, int r0, int nown, int o, int hk, int tid, int nthr) {
+                                           int row0, int rows, int c_lo, int c_hi, int o, int hk, int tid,
+                                           int nthr) {
   // partial s lives in slot slot_a (s = 0) or slot_b + (s - 1) * stride
   auto slot = [&](int s) -> const uint8_t* {
     return p.part + (s == 0 ? slot_a : slot_b + (size_t)(s - 1) * stride) * kAttnPartBytes;
   };
-  const int tpr = nthr / nown;
-  const int cg = tid / nown, j = tid - cg * nown;
+  const int tpr = nthr / rows;                   // >= 1: rows <= 128 <= nthr
+  const int cg = tid / rows, j = tid - cg * rows;
   if (cg >= tpr) return;
   float2 ml[kMax];
 #pragma unroll
   for (int s = 0; s < kMax; ++s)
-    ml[s] = s < K ? __ldcg(reinterpret_cast<const float2*>(slot(s) + kAttnMlOff) + r0 + j)
+    ml[s] = s < K ? __ldcg(reinterpret_cast<const float2*>(slot(s) + kAttnMlOff) + j)
                   : make_float2(-INFINITY, 0.f);
   const int rrow = row0 + j;
   const int nd = rrow / p.g;
   float4* dst = reinterpret_cast<float4*>(p.out + ((size_t)(o + nd) * p.n_q + hk * p.g + (rrow - nd * p.g)) * kD);
   float M = -INFINITY, il = 0.f, w[kMax];
-  for (int c0 = cg; c0 < kD / 4; c0 += kOut * tpr) {
+  for (int c0 = c_lo + cg; c0 < c_hi; c0 += kOut * tpr) {
     float4 v[kOut][kMax];
 #pragma unroll
     for (int k = 0; k < kOut; ++k) {
       const int c = c0 + k * tpr;
 #pragma unroll
       for (int s = 0; s < kMax; ++s)
-        v[k][s] = (c < kD / 4 && s < K)
-                      ? __ldcg(reinterpret_cast<const float4*>(slot(s)) + (size_t)c * kRows + r0 + j)
+        v[k][s] = (c < c_hi && s < K)
+                      ? __ldcg(reinterpret_cast<const float4*>(slot(s)) + (size_t)c * kRows + j)
                       : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    if (c0 == cg) {   // the weights, while the first chunks are in flight
+    if (c0 == c_lo + cg) {   // the weights, while the first chunks are in flight
 #pragma unroll
       for (int s = 0; s < kMax; ++s) M = fmaxf(M, ml[s].x);
       float L = 0.f;
@@ -203,7 +207,7 @@ __device__ __forceinline__ void merge_rows(const AttnParams& p, size_t slot_a, s
 #pragma unroll
     for (int k = 0; k < kOut; ++k) {
       const int c = c0 + k * tpr;
-      if (c >= kD / 4) break;
+      if (c >= c_hi) break;
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int s = 0; s < kMax; ++s) {
@@ -219,12 +223,13 @@ __device__ __forceinline__ void merge_rows(const AttnParams& p, size_t slot_a, s
 }
 // kX: 16 kX loads per thread in flight
 template <int kX>
-__device__ __forceinline__ void merge_pieces(const AttnParams& p, size_t slot_a, size_t slot_b, int stride, int K,
-                                             int row0, int r0, int nown, int o, int hk, int tid, int nthr) {
-  if (K <= 2) merge_rows<2, 8 * kX>(p, slot_a, slot_b, stride, K, row0, r0, nown, o, hk, tid, nthr);
-  else if (K <= 4) merge_rows<4, 4 * kX>(p, slot_a, slot_b, stride, K, row0, r0, nown, o, hk, tid, nthr);
-  else if (K <= 8) merge_rows<8, 2 * kX>(p, slot_a, slot_b, stride, K, row0, r0, nown, o, hk, tid, nthr);
-  else merge_rows<16, kX>(p, slot_a, slot_b, stride, K, row0, r0, nown, o, hk, tid, nthr);
+__device__ __forceinline__ void merge_pieces(const AttnParams& p, size_t slot_a, size_t slot_b, int stride, int K, int k,
+                                             int row0, int rows, int o, int hk, int tid, int nthr) {
+  const int c_lo = kD / 4 * k / K, c_hi = kD / 4 * (k + 1) / K;   // piece k's chunks
+  if (K <= 2) merge_rows<2, 8 * kX>(p, slot_a, slot_b, stride, K, row0, rows, c_lo, c_hi, o, hk, tid, nthr);
+  else if (K <= 4) merge_rows<4, 4 * kX>(p, slot_a, slot_b, stride, K, row0, rows, c_lo, c_hi, o, hk, tid, nthr);
+  else if (K <= 8) merge_rows<8, 2 * kX>(p, slot_a, slot_b, stride, K, row0, rows, c_lo, c_hi, o, hk, tid, nthr);
+  else merge_rows<16, kX>(p, slot_a, slot_b, stride, K, row0, rows, c_lo, c_hi, o, hk, tid, nthr);
 }
 
 // A row block's partial that this CTA merges with the other pieces of the same
@@ -1234,16 +1239,14 @@ if constexpr (!kBal) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kR
       s_ready[i] = ready;
     }
     asm volatile("bar.sync %0, %1;" ::"r"(2 + i), "r"(nthr) : "memory");
-    const int rpc = (kRows + q.K - 1) / q.K;
-    const int r0 = q.k * rpc;
-    const int nown = s_ready[i] ? max(0, min(rpc, min(kRows, q.R - q.rb * kRows) - r0)) : 0;
-    if (nown > 0)
-      merge_pieces<1>(p, (size_t)q.slot0, (size_t)q.slot1, 2, q.K, q.rb * kRows + r0, r0, nown, q.o, q.hk, t, nthr);
+    if (s_ready[i])
+      merge_pieces<1>(p, (size_t)q.slot0, (size_t)q.slot1, 2, q.K, q.k, q.rb * kRows, min(kRows, q.R - q.rb * kRows),
+                      q.o, q.hk, t, nthr);
   } else {
     if (s_uni.y == 0 || p.S == 1) return;   // (y == 0: the row block has no work)
     // ---- merge (uniform modes) -------------------------------------------------------
     // once every slot of the row block is complete and visible, chunk `split`
-    // merges rows [r0, r0 + nown) of the row block
+    // merges its share of the columns
     const int split = (int)(blockIdx.x % p.S);   // == cluster rank in the cluster mode
     const int R = s_uni.y, o = s_uni.x;
     const int rb = blockIdx.x / p.S;
@@ -1262,11 +1265,9 @@ if constexpr (!kBal) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kR
       if (tid == 0) s_ready[0] = 1;
     }
     asm volatile("bar.sync 2, %0;" ::"n"(kSoftThreads) : "memory");
-    const int rpc = (kRows + p.S - 1) / p.S;
-    const int r0 = split * rpc;
-    const int nown = s_ready[0] ? max(0, min(rpc, min(kRows, R - rb * kRows) - r0)) : 0;
-    if (nown > 0)
-      merge_pieces<2>(p, cta0, cta0 + 1, 1, p.S, rb * kRows + r0, r0, nown, o, (int)blockIdx.y, tid, kSoftThreads);
+    if (s_ready[0])
+      merge_pieces<2>(p, cta0, cta0 + 1, 1, p.S, split, rb * kRows, min(kRows, R - rb * kRows), o, (int)blockIdx.y, tid,
+                      kSoftThreads);
   }
 }
 
