@@ -301,7 +301,8 @@ __device__ void accept_sequences(const AcceptArgs& a, const int32_t* am, const i
 }
 
 
-template <bool kVerify>
+// kPair: the CTAs of a cluster of two share every MMA (see the pair rule at the launch).
+template <bool kVerify, bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
 lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                      const LmParams p) {
@@ -311,7 +312,11 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
   ee::pdl_allow_next();
   ee::pdl_wait();   // no global access before the previous kernel's writes are visible
   const int S = p.stages, BN = p.BN;
-  const uint32_t bBytes = (uint32_t)BN * BK * 2;
+  const uint32_t bBytes = (uint32_t)(kPair ? BN / 2 : BN) * BK * 2;   // node rows a CTA's stage receives
+  // pair: this CTA's rank; work is counted in pairs of vocabulary tiles
+  const int rank = kPair ? (int)(blockIdx.x & 1) : 0;
+  const int first_tile = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+  const int tile_step = kPair ? (int)(gridDim.x >> 1) : (int)gridDim.x;
   const uint32_t aBytes = (uint32_t)p.BMr * BK * 2;   // W rows a stage receives
   uint8_t* sA = smem;
   uint8_t* sB = smem + (size_t)S * kABytes;
@@ -346,7 +351,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull0 + 8 * a, 1);
-      mbar_init(tempty0 + 8 * a, kEpiWarps);
+      mbar_init(tempty0 + 8 * a, kPair ? 2 * kEpiWarps : kEpiWarps);
     }
     mbar_init(drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -356,7 +361,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
     // stream starts while the other warps allocate TMEM and clear their state
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmW)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmX)) : "memory");
-    if ((int)blockIdx.x < p.n_vt * p.n_nt) {
+    if (!kPair && (int)blockIdx.x < p.n_vt * p.n_nt) {   // (a pair's barriers must exist in both CTAs first)
       const int vt = (int)blockIdx.x / p.n_nt, nt = (int)blockIdx.x % p.n_nt;
       const int pre = min(S, p.nkb);
       for (int kb = 0; kb < pre; ++kb) {
@@ -372,11 +377,19 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
     }
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32(s_tmem)),
-                 "r"(p.tmem_cols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (kPair) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                       smem_u32(s_tmem)),
+                   "r"(p.tmem_cols)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                       smem_u32(s_tmem)),
+                   "r"(p.tmem_cols)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   for (int i = threadIdx.x; i < 4 * BN; i += kThreads) s_best[i] = BestPair{-INFINITY, 0x7fffffff};
   if (kVerify) {
@@ -392,10 +405,11 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (kPair) cluster_sync();   // both CTAs' barriers exist
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
 
-  const int num_tiles = p.n_vt * p.n_nt;
+  const int num_tiles = (kPair ? (p.n_vt + 1) / 2 : p.n_vt) * p.n_nt;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -404,12 +418,27 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
       int stage = pre % S;
       uint32_t phase = pre == S ? 1u : 0u;
       bool ok = true;
-      for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
-        const int vt = t / p.n_nt, nt = t % p.n_nt;
-        for (int kb = (t == (int)blockIdx.x ? pre : 0); kb < p.nkb; ++kb) {
+      for (int t = first_tile; t < num_tiles && ok; t += tile_step) {
+        const int vt = kPair ? 2 * (t / p.n_nt) + rank : t / p.n_nt, nt = t % p.n_nt;
+        for (int kb = (t == first_tile ? pre : 0); kb < p.nkb; ++kb) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, &s_abort)) {
             ok = false;
             break;
+          }
+          if constexpr (kPair) {
+            // both CTAs' loads signal rank 0's barrier, which expects them all
+            const uint32_t fb = map_cluster(full0 + 8 * stage, 0);
+            if (rank == 0) mbar_expect_tx(full0 + 8 * stage, 2 * (aBytes + bBytes));
+            const uint32_t da = smem_u32(sA + (size_t)stage * kABytes);
+            if (p.packed) tma2_load_2d(da, &tmW, fb, 0, (vt * p.nkb + kb) * BM);
+            else tma2_load_2d(da, &tmW, fb, kb * BK, vt * p.BMr);
+            tma2_load_2d(smem_u32(sB + (size_t)stage * bBytes), &tmX, fb, kb * BK, nt * BN + rank * (BN / 2));
+            ++s_issued;
+            if (++stage == S) {
+              stage = 0;
+              phase ^= 1;
+            }
+            continue;
           }
           const uint32_t fb = full0 + 8 * stage;
           mbar_expect_tx(fb, aBytes + bBytes);
@@ -426,10 +455,10 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
         }
       }
     }
-  } else if (warp == 1) {
+  } else if (warp == 1 && rank == 0) {
     // the whole warp walks the loop (wait outcomes made warp-uniform) and one
     // elected lane issues the MMAs, every descriptor an offset from a uniform base
-    const uint32_t idesc = idesc_bf16(BM, BN);
+    const uint32_t idesc = idesc_bf16(kPair ? 2 * BM : BM, BN);
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
     const uint64_t ad0 = smem_desc_sw128(__shfl_sync(0xffffffffu, smem_u32(sA), 0));
     const uint64_t bd0 = smem_desc_sw128(__shfl_sync(0xffffffffu, smem_u32(sB), 0));
@@ -437,7 +466,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
     uint32_t phase = 0;
     bool ok = true;
     int lt = 0, consumed = 0;
-    for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++lt) {
+    for (int t = first_tile; t < num_tiles && ok; t += tile_step, ++lt) {
       const int acc = lt & 1;
       const uint32_t acc_phase = (lt >> 1) & 1;
       if (!__all_sync(0xffffffffu, mbar_wait(tempty0 + 8 * acc, acc_phase ^ 1, &s_abort))) break;
@@ -453,10 +482,19 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
           const uint64_t ad = ad0 + (uint64_t)(stage * (kABytes >> 4));
           const uint64_t bd = bd0 + (uint64_t)(stage * (bBytes >> 4));
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k)
-            tc_mma(d_tmem, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kb | k) != 0 ? 1u : 0u);
-          tc_commit(empty0 + 8 * stage);
-          if (kb == p.nkb - 1) tc_commit(tfull0 + 8 * acc);
+          for (int k = 0; k < BK / 16; ++k) {
+            if constexpr (kPair)
+              tc2_mma(d_tmem, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kb | k) != 0 ? 1u : 0u);
+            else
+              tc_mma(d_tmem, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kb | k) != 0 ? 1u : 0u);
+          }
+          if constexpr (kPair) {
+            tc2_commit_both(empty0 + 8 * stage);
+            if (kb == p.nkb - 1) tc2_commit_both(tfull0 + 8 * acc);
+          } else {
+            tc_commit(empty0 + 8 * stage);
+            if (kb == p.nkb - 1) tc_commit(tfull0 + 8 * acc);
+          }
         }
         __syncwarp();
         ++consumed;
@@ -467,15 +505,15 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
       }
     }
     if (lane == 0) s_consumed = consumed;
-  } else {
-    // epilogue warps 2..5: TMEM lane quarter = warp % 4
+  } else if (warp >= 2) {
+    // epilogue warps 2..9: TMEM lane quarter = warp % 4
     const int q = warp & 3;                 // TMEM lane quarter
     const int ew = q;                       // per-quarter state index
     const int half = (warp - 2) >> 2;       // which 16-column chunks: c0 / 16 = half mod 2
     BestPair* mybest = s_best + ew * BN;
     int lt = 0;
-    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++lt) {
-      const int vt = t / p.n_nt, nt = t % p.n_nt;
+    for (int t = first_tile; t < num_tiles; t += tile_step, ++lt) {
+      const int vt = kPair ? 2 * (t / p.n_nt) + rank : t / p.n_nt, nt = t % p.n_nt;
       const int acc = lt & 1;
       const uint32_t acc_phase = (lt >> 1) & 1;
       // warp-uniform outcome: the tcgen05.ld below is warp-collective
@@ -625,7 +663,10 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(tempty0 + 8 * acc);
+      if (lane == 0) {
+        if constexpr (kPair) mbar_arrive_cluster(map_cluster(tempty0 + 8 * acc, 0));
+        else mbar_arrive(tempty0 + 8 * acc);
+      }
       if (kVerify) {
         // publish this CTA's K-th keys: no row below another CTA's K-th entry
         // can be among the K best of the whole vocabulary
@@ -640,8 +681,8 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
     }
     // publish this CTA's best per node (every tile of a CTA has the same node tile)
     asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
-    if (blockIdx.x < num_tiles) {
-      const int nt = blockIdx.x % p.n_nt;
+    if (first_tile < num_tiles) {
+      const int nt = first_tile % p.n_nt;
       for (int c = threadIdx.x - 64; c < BN; c += kEpiThreads) {
         BestPair b = s_best[c];
         for (int w = 1; w < 4; ++w) {
@@ -652,7 +693,9 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
         if (node < p.total_nodes && b.i != 0x7fffffff) atomicMax(&p.keys[node], make_key(b.v, b.i));
         if (kVerify) {
           // this CTA's partial for the node: the 4 warps' lists merged, their sums added
-          uint8_t* rec = p.part + ((size_t)blockIdx.x * BN + c) * lm_rec_bytes(K);
+          // source q of node tile nt is record q n_nt + nt (pair: q = 2 x pair + rank)
+          const int src = kPair ? (first_tile / p.n_nt * 2 + rank) * p.n_nt + nt : (int)blockIdx.x;
+          uint8_t* rec = p.part + ((size_t)src * BN + c) * lm_rec_bytes(K);
           float* pv = reinterpret_cast<float*>(rec);
           int* pi = reinterpret_cast<int*>(rec + 4 * K);
           float2* pl = reinterpret_cast<float2*>(rec + 8 * K);
@@ -697,20 +740,38 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
     if (threadIdx.x == 0) {
       ee::flag_error(p.err, EE_DEVERR_TIMEOUT);
       // TMA loads issued but never consumed still land in shared memory: wait for them
-      for (int k = s_consumed; k < s_issued; ++k)
+      for (int k = s_consumed; rank == 0 && k < s_issued; ++k)
         if (!mbar_wait_plain(full0 + 8 * (k % S), (uint32_t)((k / S) & 1))) break;
     }
   }
   if (warp == 1) {
-    if (aborted && elect_one()) {   // the lane that issued the MMAs
+    if (aborted && !kPair && elect_one()) {   // the lane that issued the MMAs
       tc_commit(drain);
       mbar_wait_plain(drain, 0);
     }
+    if (aborted && kPair && rank == 0 && elect_one()) {
+      tc2_commit_both(drain);
+      mbar_wait_plain(drain, 0);
+    }
     __syncwarp();
+  }
+  // the pair's products and loads are over in both CTAs before either frees its
+  // tensor memory or leaves (a wait limit of 1 s has passed on abort)
+  if constexpr (kPair) {
+    __syncwarp();
+    tc_fence_before();
+    cluster_sync();
+  }
+  if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
-                 "r"(p.tmem_cols)
-                 : "memory");
+    if constexpr (kPair)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                   "r"(p.tmem_cols)
+                   : "memory");
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                   "r"(p.tmem_cols)
+                   : "memory");
   }
   if (aborted) return;
 
@@ -1025,21 +1086,33 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
   p.B = B;
   p.max_T = max_T;
   p.n_nt = (total_nodes + 255) / 256;
-  p.BN = ((total_nodes + p.n_nt - 1) / p.n_nt + 15) / 16 * 16;
+  // Pair rule: with several node tiles (more than 256 nodes) the kernel is bound
+  // by the tensor pipe, but a CTA of its own loads 128 rows of W and BN rows of X
+  // per k-block, 48 KB at BN = 256, through an L2-to-SM port of 64 bytes a cycle:
+  // 768 cycles against 512 of MMA.  Two CTAs that share their MMAs (cta_group::2,
+  // M = 256) load 128 rows of W and BN / 2 rows of X each, 32 KB in the 512 cycles,
+  // and the ring holds six k-blocks instead of four.  With one node tile the weight
+  // stream from HBM is the bound (161 us for 64 nodes at 7B shapes) and the plain
+  // CTA reaches it.
+  const bool pair = p.n_nt > 1;
+  const int bn_step = pair ? 32 : 16;
+  p.BN = ((total_nodes + p.n_nt - 1) / p.n_nt + bn_step - 1) / bn_step * bn_step;
   // vocabulary tiles: as many per CTA for every CTA (the launch's end is the
   // busiest CTA's), each of ceil(V / tiles) <= 128 rows; the MMA's remaining
   // rows hold stale shared memory and are dropped by the epilogue.  Below 64
   // rows a tile would waste most of its MMA: plain 128-row tiles then.
   {
     const int n_vt0 = (vocab + BM - 1) / BM;
-    const int per_group = std::max(1, ee::kNumSMs / p.n_nt);   // CTAs per node tile
+    // CTAs per node tile
+    const int per_group = pair ? 2 * std::max(1, ee::kNumSMs / 2 / p.n_nt) : std::max(1, ee::kNumSMs / p.n_nt);
     const int k = (n_vt0 + per_group - 1) / per_group;
     const int rows = (vocab + k * per_group - 1) / (k * per_group);
     p.BMr = rows >= 64 && !packed ? rows : BM;
     p.n_vt = (vocab + p.BMr - 1) / p.BMr;
   }
   p.nkb = (hidden_dim + BK - 1) / BK;
-  const size_t stage_bytes = (size_t)kABytes + (size_t)p.BN * BK * 2;
+  const int bn_cta = pair ? p.BN / 2 : p.BN;   // node rows a CTA loads
+  const size_t stage_bytes = (size_t)kABytes + (size_t)bn_cta * BK * 2;
   const int K = va ? va->k : 1;
   // epilogue state: running best per warp and node (+ top-K lists and sums)
   const size_t epi = 4 * (size_t)p.BN * sizeof(BestPair) +
@@ -1080,7 +1153,7 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
   } else if (!encode_2d(&tmW, lm_w, (uint64_t)hidden_dim, (uint64_t)vocab, BK, (uint32_t)p.BMr)) {
     return EE_ERR_CUDA;
   }
-  if (!encode_2d(&tmX, hidden, (uint64_t)hidden_dim, (uint64_t)total_nodes, BK, p.BN))
+  if (!encode_2d(&tmX, hidden, (uint64_t)hidden_dim, (uint64_t)total_nodes, BK, (uint32_t)bn_cta))
     return EE_ERR_CUDA;
 
   const size_t smem = 1024 + (size_t)p.stages * stage_bytes + 8 * (2 * p.stages + 5) + 8 + epi;
@@ -1089,32 +1162,31 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
   const size_t last = 1024 + (size_t)(2 * EE_MAX_LM_NODES + 5) * 4;
   const size_t smem_acc = std::max(smem, last);
   if (smem_acc > 227 * 1024) return EE_ERR_UNSUPPORTED;
+  decltype(&lmhead_accept_kernel<false, false>) fn =
+      va ? (pair ? lmhead_accept_kernel<true, true> : lmhead_accept_kernel<true, false>)
+         : (pair ? lmhead_accept_kernel<false, true> : lmhead_accept_kernel<false, false>);
   {
     // the dynamic shared memory attribute, raised once per device and kernel
     int dev = 0;
     const ee_status ds = ee::current_device(&dev);
     if (ds != EE_OK) return ds;
     static std::mutex mu;
-    static size_t attr_bytes[ee::kMaxDevices][2] = {};
+    static size_t attr_bytes[ee::kMaxDevices][4] = {};
     std::lock_guard<std::mutex> lock(mu);
-    if (attr_bytes[dev][va ? 1 : 0] < smem_acc) {
-      if (va)
-        EE_CUDA_OK(cudaFuncSetAttribute(lmhead_accept_kernel<true>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_acc));
-      else
-        EE_CUDA_OK(cudaFuncSetAttribute(lmhead_accept_kernel<false>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_acc));
-      attr_bytes[dev][va ? 1 : 0] = smem_acc;
+    size_t& have = attr_bytes[dev][(va ? 1 : 0) + (pair ? 2 : 0)];
+    if (have < smem_acc) {
+      EE_CUDA_OK(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_acc));
+      have = smem_acc;
     }
   }
-  const int num_tiles = p.n_vt * p.n_nt;
-  int grid = (ee::kNumSMs / p.n_nt) * p.n_nt;   // multiple of n_nt: each CTA keeps one node tile
-  if (grid > num_tiles) grid = num_tiles;
-  if (grid < 1) grid = 1;
+  // a multiple of n_nt CTAs (or pairs): each keeps one node tile
+  const int num_tiles = (pair ? (p.n_vt + 1) / 2 : p.n_vt) * p.n_nt;
+  int grid = std::max(1, std::min((ee::kNumSMs / (pair ? 2 : 1) / p.n_nt) * p.n_nt, num_tiles));
+  if (pair) grid *= 2;
   if (va && (size_t)grid * p.BN * ee::lm_rec_bytes(K) > ee::kLmPartBytes) return EE_ERR_UNSUPPORTED;
   if (va) {
-    EE_CUDA_OK(ee::launch_pdl(lmhead_accept_kernel<true>, dim3(grid), dim3(kThreads), smem_acc,
-                              (cudaStream_t)stream, 1, tmW, tmX, p));
+    EE_CUDA_OK(ee::launch_pdl(fn, dim3(grid), dim3(kThreads), smem_acc, (cudaStream_t)stream, pair ? 2u : 1u, tmW,
+                              tmX, p));
     FinParams fp;
     fp.total = total_nodes;
     fp.B = B;
@@ -1150,11 +1222,22 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
     }
     EE_CUDA_OK(fe);
   } else if (pdl) {
-    EE_CUDA_OK(ee::launch_pdl(lmhead_accept_kernel<false>, dim3(grid), dim3(kThreads), smem_acc,
-                              (cudaStream_t)stream, 1, tmW, tmX, p));
+    EE_CUDA_OK(ee::launch_pdl(fn, dim3(grid), dim3(kThreads), smem_acc, (cudaStream_t)stream, pair ? 2u : 1u, tmW,
+                              tmX, p));
   } else {
-    lmhead_accept_kernel<false><<<grid, kThreads, smem_acc, (cudaStream_t)stream>>>(tmW, tmX, p);
-    EE_LAUNCH_OK();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem_acc;
+    cfg.stream = (cudaStream_t)stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pair ? 1 : 0;
+    EE_CUDA_OK(cudaLaunchKernelEx(&cfg, fn, tmW, tmX, p));
   }
   return EE_OK;
 }
