@@ -1,0 +1,142 @@
+"""GPU parity at the sizes where the attention's segments and merges and the LM
+head's CTA pairs and top-K lists can go wrong: CTAs that walk more segments than
+the published ring holds, row blocks of a few rows split over many CTAs, a row of
+NaN scores, node counts just above one node tile, odd numbers of vocabulary
+tiles, list quarters with fewer rows than k.  References and tolerances are those
+of the other parity tests (the fp64 oracle; parity_util)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+import parity_util as U
+import test_gpu_verify as V
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    import paper_2506_02780_gb300 as E
+    from paper_2506_02780_gb300 import build
+    build.build_lib()
+    E.lib()
+
+
+@pytest.mark.parametrize("kind", ["tree", "inplace", "chain"])
+@pytest.mark.parametrize("n_q,n_kv", [(8, 8), (24, 8)])
+def test_many_short_segments(kind, n_q, n_kv):
+    """400 sequences of 0 to 120 cached positions and 1 to 5 nodes: a balanced
+    launch whose CTAs each walk about 20 segments of one or two tiles (more than
+    the 16 the ring of published segments holds)."""
+    import paper_2506_02780_gb300 as E
+    from paper_2506_02780_gb300 import step as S
+    rng = np.random.default_rng(7)
+    B = 400
+    Ts = rng.integers(1, 6, B)
+    w = W.build("tiny", seed=71, device="cuda", vocab=512, hidden=64, n_q=n_q, n_kv=n_kv,
+                trees=[W.TreeSpec(int(t), [], [0]) for t in Ts], ctxs=[int(c) for c in rng.integers(0, 121, B)])
+    mode = {"tree": False, "inplace": True, "chain": "chain"}[kind]
+    plan = E.ee_attn_plan(w.B, w.max_T, n_q, n_kv, int(w.ctx_len.max()), inplace=mode)
+    assert plan["mode"] == "balanced"
+    kc, vc = (torch.from_numpy(U.raw16(t).copy()).view(torch.bfloat16) for t in (w.k_cache, w.v_cache))
+    st = S.from_workload(w, inplace_kv=kind == "inplace", chain=kind == "chain")
+    st.run()
+    torch.cuda.synchronize()
+    assert E.ee_read_errors(st.ws) == 0
+    anc = O.tree_prepare(w.parent, w.node_off)[1]
+    ref = O.tree_attention(w.q[0], w.k_tree[0], w.v_tree[0], kc[0], vc[0], w.block_table, w.ctx_len, w.node_off, anc)
+    U.assert_close(st.attn_out[0].cpu().numpy(), ref, f"{kind} attention")
+
+
+@pytest.mark.parametrize("T,ctx", [(1, 3001), (2, 129), (3, 1999), (19, 2500), (64, 4096)])
+def test_few_rows_split_over_many_ctas(T, ctx):
+    """One sequence, 28 / 4 heads: row blocks of 7 to 128 rows cut into up to 15
+    chunks, merged by column chunks."""
+    import paper_2506_02780_gb300 as E
+    from paper_2506_02780_gb300 import step as S
+    w = W.build("7b", seed=72, device="cuda", layers=1, vocab=512, hidden=64, trees=[W.TreeSpec(T, [], [0])], ctx=ctx)
+    kc, vc = (torch.from_numpy(U.raw16(t).copy()).view(torch.bfloat16) for t in (w.k_cache, w.v_cache))
+    st = S.from_workload(w)
+    st.run()
+    torch.cuda.synchronize()
+    assert E.ee_read_errors(st.ws) == 0
+    anc = O.tree_prepare(w.parent, w.node_off)[1]
+    ref = O.tree_attention(w.q[0], w.k_tree[0], w.v_tree[0], kc[0], vc[0], w.block_table, w.ctx_len, w.node_off, anc)
+    U.assert_close(st.attn_out[0].cpu().numpy(), ref, f"T = {T}, ctx = {ctx}")
+
+
+@pytest.mark.parametrize("ctxs", [[512], [700] * 40])
+def test_nan_scores_stay_in_their_row(ctxs):
+    """A query row of NaN (split and balanced launches): its output is NaN, every
+    other row is bit-identical to a run without it, and no wait gives up."""
+    import paper_2506_02780_gb300 as E
+    from paper_2506_02780_gb300 import step as S
+    w = W.build("tiny", seed=73, device="cuda", vocab=512, hidden=64,
+                trees=[W.TreeSpec(12, [(0, 4)], [0]) for _ in ctxs], ctxs=ctxs)
+    st = S.from_workload(w)
+    st.run()
+    torch.cuda.synchronize()
+    clean = st.attn_out[0].clone()
+    w.q[0, 3, 2] = float("nan")
+    st.run()
+    torch.cuda.synchronize()
+    assert E.ee_read_errors(st.ws) == 0
+    got = st.attn_out[0]
+    assert torch.isnan(got[3, 2]).all()
+    keep = torch.ones(got.shape[:2], dtype=torch.bool, device=got.device)
+    keep[3, 2] = False
+    assert torch.equal(got[keep], clean[keep])
+
+
+@pytest.mark.parametrize("nodes,vocab,hidden,packed", [(256, 4100, 512, True), (257, 4100, 520, False),
+                                                       (288, 4097, 512, True), (513, 4224, 512, True),
+                                                       (1025, 4100, 64, False)])
+def test_lmhead_around_one_node_tile(nodes, vocab, hidden, packed):
+    """256 nodes (one tile, a CTA of its own) and just above (CTA pairs), with odd
+    numbers of 128-row vocabulary tiles: argmax, longest prefix and logits."""
+    import paper_2506_02780_gb300 as E
+    w = W.build("long", seed=74, device="cuda", layers=1, vocab=vocab, hidden=hidden, n_q=8, n_kv=2,
+                trees=[W.TreeSpec(nodes, [], W.chain_path(nodes // 2))], ctxs=[16])
+    i32 = dict(dtype=torch.int32, device="cuda")
+    ws = E.new_workspace(1, nodes, 1, 0)
+    am, acc, bonus = (torch.empty(n, **i32) for n in (nodes, 1, 1))
+    path = torch.empty((1, nodes), **i32)
+    logits = torch.full((nodes, vocab), float("nan"), device="cuda")
+    node_off = torch.as_tensor(w.node_off, **i32)
+    draft = torch.as_tensor(w.draft_tok, **i32)
+    for _ in range(2):   # the running state returns to zero after a call
+        if packed:
+            wp = torch.empty(E.ee_lmhead_packed_bytes(vocab, hidden) // 2, dtype=torch.bfloat16, device="cuda")
+            E.ee_lmhead_pack_weights(w.lm_w, wp)
+            E.ee_lmhead_accept_packed(w.hidden_states, wp, vocab, draft, None, None, None, node_off, nodes, am, acc,
+                                      path, bonus, ws, logits=logits)
+        else:
+            E.ee_lmhead_accept(w.hidden_states, w.lm_w, draft, None, None, None, node_off, nodes, am, acc, path,
+                               bonus, ws, logits=logits)
+        torch.cuda.synchronize()
+        assert E.ee_read_errors(ws) == 0
+    U.check_argmax(w, type("S", (), {"argmax": am})(), logits=logits)
+    ra, rp, rb = O.accept_chain(am.cpu().numpy(), w.draft_tok, w.node_off, nodes)
+    np.testing.assert_array_equal(acc.cpu().numpy(), ra)
+    np.testing.assert_array_equal(path.cpu().numpy(), rp)
+    np.testing.assert_array_equal(bonus.cpu().numpy(), rb)
+
+
+@pytest.mark.parametrize("mode,k", [("entropy", 5), ("topk", 8)])
+def test_verify_above_one_node_tile(mode, k):
+    """15 trees of 20 nodes: the verification rules on CTA pairs."""
+    w = W.build("tiny", seed=75, device="cuda", verify_plant=True, trees=[V.TREE] * 15)
+    V._check(w, V._run(w, mode, k), mode, k)
+
+
+@pytest.mark.parametrize("vocab", [40, 130, 200])
+@pytest.mark.parametrize("k", [2, 8])
+def test_verify_lists_with_few_rows(vocab, k):
+    """Lists that a tile fills only in part (a quarter of 32 rows holds 0, 2 or 8
+    of them): top-k ids, entropy and acceptance."""
+    w = W.build("tiny", seed=76, device="cuda", vocab=vocab)
+    V._check(w, V._run(w, "entropy", k), "entropy", k)
