@@ -91,6 +91,7 @@ constexpr int kSB = 3;                           // S buffers in TMEM (Q.K^T run
 constexpr uint32_t kKVHalf = kKT * 128;          // 16 KB: one 64-dim half of a K or V tile
 constexpr uint32_t kKVBytes = 2 * kKVHalf;       // 32 KB
 constexpr int kMaxCtaPages = 2048;               // context pages one CTA owns at most (32768 keys)
+constexpr int kUnitCost = 3;                      // balanced: a unit's weight beyond its tiles (see the work list)
 constexpr int kSegRing = 16;                     // published segments (K runs at most 8 ahead of the softmax)
 constexpr int kMaskRing = 8;                     // page-validity masks in flight (K runs at most 6 tiles ahead)
 constexpr uint32_t kOffK = 0;
@@ -292,7 +293,7 @@ struct Seg {
   bool alone;                  // the segment is its whole row block
   int slot;                    // partial slot (alone: unused)
   int y;                       // balanced: where the segment starts in the work list
-  int U0, tiles;               // balanced: the unit's first tile in the work list and its tiles
+  int U0, tiles;               // balanced: the unit's start in the work list and its weight
 };
 
 // Shared state of a CTA's work: balanced mode, per sequence (node offset, T,
@@ -328,8 +329,8 @@ __device__ __forceinline__ void bal_segment(const AttnParams& p, const WorkList&
   s.o = sq.x;
   s.T = sq.y;
   s.ctx = sq.z;
-  int tiles = sq.w;
-  int U0;                                        // the unit's first tile in the work list
+  int tiles = sq.w;                              // the unit's weight
+  int U0;                                        // its start in the work list
   const int base_w = w.wpre[lo];
   const int nrb_b = (int)((unsigned)(s.T * g + kRows - 1) / kRows);
   if constexpr (kChain) {
@@ -345,7 +346,7 @@ __device__ __forceinline__ void bal_segment(const AttnParams& p, const WorkList&
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int rr = r0 + 4 * lane + q;
-        t[q] = rr < nrb_b ? chain_tiles(p, s.ctx, s.T, rr) : 0;
+        t[q] = rr < nrb_b ? chain_tiles(p, s.ctx, s.T, rr) + kUnitCost : 0;
         sum += t[q];
       }
       int incl = sum;
@@ -383,19 +384,21 @@ __device__ __forceinline__ void bal_segment(const AttnParams& p, const WorkList&
     U0 = base_w + u * tiles;
   }
   const int seg0 = max(U0, x_begin);
-  const int t0 = seg0 - U0;
-  const int len = y - seg0;
-  const int n_ctx_b = kIP ? tiles : tiles - 1;   // paged tiles of the unit
+  // the unit's first kUnitCost places are no tiles
+  const int t0 = max(seg0 - U0 - kUnitCost, 0);
+  const int len = max(y - U0 - kUnitCost, 0) - t0;
+  const int n_tiles_b = tiles - kUnitCost;
+  const int n_ctx_b = kIP ? n_tiles_b : n_tiles_b - 1;   // paged tiles of the unit
   s.k_begin = min(t0, n_ctx_b) * kKT;
   const int unit_span =
       kChain ? s.ctx + min(s.T, row_node(p, (s.rb + 1) * kRows - 1) + 1) : (kIP ? s.ctx + s.T : s.ctx);
   s.k_end = t0 < n_ctx_b ? min(unit_span, min(t0 + len, n_ctx_b) * kKT) : s.k_begin;
   s.n_ctx = s.k_end > s.k_begin ? (s.k_end - s.k_begin + kKT - 1) / kKT : 0;
-  s.n_tiles = s.n_ctx + (!kIP && t0 + len == tiles ? 1 : 0);
+  s.n_tiles = s.n_ctx + (!kIP && len > 0 && t0 + len == n_tiles_b ? 1 : 0);
   int ph = (tb - t0) % P;
   ph += ph < 0 ? P : 0;
   s.rot = ph < len ? ph : 0;
-  s.alone = U0 >= x_begin && U0 + tiles <= x_end;
+  s.alone = U0 + kUnitCost >= x_begin && U0 + tiles <= x_end;
   s.U0 = U0;
   s.tiles = tiles;
   // a piece starts the CTA's range (slot 2c) or ends it (slot 2c + 1)
@@ -571,17 +574,20 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
 
   // ---- balanced mode: the shared work list ---------------------------------------
   // Work is counted in 128-key tiles: sequence b brings n_kv x nrb_b units (a
-  // KV head's row block) of ceil(ctx_b / 128) context tiles + 1 tree tile.
-  // Units are ordered sequence, KV head, row block; CTA c takes the tiles
+  // KV head's row block) of ceil(ctx_b / 128) context tiles + 1 tree tile, and
+  // each unit starts with kUnitCost places that are no tiles: a CTA that ends one
+  // unit and starts the next waits for the last P V, stores a partial and starts
+  // a new pipeline, 5,700 cycles or nearly three tiles more than its neighbours.
+  // Units are ordered sequence, KV head, row block; CTA c takes the places
   // [c W / N, (c + 1) W / N) of that order, so a CTA may finish one unit and
   // start the next (at most two of its segments are pieces of split units).
-  // N is capped so that every CTA gets at least m = max(2, ceil(t_max / 14))
-  // tiles, which bounds the pieces of any unit by 15.
+  // N is capped so that every CTA gets at least m = max(2, ceil((t_max +
+  // kUnitCost) / 13)) places, which bounds the pieces of any unit by 15.
   // The K producer builds it: lane l takes sequences [per l, per l + per), per = ceil(B / 32).
   if constexpr (kBal) {
     if (warp == kWarpK) {
       const int per = (p.B + 31) >> 5;     // sequences of a lane
-      int wsum = 0, tmax = 0;
+      int wsum = 0, asum = 0, tmax = 0;
       for (int k = 0; k < per; ++k) {      // (clamped indices)
         const int bb = min(lane * per + k, p.B - 1);
         s_seq[lane * per + k] = make_int4(p.node_off[bb], p.node_off[bb + 1], p.ctx_len[bb], 0);
@@ -599,7 +605,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
           const int c = min(max(sq.z, 0), p.max_ctx);
           int acc = 0;
           if (!bad)
-            for (int r = lane; r < (Tb * g + kRows - 1) / kRows; r += 32) acc += chain_tiles(p, c, Tb, r);
+            for (int r = lane; r < (Tb * g + kRows - 1) / kRows; r += 32) acc += chain_tiles(p, c, Tb, r) + kUnitCost;
           acc = __reduce_add_sync(0xffffffffu, acc);
           __syncwarp();
           if (lane == 0) s_seq[bb].w = acc;
@@ -621,18 +627,19 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
           }
           // tiles of a unit (chain: of one KV head's row blocks, whose lengths differ)
           const int nrb_b = bad ? 1 : (Tb * g + kRows - 1) / kRows;
-          int tiles = kIP ? (c + (bad ? 1 : Tb) + kKT - 1) / kKT : (c + kKT - 1) / kKT + 1;
+          int tiles = (kIP ? (c + (bad ? 1 : Tb) + kKT - 1) / kKT : (c + kKT - 1) / kKT + 1) + kUnitCost;
           int unit_max = tiles;
           if constexpr (kChain) {
             tiles = sq.w;
             if (!coop) {
               tiles = 0;
-              for (int r = 0; r < nrb_b && !bad; ++r) tiles += chain_tiles(p, c, Tb, r);
+              for (int r = 0; r < nrb_b && !bad; ++r) tiles += chain_tiles(p, c, Tb, r) + kUnitCost;
             }
-            unit_max = bad ? 1 : chain_tiles(p, c, Tb, nrb_b - 1);
+            unit_max = bad ? 1 : chain_tiles(p, c, Tb, nrb_b - 1) + kUnitCost;
           }
           if (!bad) {
             wl = p.n_kv * (kChain ? 1 : nrb_b) * tiles;
+            asum += wl - p.n_kv * nrb_b * kUnitCost;
             tmax = max(tmax, unit_max);
           }
           s_seq[bb] = make_int4(sq.x, bad ? 0 : Tb, c, tiles);
@@ -649,13 +656,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
       }
       const int W = __shfl_sync(0xffffffffu, incl, 31);
       const int tmax_all = __reduce_max_sync(0xffffffffu, tmax);
+      const int A = __reduce_add_sync(0xffffffffu, asum);   // tiles
       for (int k = 0; k < per; ++k) {
         const int bb = lane * per + k;
         if (bb < p.B) s_wpre[bb] += incl - wsum;
       }
       if (lane == 0) {
-        const int m = max(2, (tmax_all + 13) / 14);
-        const int N = W > 0 ? min((int)gridDim.x, max(1, W / m)) : 0;
+        const int m = max(2, (tmax_all + 12) / 13);
+        const int N = W > 0 ? min((int)gridDim.x, max(1, A / m)) : 0;
         const bool mine = (int)blockIdx.x < N;
         s_sched[0] = mine ? (int)blockIdx.x * W / N : 0;
         s_sched[1] = mine ? ((int)blockIdx.x + 1) * W / N : 0;
@@ -681,7 +689,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   // decoded and published
   auto publish = [&](int n, int y, int tb0, Seg& o) {
     o.n_tiles = 0;
-    if (y > s_sched[0]) bal_segment<kKV>(p, wlist, y, tb0, lane, o);
+    while (y > s_sched[0]) {
+      bal_segment<kKV>(p, wlist, y, tb0, lane, o);
+      if (o.n_tiles > 0) break;   // (else only the unit's first places: no tile)
+      y = o.y;
+    }
     if (lane == 0) {
       s_seg[kBal ? n % kSegRing : 0] = o;
       mbar_arrive(seg_full + 8 * (n % kSegRing));
@@ -837,7 +849,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
           if (!isK && t == min(1, sg.n_tiles - 1) && !sg.alone && lane == 0 && s_npc < 2) {
             // the CTAs holding the unit's first and last tiles, piece 0's slot
             const int W = s_sched[2], N = s_sched[3];
-            const int c0 = ((sg.U0 + 1) * N - 1) / W, c1 = ((sg.U0 + sg.tiles) * N - 1) / W;
+            const int c0 = ((sg.U0 + kUnitCost + 1) * N - 1) / W, c1 = ((sg.U0 + sg.tiles) * N - 1) / W;
             const int slot0 = 2 * c0 + (sg.U0 > c0 * W / N ? 1 : 0);
             const unsigned long long c = ld_relaxed64(
                 reinterpret_cast<const unsigned long long*>(p.part + (size_t)slot0 * kAttnPartBytes + kAttnCntOff));
