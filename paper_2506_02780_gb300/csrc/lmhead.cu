@@ -693,9 +693,11 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
         if (node < p.total_nodes && b.i != 0x7fffffff) atomicMax(&p.keys[node], make_key(b.v, b.i));
         if (kVerify) {
           // this CTA's partial for the node: the 4 warps' lists merged, their sums added
-          // source q of node tile nt is record q n_nt + nt (pair: q = 2 x pair + rank)
-          const int src = kPair ? (first_tile / p.n_nt * 2 + rank) * p.n_nt + nt : (int)blockIdx.x;
-          uint8_t* rec = p.part + ((size_t)src * BN + c) * lm_rec_bytes(K);
+          // records are ordered by node, then source CTA (of the node's tile): the
+          // finalize's warp reads a node's records side by side
+          const int n_src = (int)gridDim.x / p.n_nt;
+          const int src = kPair ? first_tile / p.n_nt * 2 + rank : (int)blockIdx.x / p.n_nt;
+          uint8_t* rec = p.part + ((size_t)(nt * BN + c) * n_src + src) * lm_rec_bytes(K);
           float* pv = reinterpret_cast<float*>(rec);
           int* pi = reinterpret_cast<int*>(rec + 4 * K);
           float2* pl = reinterpret_cast<float2*>(rec + 8 * K);
@@ -824,11 +826,12 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
 // top_tau, writes the ranked ids and top_tau to the workspace; the last CTA to
 // finish runs the acceptance and zeroes the pruning thresholds.
 // ---------------------------------------------------------------------------
-constexpr int kFinWarps = 8;
+constexpr int kFinWarps = 8;   // warps of a CTA: the acceptance's
 constexpr int kSurv = 256;   // per warp: entries that can still be among a node's K best
 
 struct FinParams {
-  int total, B, max_T, BN, n_nt, n_src, K, mode;
+  int total, B, max_T, n_src, K, mode;
+  int npc;                    // nodes per CTA
   const uint8_t* part;
   unsigned long long* gthr;
   int32_t* tk;                // [total][K] (workspace)
@@ -850,10 +853,8 @@ __global__ void __launch_bounds__(32 * kFinWarps, 1) lm_verify_finalize_kernel(c
   __shared__ int s_svn[kFinWarps];
   __shared__ int s_last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int BN = p.BN;
-  const int node = blockIdx.x * kFinWarps + warp;
-  if (node < p.total) {
-    const int nt = node / BN, c = node - nt * BN;
+  const int node = blockIdx.x * p.npc + warp;
+  if (warp < p.npc && node < p.total) {
     constexpr int kRec = lm_rec_bytes(K) / 16;   // 16-byte words per (CTA, node) record
     // the best K-th key any CTA published: at most the node's true K-th best,
     // so only entries reaching it can be among the K best
@@ -870,7 +871,7 @@ __global__ void __launch_bounds__(32 * kFinWarps, 1) lm_verify_finalize_kernel(c
     for (int u = 0; u < kMaxU; ++u) {
       const int q2 = lane + 32 * u;
       const uint4* rec = reinterpret_cast<const uint4*>(
-          p.part + ((size_t)(q2 < p.n_src ? q2 * p.n_nt + nt : nt) * BN + c) * lm_rec_bytes(K));
+          p.part + ((size_t)node * p.n_src + (q2 < p.n_src ? q2 : 0)) * lm_rec_bytes(K));
 #pragma unroll
       for (int t = 0; t < kRec; ++t) w[u][t] = __ldcg(rec + t);
     }
@@ -1191,8 +1192,6 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
     fp.total = total_nodes;
     fp.B = B;
     fp.max_T = max_T;
-    fp.BN = p.BN;
-    fp.n_nt = p.n_nt;
     fp.n_src = grid / p.n_nt;
     fp.K = K;
     fp.mode = va->mode;
@@ -1207,7 +1206,11 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
     fp.ticket = va->fin_ticket;
     fp.acc = AcceptArgs{B, max_T, total_nodes, va->mode, K, node_off, parent, draft_tok, depth, anc,
                         va->gen_mask, accept_len, path, bonus, err};
-    const dim3 fg((total_nodes + kFinWarps - 1) / kFinWarps), fb(32 * kFinWarps);
+    // nodes per CTA (one warp each): one while the CTAs fit on the GPU a few at a
+    // time -- a node's 152 records are scattered loads, and eight warps of them on
+    // one SM took 9 us longer than one (64 nodes, k = 5: 195.5 us against 184.9)
+    fp.npc = std::max(1, std::min(kFinWarps, (total_nodes + 4 * ee::kNumSMs - 1) / (4 * ee::kNumSMs)));
+    const dim3 fg((total_nodes + fp.npc - 1) / fp.npc), fb(32 * kFinWarps);
     cudaError_t fe = cudaErrorInvalidValue;
     switch (K) {
 #define EE_FIN_CASE(n) \
