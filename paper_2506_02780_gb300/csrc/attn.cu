@@ -1374,17 +1374,31 @@ struct Split {
   int bal_ctas = 0, bal_tiles = 0;
 };
 
-// Launch plan.  Cost, in half-tiles, = 2 x waves x (tiles of the busiest CTA
-// + a fixed per-CTA cost of about 3):
-//   cluster mode: S <= 8, waves from the clusters the GPU holds at once (one
-//   slot fewer per wave once a second wave is needed);
-//   cooperative mode: one wave by construction, S up to 16 with n_rb x S
-//   CTAs no more than the GPU holds.  Ties go to the cooperative mode;
-//   balanced mode: every resident CTA takes an equal share of all units'
-//   tiles (w_max at most, t_max per unit at most) and may cross one unit
-//   boundary (about 1.5 tiles more); it needs 2 partial slots per CTA, a
-//   share of at most 256 context tiles (the staged page ids) and B <= 512.
-Split choose_split(int dev, int span, bool tree_tile, int n_rb, long w_max, int t_max, int B, size_t part_slots) {
+// Launch plan: the kind with the least cost.  Cost is in half-tiles of the tile
+// period (0.96 us a tile), less a start that every launch has:
+//   uniform: 2 + 2 x waves x (tiles of the busiest CTA + 5).  Measured: one wave
+//   takes 7.6 (whole row blocks) to 8.7 us + 0.96 us a tile, a further wave about
+//   6 us + its tiles;
+//     cluster mode: S <= 8, waves from the clusters the GPU holds at once (one
+//     slot fewer per wave once a second wave is needed);
+//     cooperative mode: one wave by construction, S up to 16 with n_rb x S
+//     CTAs no more than the GPU holds.  Ties go to the cooperative mode, and
+//     there to the larger S (the smaller one: 0.1 % slower over 98 drawn calls,
+//     single ones 12 % slower to 7 % faster);
+//   balanced mode: 17 + 2 x share, where every resident CTA takes an equal share
+//   of all units' tiles (w_max at most, t_max per unit at most) and of kUnitCost
+//   for each unit; measured 13 us + 0.95 us per tile and unit place with all
+//   sequences at max_ctx.  The line lies 1 us lower than that says because ragged
+//   batches, whose lengths the host does not know, gain from the balance (8
+//   sequences of 1,024 to 16,384: 89 us, and 203 us in equal chunks).  Causal
+//   drafts: 9 more (a row block's CTA that ends early makes room in the uniform
+//   plan, and the units' decode costs more).  It needs 2 partial slots per CTA, a
+//   share of at most kMaxCtaPages pages and B <= 512.
+// Both sides of the line, us per layer, balanced / uniform: 4 x 4,096 keys, 56
+// heads, 64 nodes 46.1 / 38.8; 2 x 4,096, 28 heads 20.6 / 18.1; causal 133 x 4,
+// 56 heads 38.5 / 31.8; 4 x 8,192, 28 heads 38.9 / 40.8; 4 x 16,384 61 / 72.
+Split choose_split(int dev, int span, bool tree_tile, int n_rb, long w_max, int t_max, int B, size_t part_slots,
+                   bool chain) {
   Split best;
   if (span <= 0) return best;                      // the tree tile alone: one chunk
   const int min_splits = (span + kMaxCtaPages * EE_PAGE - 1) / (kMaxCtaPages * EE_PAGE);
@@ -1399,7 +1413,7 @@ Split choose_split(int dev, int span, bool tree_tile, int n_rb, long w_max, int 
     const long act = active_clusters(dev, used);
     long waves = (n_rb + act - 1) / act;
     if (waves >= 2 && act > 1) waves = (n_rb + act - 2) / (act - 1);
-    const long cost = 2 * waves * (tiles + 3);
+    const long cost = 2 + 2 * waves * (tiles + 5);
     if (best_cost < 0 || cost < best_cost) {
       best_cost = cost;
       best.S = used;
@@ -1412,7 +1426,7 @@ Split choose_split(int dev, int span, bool tree_tile, int n_rb, long w_max, int 
       int chunk, used, tiles;
       chunk_for(span, tree_tile, s, &chunk, &used, &tiles);
       if (used < 2 || (size_t)n_rb * used > part_slots) continue;
-      const long cost = 2 * (tiles + 3);
+      const long cost = 2 + 2 * (tiles + 5);
       if (cost <= best_cost) {
         best_cost = cost;
         best.S = used;
@@ -1424,10 +1438,10 @@ Split choose_split(int dev, int span, bool tree_tile, int n_rb, long w_max, int 
   const int capb = resident_ctas<true>(dev);
   if (capb > 0 && B <= kMaxBalSeqs && w_max <= (long)(kMaxCtaPages / (kKT / EE_PAGE)) * capb &&
       part_slots >= 2 * (size_t)capb) {
-    const long m = std::max(2, (t_max + 13) / 14);
+    const long m = std::max(2, (t_max + kUnitCost + 12) / 13);
     const long n_eff = std::min<long>(capb, std::max<long>(1, w_max / m));
     const long share = (w_max + n_eff - 1) / n_eff;
-    const long cost = 2 * share + 9;
+    const long cost = 2 * ((w_max + (long)kUnitCost * n_rb + n_eff - 1) / n_eff) + (chain ? 26 : 17);
     if (best_cost < 0 || cost < best_cost) {
       best_cost = cost;
       best.bal = true;
@@ -1454,7 +1468,8 @@ Split plan_for(int dev, int B, int max_T, int n_q, int n_kv, int max_ctx, int kv
     for (int r = 0; r < nrb; ++r) per_seq += chain_rb_tiles(max_ctx, max_T, g, r);
     per_seq *= n_kv;
   }
-  return choose_split(dev, span, kv == kKVTree, nrb * n_kv * B, (long)B * per_seq, t_max, B, slots);
+  return choose_split(dev, span, kv == kKVTree, nrb * n_kv * B, (long)B * per_seq, t_max, B, slots,
+                      kv == kKVChain);
 }
 
 // Shared by ee_tree_verify_attn (tree K/V from k_tree / v_tree) and

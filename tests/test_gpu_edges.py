@@ -69,7 +69,40 @@ def test_few_rows_split_over_many_ctas(T, ctx):
     U.assert_close(st.attn_out[0].cpu().numpy(), ref, f"T = {T}, ctx = {ctx}")
 
 
-@pytest.mark.parametrize("ctxs", [[512], [700] * 40])
+@pytest.mark.parametrize("B,ctx,T,n_q,n_kv,kind", [(3, 600, 64, 56, 8, "tree"), (16, 60, 120, 28, 4, "inplace"),
+                                                   (1, 72, 560, 56, 8, "chain"), (4, 300, 133, 56, 8, "chain")])
+def test_uniform_plans_beside_the_balanced_line(B, ctx, T, n_q, n_kv, kind):
+    """One to three waves of whole or split row blocks, close to where the plan
+    changes to the balanced launch: ragged contexts and draft sizes below the
+    plan's maxima."""
+    import paper_2506_02780_gb300 as E
+    import test_gpu_chain
+    import test_gpu_inplace
+    from paper_2506_02780_gb300 import step as S
+    rng = np.random.default_rng(9)
+    ctxs = [ctx] + [int(c) for c in rng.integers(0, ctx + 1, B - 1)]
+    Ts = [T] + [int(t) for t in rng.integers(1, T + 1, B - 1)]
+    w = W.build("long" if kind == "chain" else "tiny", seed=76, device="cuda", layers=1, vocab=512, hidden=64,
+                n_q=n_q, n_kv=n_kv, trees=[W.TreeSpec(t, [], [0]) for t in Ts], ctxs=ctxs)
+    mode = {"tree": False, "inplace": True, "chain": "chain"}[kind]
+    assert E.ee_attn_plan(w.B, w.max_T, n_q, n_kv, ctx, inplace=mode)["mode"] != "balanced"
+    if kind == "chain":
+        test_gpu_chain.check_chain_attention(w, nodes=sorted(set(rng.integers(0, w.total_nodes, 128).tolist())))
+    elif kind == "inplace":
+        test_gpu_inplace.check_inplace(w, layers=[0])
+    else:
+        kc, vc = (torch.from_numpy(U.raw16(t).copy()).view(torch.bfloat16) for t in (w.k_cache, w.v_cache))
+        st = S.from_workload(w)
+        st.run()
+        torch.cuda.synchronize()
+        assert E.ee_read_errors(st.ws) == 0
+        anc = O.tree_prepare(w.parent, w.node_off)[1]
+        ref = O.tree_attention(w.q[0], w.k_tree[0], w.v_tree[0], kc[0], vc[0], w.block_table, w.ctx_len, w.node_off,
+                               anc)
+        U.assert_close(st.attn_out[0].cpu().numpy(), ref, "tree attention")
+
+
+@pytest.mark.parametrize("ctxs", [[512], [2900] * 40])
 def test_nan_scores_stay_in_their_row(ctxs):
     """A query row of NaN (split and balanced launches): its output is NaN, every
     other row is bit-identical to a run without it, and no wait gives up."""
