@@ -201,20 +201,20 @@ ee_status ee_tree_prepare(const int32_t* parent, const int32_t* node_off, int32_
  * head_dim must be 128; n_q a multiple of n_kv; max_T <= 128; max_ctx <= 262144;
  * all bf16 arrays 16-byte aligned.  Q.K^T runs on bf16 tensor cores with fp32
  * accumulation in TMEM; P.V runs on bf16 tensor cores with P carried as two
- * bf16 parts (head + tail, about 2^-14 relative) and V as stored; softmax and
+ * bf16 parts (head + tail, about 2^-17 relative) and V as stored; softmax and
  * the output are fp32.  One launch per call, in one of three forms the host
  * picks from the sizes (ee_attn_plan): the context of each 128 query rows is
  * cut into equal chunks, one CTA each, met at a thread-block cluster barrier
  * or (cooperative launch) a counter; or, balanced, one CTA per SM takes an
  * equal share of all row blocks' 128-key tiles, read from the device's
- * ctx_len and node_off (ragged batches, and row-block counts that do not
- * divide the SM count).  Split work writes partial results to slots in `ws`
- * (L2-resident); once a row block's pieces are all written, each of their
- * CTAs merges a share of its rows.  The plan uses only the partial slots the
- * workspace holds: ee_workspace_size(B, total_nodes, n_q, head_dim, max_ctx)
- * bytes admit every plan for trees; a smaller workspace runs a plan with fewer
- * context chunks (one CTA per row block needs none).  EE_ERR_WORKSPACE when
- * ws_bytes is below the fixed head or no plan fits.
+ * ctx_len and node_off (large ragged batches, and row-block counts that do
+ * not divide the SM count).  Split work writes partial results to slots in
+ * `ws` (L2-resident); once a row block's pieces are all written, each of their
+ * CTAs merges a share of its columns.  The plan uses only the partial slots
+ * the workspace holds: ee_workspace_size(B, total_nodes, n_q, head_dim,
+ * max_ctx) bytes admit every plan for trees; a smaller workspace runs a plan
+ * with fewer context chunks (one CTA per row block needs none).
+ * EE_ERR_WORKSPACE when ws_bytes is below the fixed head or no plan fits.
  * Device errors: EE_DEVERR_PAGE (the key is skipped), EE_DEVERR_CTX,
  * EE_DEVERR_TIMEOUT (outputs undefined).
  */
@@ -302,8 +302,9 @@ ee_status ee_lmhead_verify(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t h
  * cluster) or 2 (cooperative launch, merge counters in the workspace),
  * *ctas = CTAs launched.  Mode 3 (balanced, cooperative, one CTA per SM):
  * *splits = CTAs that share the work at most, *chunk = keys per CTA when
- * every sequence holds max_ctx positions and max_T nodes.  Needs the device (occupancy queries): EE_ERR_CUDA
- * without one; EE_ERR_INVALID_ARG for sizes ee_tree_verify_attn rejects.
+ * every sequence holds max_ctx positions and max_T nodes.  Needs the device
+ * (occupancy queries): EE_ERR_CUDA without one; EE_ERR_INVALID_ARG for sizes
+ * ee_tree_verify_attn rejects.
  */
 ee_status ee_attn_plan(int32_t B, int32_t max_T, int32_t n_q, int32_t n_kv, int32_t max_ctx,
                        int32_t inplace, int32_t* splits, int32_t* chunk, int32_t* mode, int32_t* ctas);

@@ -12,32 +12,36 @@
 //     M side of a tcgen05 MMA.
 //   - A CTA processes segments: contiguous 128-key tile ranges of one row
 //     block.  Uniform launches cut each row block's context into S <= 16
-//     chunks of `chunk` keys (a multiple of the 16-token page, at most 2048
-//     pages), one CTA each; the last chunk also processes the tree keys (one
-//     128-key tile, masked by the ancestor bitmask).  Balanced launches give
-//     each of one CTA per SM an equal share of all row blocks' tiles (a CTA
-//     may finish one row block and start the next).  A CTA stages each
-//     segment's page ids in shared memory.
-//   - Q lives in shared memory (the softmax threads load the block's rows
-//     coalesced and store them in the 128-byte-swizzled K-major layout TMA
-//     gives the K tiles) and is the A operand of S = Q K^T; TMEM holds three S
-//     buffers and O (4 x 128 fp32 columns).
+//     chunks of `chunk` keys (a multiple of the 16-token page), one CTA each;
+//     the last chunk also processes the tree keys (one 128-key tile, masked by
+//     the ancestor bitmask).  Balanced launches give each of one CTA per SM an
+//     equal share of all row blocks' tiles (a CTA may finish one row block and
+//     start the next); choose_split picks between them.
+//   - Every role walks the CTA's segments by itself, tiles numbered through over
+//     all of them: nothing but the ring barriers separates one segment from the
+//     next.  In a balanced launch the K producer, which runs ahead of all others,
+//     builds the work list, decodes each segment and publishes it in a ring.
 //   - Keys come in 128-key tiles.  Warps 0 and 2 stream K and V tiles with TMA
-//     (one 16-row box per page and 64-dim half, spread over 8 lanes; the tree's
-//     K/V through a 3-D map) into a 3-stage K ring and a 2-stage V ring.  Warp
-//     1 issues tcgen05.mma in a fixed order: S = Q K^T for the first three
-//     tiles (bf16, fp32 accumulators in TMEM), then for each tile O += P V
-//     followed by the Q K^T three tiles ahead, which overwrites the TMEM
-//     columns P lived in (the in-order tensor pipe finishes reading P first).
-//     With three S buffers the hand-off chain P(t) -> P.V(t) -> Q.K^T(t+3) ->
-//     softmax(t+3) spans three tiles, so it no longer sets the tile period.
+//     (one 16-row box per page and 64-dim half, all issued by one elected lane
+//     from rows that are the same in every lane; the tree's K/V through a 3-D
+//     map) into a 3-stage K ring and a 2-stage V ring; page ids are loaded four
+//     tiles ahead into registers.
+//   - Q lives in shared memory (asynchronous copies in the 128-byte-swizzled
+//     K-major layout TMA gives the K tiles: the softmax warps load the first row
+//     block, the Q.K^T warp later ones) and is the A operand of S = Q K^T; TMEM
+//     holds three S buffers and O (4 x 128 fp32 columns).
+//   - Warp 3 issues S = Q K^T up to three tiles ahead (bf16, fp32 accumulators in
+//     TMEM), warp 1 O += P V, each from one elected lane; a tile's Q K^T waits
+//     for the P V three tiles before, whose P lives in the same TMEM columns.  Two
+//     issuing warps, because a warp that waits for one product's operands would
+//     hold back the other's.
 //   - P.V runs on bf16 operands: P is split into a bf16 head (the fp32 value
 //     rounded to nearest bf16) and a bf16 tail (the exact remainder, rounded
 //     to nearest bf16), both written over S in TMEM and used as the MMA A
 //     operand; V is read straight from shared memory (MN-major).  P is carried
 //     to about 2^-17 relative (fp16 would give 2^-11) and V needs no
-//     conversion; per column pair the split is two packing conversions, a
-//     shift, a mask and one packed subtraction.
+//     conversion.  Per column pair the split is two packing conversions and two
+//     mixed-type subtractions head - p; the MMA negates the tail back.
 //   - Warps 4-11 own one query row per thread (its TMEM lane), two warps per
 //     lane quarter splitting each tile's keys: they read S, mask, keep the
 //     running max/sum, write P, and rescale O in TMEM only when a row's max
@@ -45,11 +49,11 @@
 //     O / l is unchanged).
 //   - Every chunk-CTA writes its unnormalised O rows and (max, sum) from TMEM
 //     to its own slot of the workspace (fp32, column-chunk major so that a
-//     warp's stores are contiguous; the slots stay in L2).  Once all S slots of
-//     a row block are written, chunk k merges the contiguous rows
-//     [k * ceil(128 / S), ...) of all S slots with log-sum-exp weights and
-//     writes the fp32 output: one launch, no second pass, and L2 moves the
-//     partials several times faster than distributed shared memory does.
+//     warp's stores are contiguous; the slots stay in L2).  Once all K slots of
+//     a row block are written, the softmax warps of piece k merge 32 / K of the
+//     32 four-column chunks of all its rows with log-sum-exp weights and write
+//     the fp32 output: one launch, no second pass, and L2 moves the partials
+//     several times faster than distributed shared memory does.
 //     A segment that is a whole row block writes O / l directly.  The CTAs of
 //     a row block learn that all slots are written in one of two ways, chosen
 //     by the host:
@@ -57,21 +61,31 @@
 //         barrier (release / acquire at cluster scope);
 //       cooperative: the launch is cooperative (every CTA resident at once);
 //         the row block's 64-bit count grows by 720720 = lcm(1..16) per
-//         launch: each of its S CTAs reads the count at its start (a
-//         multiple of 720720 plus some of this launch's arrivals, never all:
-//         its own is missing; a relaxed load whose value is first used at the
-//         end), stores its partial, and after a CTA barrier one thread adds
-//         720720 / S with a release reduction and waits (acquire) for the next
-//         multiple.  One release per CTA orders all its threads'
-//         stores, and nothing resets the count at the end of the kernel.  No
-//         GPC packing constraint: S can be any value up to 16, so the grid can
-//         cover every SM.  Balanced launches count the pieces of each split
-//         row block the same way.
+//         launch: the V producer reads the count early (a multiple of 720720
+//         plus some of this launch's arrivals, never all: this CTA's own is
+//         missing; a relaxed load whose value is first used at the end), and
+//         after the CTA's partial is stored and its threads have met at a
+//         barrier one thread adds 720720 / K with a release reduction and waits
+//         (acquire) for the next multiple.  One release per CTA orders all its
+//         threads' stores, and nothing resets the count at the end of the
+//         kernel.  No GPC packing constraint: K can be any value up to 16, so
+//         the grid can cover every SM.  Balanced launches count the pieces of
+//         each split row block the same way.
 //     Every CTA, also one whose chunk is empty for a short sequence, arrives:
 //     every wait before the arrival is bounded.
 //   - The next kernel in the stream may launch (programmatic dependent launch)
 //     once every CTA has drained its pipeline; triggering earlier lets its
 //     CTAs hold SMs that a later wave of this grid still needs.
+//
+// What bounds it (SM cycles at 2.07 GHz).  Long work: the tile period, 2,000 to
+// 2,040.  A tile's MMAs take 1,536 (24 of 128 x 128 x 16) and about 1,700 with
+// their operand waits; the softmax warps, two per sub-partition, walk the rest:
+// wait for S 140, load and maxima 400, the pair's exchange 165, exponentials,
+// split and stores 1,050 to 1,150, sums and arrival 200.  Tensor pipe 65 % active
+// (56 heads, 128 nodes, 32,768 keys, one layer: 148 -> 125 us).  A segment switch
+// costs 5,700 more.  Short work: latency.  28 heads, 64 nodes, 4,096 keys, 4 tiles
+// a CTA: 13.3 us, of which 2.8 until the first scores, 4 x 1 for the tiles, 1.3 to
+// store the partial, 0.9 for its release, 0.6 for the count and 2 to merge.
 // Shared-memory traffic per 128-key tile: K 64 KB + V 64 KB (TMA write, MMA
 // read) + Q 32 KB (MMA read).
 #include "ee_common.cuh"
@@ -90,7 +104,7 @@ constexpr int kVST = 2;                          // V ring depth
 constexpr int kSB = 3;                           // S buffers in TMEM (Q.K^T runs kSB tiles ahead)
 constexpr uint32_t kKVHalf = kKT * 128;          // 16 KB: one 64-dim half of a K or V tile
 constexpr uint32_t kKVBytes = 2 * kKVHalf;       // 32 KB
-constexpr int kMaxCtaPages = 2048;               // context pages one CTA owns at most (32768 keys)
+constexpr int kMaxCtaPages = 2048;               // context pages of one CTA's share at most (32768 keys)
 constexpr int kUnitCost = 3;                      // balanced: a unit's weight beyond its tiles (see the work list)
 constexpr int kSegRing = 16;                     // published segments (K runs at most 8 ahead of the softmax)
 constexpr int kMaskRing = 8;                     // page-validity masks in flight (K runs at most 6 tiles ahead)
@@ -224,8 +238,8 @@ __device__ __forceinline__ void merge_rows(const AttnParams& p, size_t slot_a, s
 }
 // kX: 16 kX loads per thread in flight
 template <int kX>
-__device__ __forceinline__ void merge_pieces(const AttnParams& p, size_t slot_a, size_t slot_b, int stride, int K, int k,
-                                             int row0, int rows, int o, int hk, int tid, int nthr) {
+__device__ __forceinline__ void merge_pieces(const AttnParams& p, size_t slot_a, size_t slot_b, int stride, int K,
+                                             int k, int row0, int rows, int o, int hk, int tid, int nthr) {
   const int c_lo = kD / 4 * k / K, c_hi = kD / 4 * (k + 1) / K;   // piece k's chunks
   if (K <= 2) merge_rows<2, 8 * kX>(p, slot_a, slot_b, stride, K, row0, rows, c_lo, c_hi, o, hk, tid, nthr);
   else if (K <= 4) merge_rows<4, 4 * kX>(p, slot_a, slot_b, stride, K, row0, rows, c_lo, c_hi, o, hk, tid, nthr);
@@ -735,215 +749,217 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   // launch's).  A balanced launch's producers need theirs: with 88 registers the K
   // warp spills and the tile period grows (33B-shaped layer 129.5 -> 134 us).
   if (warp < kWarpSoft0) {
-  if constexpr (!kBal) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
-  if (warp == kWarpK || warp == kWarpV) {
-    // ---------------- TMA producers: warp 0 streams K, warp 2 streams V ----------------
-    // Ring slots and phases count the CTA's tiles over all its segments.  Lane l
-    // holds the page id of 16-row block l % 8 of the (l / 8)-th of four
-    // consecutive tiles, loaded four tiles ahead; one elected lane issues the
-    // tile's 16 boxes (eight blocks, two 64-dim halves) from warp-uniform rows.
-    // Boxes issued by different lanes are serialised one by one: 1100 cycles a
-    // tile (and the K stream behind the tensor pipe), against about 300.
-    const bool isK = warp == kWarpK;
-    const int nst = isK ? kKST : kVST;
-    const uint32_t full0 = isK ? k_full : v_full, empty0 = isK ? k_empty : v_empty;
-    const uint32_t ring = isK ? sK : sV;
-    const CUtensorMap* mc = isK ? &tmKc : &tmVc;
-    const CUtensorMap* mt = isK ? &tmKt : &tmVt;
-    int* issued = isK ? s_kissued : s_vissued;
-    int32_t early = -1;
-    unsigned long long u_count = 0;
-    if constexpr (!kBal) {
-      // the chunk's first page ids (and the row block's count), issued beside the
-      // node range and context length so that the round trips overlap
-      const int split = (int)(blockIdx.x % p.S);
-      const int pg = split * (p.chunk / EE_PAGE) + lane;
-      if (pg < p.max_pages) early = ld_nc_pinned(p.block_table + (size_t)blockIdx.z * p.max_pages + pg);
-      if (!isK && lane == 0 && p.coop && p.S > 1)
-        u_count = ld_relaxed64(reinterpret_cast<const unsigned long long*>(
-            p.part + (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x - split) * kAttnPartBytes +
-            kAttnCntOff));
-    }
-    bool more = first(isK && lane == 0);
-    if constexpr (!kBal) {
-      // the count any time before this CTA's own arrival is a multiple of
-      // kCountGen plus the arrivals of this launch so far, never all of them
-      if (!isK && lane == 0 && more) {
-        s_uni = make_int2(sg.o, sg.T * g);
-        s_pc[0].target = (u_count / kCountGen + 1) * kCountGen;
+    if constexpr (!kBal) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
+    if (warp == kWarpK || warp == kWarpV) {
+      // ---------------- TMA producers: warp 0 streams K, warp 2 streams V ----------------
+      // Ring slots and phases count the CTA's tiles over all its segments.  Lane l
+      // holds the page id of 16-row block l % 8 of the (l / 8)-th of four
+      // consecutive tiles, loaded four tiles ahead; one elected lane issues the
+      // tile's 16 boxes (eight blocks, two 64-dim halves) from warp-uniform rows.
+      // Boxes issued by different lanes are serialised one by one: 1100 cycles a
+      // tile (and the K stream behind the tensor pipe), against about 300.
+      const bool isK = warp == kWarpK;
+      const int nst = isK ? kKST : kVST;
+      const uint32_t full0 = isK ? k_full : v_full, empty0 = isK ? k_empty : v_empty;
+      const uint32_t ring = isK ? sK : sV;
+      const CUtensorMap* mc = isK ? &tmKc : &tmVc;
+      const CUtensorMap* mt = isK ? &tmKt : &tmVt;
+      int* issued = isK ? s_kissued : s_vissued;
+      int32_t early = -1;
+      unsigned long long u_count = 0;
+      if constexpr (!kBal) {
+        // the chunk's first page ids (and the row block's count), issued beside the
+        // node range and context length so that the round trips overlap
+        const int split = (int)(blockIdx.x % p.S);
+        const int pg = split * (p.chunk / EE_PAGE) + lane;
+        if (pg < p.max_pages) early = ld_nc_pinned(p.block_table + (size_t)blockIdx.z * p.max_pages + pg);
+        if (!isK && lane == 0 && p.coop && p.S > 1)
+          u_count = ld_relaxed64(reinterpret_cast<const unsigned long long*>(
+              p.part +
+              (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x - split) * kAttnPartBytes +
+              kAttnCntOff));
       }
-    }
-    bool go = true;
-    // page ids of tiles 4 c .. 4 c + 3 of the segment's order (INT_MIN: no keys
-    // there), one predicated load that nothing waits for before the ids are used
-    auto fetch = [&](const Seg& sg, int c) -> int32_t {
-      const int t = 4 * c + (lane >> 3);
-      const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;
-      const int pos = sg.k_begin + i * kKT + 16 * (lane & 7);
-      const bool need = t < sg.n_tiles && i < sg.n_ctx && pos < sg.k_end;
-      if (!kBal && c == 0) return need ? early : INT32_MIN;
-      int32_t v = INT32_MIN;
-      if (need) v = ld_nc_pinned(p.block_table + (size_t)sg.b * p.max_pages + pos / EE_PAGE);
-      return v;
-    };
-    // balanced, the K producer: the next segment (decoded and published, its first
-    // page ids on the way, while this one's tiles wait for ring slots)
-    int32_t nx_ids = INT32_MIN;
-    while (more && go) {
-      int32_t ids = kBal && isK && nseg > 0 ? nx_ids : fetch(sg, 0), ids_next = INT32_MIN;
-      for (int t = 0; t < sg.n_tiles; ++t) {
-        if ((t & 3) == 0) {
-          if (t > 0) ids = ids_next;
-          ids_next = fetch(sg, (t >> 2) + 1);
+      bool more = first(isK && lane == 0);
+      if constexpr (!kBal) {
+        // the count any time before this CTA's own arrival is a multiple of
+        // kCountGen plus the arrivals of this launch so far, never all of them
+        if (!isK && lane == 0 && more) {
+          s_uni = make_int2(sg.o, sg.T * g);
+          s_pc[0].target = (u_count / kCountGen + 1) * kCountGen;
         }
-        const int tg = tb + t;
-        const int st = tg % nst, use = tg / nst;
-        // the tile's eight blocks, the same in every lane: first cache row, -EE_PAGE
-        // without a page; need8: the blocks that hold keys
-        const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;   // the segment's tile
-        const int left = sg.k_end - (sg.k_begin + i * kKT);
-        const unsigned need8 = i >= sg.n_ctx ? 0u : left >= kKT ? 0xFFu : (1u << ((left + 15) >> 4)) - 1u;
-        int row[kKT / 16];
-        unsigned okm = 0u;      // bit i: block i has keys in a valid page
-        bool bad = false;
+      }
+      bool go = true;
+      // page ids of tiles 4 c .. 4 c + 3 of the segment's order (INT_MIN: no keys
+      // there), one predicated load that nothing waits for before the ids are used
+      auto fetch = [&](const Seg& sg, int c) -> int32_t {
+        const int t = 4 * c + (lane >> 3);
+        const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;
+        const int pos = sg.k_begin + i * kKT + 16 * (lane & 7);
+        const bool need = t < sg.n_tiles && i < sg.n_ctx && pos < sg.k_end;
+        if (!kBal && c == 0) return need ? early : INT32_MIN;
+        int32_t v = INT32_MIN;
+        if (need) v = ld_nc_pinned(p.block_table + (size_t)sg.b * p.max_pages + pos / EE_PAGE);
+        return v;
+      };
+      // balanced, the K producer: the next segment (decoded and published, its first
+      // page ids on the way, while this one's tiles wait for ring slots)
+      int32_t nx_ids = INT32_MIN;
+      while (more && go) {
+        int32_t ids = kBal && isK && nseg > 0 ? nx_ids : fetch(sg, 0), ids_next = INT32_MIN;
+        for (int t = 0; t < sg.n_tiles; ++t) {
+          if ((t & 3) == 0) {
+            if (t > 0) ids = ids_next;
+            ids_next = fetch(sg, (t >> 2) + 1);
+          }
+          const int tg = tb + t;
+          const int st = tg % nst, use = tg / nst;
+          // the tile's eight blocks, the same in every lane: first cache row, -EE_PAGE
+          // without a page; need8: the blocks that hold keys
+          const int i = t + sg.rot < sg.n_tiles ? t + sg.rot : t + sg.rot - sg.n_tiles;   // the segment's tile
+          const int left = sg.k_end - (sg.k_begin + i * kKT);
+          const unsigned need8 = i >= sg.n_ctx ? 0u : left >= kKT ? 0xFFu : (1u << ((left + 15) >> 4)) - 1u;
+          int row[kKT / 16];
+          unsigned okm = 0u;      // bit i: block i has keys in a valid page
+          bool bad = false;
 #pragma unroll
-        for (int q = 0; q < kKT / 16; ++q) {
-          const int32_t id = __shfl_sync(0xffffffffu, ids, 8 * (t & 3) + q);
-          const bool ok = id >= 0 && id < p.num_pages;
-          row[q] = ok ? (id * p.n_kv + sg.hk) * EE_PAGE : -EE_PAGE;
-          okm |= ok ? 1u << q : 0u;
-          bad |= !ok && (need8 >> q & 1u);
-        }
-        if (isK && bad && lane == 0) flag_error(p.err, EE_DEVERR_PAGE);
-        go = wait(empty0 + 8 * st, use + 1);
-        if (!go) break;
-        const uint32_t full = full0 + 8 * st;
-        const uint32_t dst = ring + st * kKVBytes;
-        if (elect_one()) {
-          if (isK) s_mask[tg % kMaskRing] = okm;
-          mbar_expect_tx(full, 2 * kKVHalf);
-          if (i < sg.n_ctx) {
-            // every 16-row block is written: blocks without a loaded page are read at
-            // row -16, wholly out of range, which the TMA unit fills with zeros (a
-            // stale V row would turn 0 * P into NaN)
+          for (int q = 0; q < kKT / 16; ++q) {
+            const int32_t id = __shfl_sync(0xffffffffu, ids, 8 * (t & 3) + q);
+            const bool ok = id >= 0 && id < p.num_pages;
+            row[q] = ok ? (id * p.n_kv + sg.hk) * EE_PAGE : -EE_PAGE;
+            okm |= ok ? 1u << q : 0u;
+            bad |= !ok && (need8 >> q & 1u);
+          }
+          if (isK && bad && lane == 0) flag_error(p.err, EE_DEVERR_PAGE);
+          go = wait(empty0 + 8 * st, use + 1);
+          if (!go) break;
+          const uint32_t full = full0 + 8 * st;
+          const uint32_t dst = ring + st * kKVBytes;
+          if (elect_one()) {
+            if (isK) s_mask[tg % kMaskRing] = okm;
+            mbar_expect_tx(full, 2 * kKVHalf);
+            if (i < sg.n_ctx) {
+              // every 16-row block is written: blocks without a loaded page are read at
+              // row -16, wholly out of range, which the TMA unit fills with zeros (a
+              // stale V row would turn 0 * P into NaN)
 #pragma unroll
-            for (int q = 0; q < kKT / 16; ++q) {
-              tma_load_2d(dst + q * 2048, mc, full, 0, row[q]);
-              tma_load_2d(dst + kKVHalf + q * 2048, mc, full, 64, row[q]);
+              for (int q = 0; q < kKT / 16; ++q) {
+                tma_load_2d(dst + q * 2048, mc, full, 0, row[q]);
+                tma_load_2d(dst + kKVHalf + q * 2048, mc, full, 64, row[q]);
+              }
+            } else {
+              tma_load_3d(dst, mt, full, 0, sg.hk, sg.o);
+              tma_load_3d(dst + kKVHalf, mt, full, 64, sg.hk, sg.o);
             }
-          } else {
-            tma_load_3d(dst, mt, full, 0, sg.hk, sg.o);
-            tma_load_3d(dst + kKVHalf, mt, full, 64, sg.hk, sg.o);
+          }
+          __syncwarp();
+          if (lane == 0) issued[st] = use;
+          if constexpr (kBal) {
+            if (isK && t == min(kKST - 1, sg.n_tiles - 1)) {
+              Seg nx;
+              publish(nseg + 1, sg.y, tb + sg.n_tiles, nx);
+              nx_ids = fetch(nx, 0);
+            }
+            // the piece of a split row block, and its count as read before this
+            // CTA's own arrival
+            if (!isK && t == min(1, sg.n_tiles - 1) && !sg.alone && lane == 0 && s_npc < 2) {
+              // the CTAs holding the unit's first and last tiles, piece 0's slot
+              const int W = s_sched[2], N = s_sched[3];
+              const int c0 = ((sg.U0 + kUnitCost + 1) * N - 1) / W, c1 = ((sg.U0 + sg.tiles) * N - 1) / W;
+              const int slot0 = 2 * c0 + (sg.U0 > c0 * W / N ? 1 : 0);
+              const unsigned long long c = ld_relaxed64(
+                  reinterpret_cast<const unsigned long long*>(p.part + (size_t)slot0 * kAttnPartBytes + kAttnCntOff));
+              s_pc[s_npc] = BalPiece{sg.hk, sg.rb, sg.o, sg.T * g, c1 - c0 + 1, (int)blockIdx.x - c0,
+                                     slot0, 2 * (c0 + 1), (c / kCountGen + 1) * kCountGen};
+              s_npc = s_npc + 1;
+            }
           }
         }
-        __syncwarp();
-        if (lane == 0) issued[st] = use;
-        if constexpr (kBal) {
-          if (isK && t == min(kKST - 1, sg.n_tiles - 1)) {
-            Seg nx;
-            publish(nseg + 1, sg.y, tb + sg.n_tiles, nx);
-            nx_ids = fetch(nx, 0);
-          }
-          // the piece of a split row block, and its count as read before this
-          // CTA's own arrival
-          if (!isK && t == min(1, sg.n_tiles - 1) && !sg.alone && lane == 0 && s_npc < 2) {
-            // the CTAs holding the unit's first and last tiles, piece 0's slot
-            const int W = s_sched[2], N = s_sched[3];
-            const int c0 = ((sg.U0 + kUnitCost + 1) * N - 1) / W, c1 = ((sg.U0 + sg.tiles) * N - 1) / W;
-            const int slot0 = 2 * c0 + (sg.U0 > c0 * W / N ? 1 : 0);
-            const unsigned long long c = ld_relaxed64(
-                reinterpret_cast<const unsigned long long*>(p.part + (size_t)slot0 * kAttnPartBytes + kAttnCntOff));
-            s_pc[s_npc] = BalPiece{sg.hk, sg.rb, sg.o, sg.T * g, c1 - c0 + 1, (int)blockIdx.x - c0,
-                                   slot0, 2 * (c0 + 1), (c / kCountGen + 1) * kCountGen};
-            s_npc = s_npc + 1;
-          }
+        if (kBal && isK) {
+          tb += sg.n_tiles;
+          ++nseg;
+          sg = s_seg[kBal ? nseg % kSegRing : 0];
+          more = sg.n_tiles > 0;
+        } else {
+          more = next();
         }
       }
-      if (kBal && isK) {
-        tb += sg.n_tiles;
-        ++nseg;
-        sg = s_seg[kBal ? nseg % kSegRing : 0];
-        more = sg.n_tiles > 0;
-      } else {
-        more = next();
-      }
-    }
-  } else if (warp == kWarpQk) {
-    // ---------------- S = Q K^T, up to kSB tiles ahead of P.V ----------------
-    // One warp issues Q.K^T and another P.V: while one waits for its operands (a
-    // ready mbarrier still costs about 100 cycles to see), the other's MMAs keep
-    // the tensor pipe busy.  The whole warp walks the loop and one elected lane
-    // issues, every descriptor an offset from a uniform base.
-    const uint32_t id_qk = idesc_f16(kRows, kKT, 1, 1, 0);
-    const uint64_t dq = smem_desc_sw128(__shfl_sync(0xffffffffu, sQ, 0));
-    const uint64_t dk0 = smem_desc_sw128(__shfl_sync(0xffffffffu, sK, 0));
-    bool go = true;
-    for (bool more = first(false); more && go; more = next()) {
-      if (sg.n_tiles == 0) continue;
-      if (nseg == 0) {
-        go = wait(q_ready, 0);       // the softmax warps load the first row block
-      } else {
-        // the previous segment's last Q.K^T has read its rows; the load runs while
-        // its last kSB tiles are in the softmax
-        go = wait(q_empty, nseg - 1);
-        if (go) load_q<2, kRows / 2>(p, sg, sQ, 0, lane);
-      }
-      tc_fence_after();
-      for (int t = 0; t < sg.n_tiles && go; ++t) {
-        const int tg = tb + t;
-        const int st = tg % kKST, sb = tg % kSB;
-        if (tg >= kSB) go = wait(pv_done + 8 * sb, tg / kSB - 1);   // S buffer's P consumed
-        go = go && wait(k_full + 8 * st, tg / kKST);
-        if (!go) break;
+    } else if (warp == kWarpQk) {
+      // ---------------- S = Q K^T, up to kSB tiles ahead of P.V ----------------
+      // One warp issues Q.K^T and another P.V: while one waits for its operands (a
+      // ready mbarrier still costs about 100 cycles to see), the other's MMAs keep
+      // the tensor pipe busy.  The whole warp walks the loop and one elected lane
+      // issues, every descriptor an offset from a uniform base.
+      const uint32_t id_qk = idesc_f16(kRows, kKT, 1, 1, 0);
+      const uint64_t dq = smem_desc_sw128(__shfl_sync(0xffffffffu, sQ, 0));
+      const uint64_t dk0 = smem_desc_sw128(__shfl_sync(0xffffffffu, sK, 0));
+      bool go = true;
+      for (bool more = first(false); more && go; more = next()) {
+        if (sg.n_tiles == 0) continue;
+        if (nseg == 0) {
+          go = wait(q_ready, 0);       // the softmax warps load the first row block
+        } else {
+          // the previous segment's last Q.K^T has read its rows; the load runs while
+          // its last kSB tiles are in the softmax
+          go = wait(q_empty, nseg - 1);
+          if (go) load_q<2, kRows / 2>(p, sg, sQ, 0, lane);
+        }
         tc_fence_after();
-        if (elect_one()) {
-          const uint64_t dk = dk0 + (uint64_t)(st * (kKVBytes >> 4));
+        for (int t = 0; t < sg.n_tiles && go; ++t) {
+          const int tg = tb + t;
+          const int st = tg % kKST, sb = tg % kSB;
+          if (tg >= kSB) go = wait(pv_done + 8 * sb, tg / kSB - 1);   // S buffer's P consumed
+          go = go && wait(k_full + 8 * st, tg / kKST);
+          if (!go) break;
+          tc_fence_after();
+          if (elect_one()) {
+            const uint64_t dk = dk0 + (uint64_t)(st * (kKVBytes >> 4));
 #pragma unroll
-          for (int kk = 0; kk < kD / 16; ++kk) {
-            const uint64_t off = ((kk >> 2) * kKVHalf + (kk & 3) * 32) >> 4;
-            tc_mma(tmem + sb * kKT, dq + off, dk + off, id_qk, kk > 0 ? 1u : 0u);
+            for (int kk = 0; kk < kD / 16; ++kk) {
+              const uint64_t off = ((kk >> 2) * kKVHalf + (kk & 3) * 32) >> 4;
+              tc_mma(tmem + sb * kKT, dq + off, dk + off, id_qk, kk > 0 ? 1u : 0u);
+            }
+            tc_commit(s_full + 8 * sb);
+            tc_commit(k_empty + 8 * st);
+            if (t == sg.n_tiles - 1) tc_commit(q_empty);
+            mbar_arrive(s_full + 8 * sb);   // releases the tile's page mask (acquired with k_full)
           }
-          tc_commit(s_full + 8 * sb);
-          tc_commit(k_empty + 8 * st);
-          if (t == sg.n_tiles - 1) tc_commit(q_empty);
-          mbar_arrive(s_full + 8 * sb);   // releases the tile's page mask (acquired with k_full)
+          __syncwarp();
         }
-        __syncwarp();
+      }
+    } else if (warp == kWarpPv) {
+      // ---------------- O += P V ----------------
+      const uint32_t id_pv = idesc_f16(kRows, kD, 1, 1, 1);
+      const uint64_t dv0 = smem_desc_sw128_mn(__shfl_sync(0xffffffffu, sV, 0), kKVHalf, 1024);
+      bool go = true;
+      int filled = 0;    // segments with tiles so far
+      for (bool more = first(false); more && go; more = next()) {
+        if (sg.n_tiles == 0) continue;
+        // the softmax has read the previous segment's O
+        if (filled > 0) go = wait(o_free, filled - 1);
+        ++filled;
+        for (int t = 0; t < sg.n_tiles && go; ++t) {
+          const int tg = tb + t;
+          const int st = tg % kVST, sb = tg % kSB;
+          go = wait(v_full + 8 * st, tg / kVST) && wait(p_full + 8 * sb, tg / kSB);
+          if (!go) break;
+          tc_fence_after();
+          if (elect_one()) {
+            const uint32_t pa = tmem + sb * kKT;       // bf16 P head: cols 0..63, tail: 64..127
+            const uint64_t dv = dv0 + (uint64_t)(st * (kKVBytes >> 4));
+#pragma unroll
+            for (int part = 0; part < 2; ++part)
+#pragma unroll
+              for (int j = 0; j < kKT / 16; ++j)
+                tc_mma_ts(tmem + kColO, pa + 64 * part + 8 * j, dv + (uint64_t)(j * (2048 >> 4)),
+                          part ? (id_pv | kIdescNegA) : id_pv,
+                          (t > 0 || part > 0 || j > 0) ? 1u : 0u);
+            tc_commit(pv_done + 8 * sb);
+            tc_commit(v_empty + 8 * st);
+          }
+          __syncwarp();
+        }
       }
     }
-  } else if (warp == kWarpPv) {
-    // ---------------- O += P V ----------------
-    const uint32_t id_pv = idesc_f16(kRows, kD, 1, 1, 1);
-    const uint64_t dv0 = smem_desc_sw128_mn(__shfl_sync(0xffffffffu, sV, 0), kKVHalf, 1024);
-    bool go = true;
-    int filled = 0;    // segments with tiles so far
-    for (bool more = first(false); more && go; more = next()) {
-      if (sg.n_tiles == 0) continue;
-      // the softmax has read the previous segment's O
-      if (filled > 0) go = wait(o_free, filled - 1);
-      ++filled;
-      for (int t = 0; t < sg.n_tiles && go; ++t) {
-        const int tg = tb + t;
-        const int st = tg % kVST, sb = tg % kSB;
-        go = wait(v_full + 8 * st, tg / kVST) && wait(p_full + 8 * sb, tg / kSB);
-        if (!go) break;
-        tc_fence_after();
-        if (elect_one()) {
-          const uint32_t pa = tmem + sb * kKT;       // bf16 P head: cols 0..63, tail: 64..127
-          const uint64_t dv = dv0 + (uint64_t)(st * (kKVBytes >> 4));
-#pragma unroll
-          for (int part = 0; part < 2; ++part)
-#pragma unroll
-            for (int j = 0; j < kKT / 16; ++j)
-              tc_mma_ts(tmem + kColO, pa + 64 * part + 8 * j, dv + (uint64_t)(j * (2048 >> 4)), part ? (id_pv | kIdescNegA) : id_pv,
-                        (t > 0 || part > 0 || j > 0) ? 1u : 0u);
-          tc_commit(pv_done + 8 * sb);
-          tc_commit(v_empty + 8 * st);
-        }
-        __syncwarp();
-      }
-    }
-  }
 
     // ---- producers and MMA issuers: drain on abort, free TMEM ----------------------
     tc_fence_before();
@@ -974,7 +990,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
     if (!kBal && s_uni.y > 0 && p.S > 1 && !p.coop) cluster_sync();   // with the softmax warps' below
     return;
   }
-if constexpr (!kBal) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoft));
+  if constexpr (!kBal) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoft));
   // ---------------- softmax: one query row and half of every tile per thread ----------------
   // Warps w and w + 4 share TMEM lane quarter w & 3 (32 query rows); half hf
   // of the pair takes keys [64 hf, 64 hf + 64) of every tile and O columns
@@ -1359,7 +1375,7 @@ cudaError_t set_attrs(int dev) {
 void chunk_for(int span, bool tree_tile, int s, int* chunk, int* used, int* tiles) {
   int c = (span + (tree_tile ? kKT : 0) + s - 1) / s;
   c = (c + EE_PAGE - 1) / EE_PAGE * EE_PAGE;
-  c = std::min(c, kMaxCtaPages * EE_PAGE);          // a CTA stages at most kMaxCtaPages page ids
+  c = std::min(c, kMaxCtaPages * EE_PAGE);
   *chunk = c;
   *used = attn_splits_for(span, c);
   const int last = span - (*used - 1) * c;
@@ -1394,15 +1410,20 @@ struct Split {
 //   drafts: 9 more (a row block's CTA that ends early makes room in the uniform
 //   plan, and the units' decode costs more).  It needs 2 partial slots per CTA, a
 //   share of at most kMaxCtaPages pages and B <= 512.
-// Both sides of the line, us per layer, balanced / uniform: 4 x 4,096 keys, 56
-// heads, 64 nodes 46.1 / 38.8; 2 x 4,096, 28 heads 20.6 / 18.1; causal 133 x 4,
-// 56 heads 38.5 / 31.8; 4 x 8,192, 28 heads 38.9 / 40.8; 4 x 16,384 61 / 72.
+// Both sides, us per layer, balanced / uniform: causal 560, 56 heads 30.0 / 24.9;
+// causal 4 x 133 after 880 keys 38.5 / 31.8; 16 x 120 nodes after 60 keys, 28
+// heads 25.9 / 23.6; 4 x 16,384 keys, 28 heads 61 / 72.
+// The relative error against 64 bits grows with the tiles that one CTA adds up in
+// its accumulator (about 2.8e-7 a tile).  Where equal chunks would be longer than
+// the balanced shares the time therefore does not decide: the balanced launch is
+// taken from 1.5 tiles fewer on (4 x 4,096 keys, 56 heads: 46.1 us balanced with
+// an error of 6.6e-6; equal chunks would take 38.8 us with 9.4e-6).
 Split choose_split(int dev, int span, bool tree_tile, int n_rb, long w_max, int t_max, int B, size_t part_slots,
                    bool chain) {
   Split best;
   if (span <= 0) return best;                      // the tree tile alone: one chunk
   const int min_splits = (span + kMaxCtaPages * EE_PAGE - 1) / (kMaxCtaPages * EE_PAGE);
-  long best_cost = -1;
+  long best_cost = -1, best_tiles = 0, best_len = 0;   // (best_len: 2 x waves x (tiles + 3))
   for (int s = std::max(1, min_splits); s <= kMaxCluster; ++s) {
     int chunk, used, tiles;
     chunk_for(span, tree_tile, s, &chunk, &used, &tiles);
@@ -1416,6 +1437,8 @@ Split choose_split(int dev, int span, bool tree_tile, int n_rb, long w_max, int 
     const long cost = 2 + 2 * waves * (tiles + 5);
     if (best_cost < 0 || cost < best_cost) {
       best_cost = cost;
+      best_tiles = tiles;
+      best_len = 2 * waves * (tiles + 3);
       best.S = used;
       best.chunk = chunk;
     }
@@ -1429,6 +1452,8 @@ Split choose_split(int dev, int span, bool tree_tile, int n_rb, long w_max, int 
       const long cost = 2 + 2 * (tiles + 5);
       if (cost <= best_cost) {
         best_cost = cost;
+        best_tiles = tiles;
+        best_len = 2 * (tiles + 3);
         best.S = used;
         best.chunk = chunk;
         best.coop = true;
@@ -1442,7 +1467,7 @@ Split choose_split(int dev, int span, bool tree_tile, int n_rb, long w_max, int 
     const long n_eff = std::min<long>(capb, std::max<long>(1, w_max / m));
     const long share = (w_max + n_eff - 1) / n_eff;
     const long cost = 2 * ((w_max + (long)kUnitCost * n_rb + n_eff - 1) / n_eff) + (chain ? 26 : 17);
-    if (best_cost < 0 || cost < best_cost) {
+    if (best_cost < 0 || cost < best_cost || (best_tiles > share && 2 * share + 9 < best_len)) {
       best_cost = cost;
       best.bal = true;
       best.coop = true;
@@ -1500,7 +1525,7 @@ ee_status verify_attn(const ee_bf16* q, const ee_bf16* k_tree, const ee_bf16* v_
     return EE_ERR_INVALID_ARG;
   if (ws_bytes < kWorkspaceBytes) return EE_ERR_WORKSPACE;
   if ((int64_t)num_pages * n_kv * EE_PAGE >= ((int64_t)1 << 31)) return EE_ERR_UNSUPPORTED;
-  // a CTA stages at most kMaxCtaPages page ids, and a cluster holds at most 8 chunks
+  // the plans' limits: kMaxCtaPages pages a chunk, 8 chunks in a cluster
   if (span > (int64_t)kMaxCluster * kMaxCtaPages * EE_PAGE) return EE_ERR_UNSUPPORTED;
 
   int dev = 0;

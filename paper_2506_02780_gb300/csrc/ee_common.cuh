@@ -34,9 +34,10 @@ constexpr size_t kNeverSetOff = 32;
 constexpr size_t kArgmaxOff = 256;
 constexpr size_t kWorkspaceBytes = 256 + 8 * (size_t)EE_MAX_LM_NODES + 256;   // the fixed head
 constexpr int kNumSMsMax = 152;       // LM-head grid bound (one persistent CTA per SM)
-// LM-head verification partials (ee_lmhead_verify): per CTA and node of its
-// node tile, the CTA's top-k (value, id) list and its (max, sum) of 2^logit;
-// then the per-node global pruning threshold
+// LM-head verification partials (ee_lmhead_verify): per node and CTA of its
+// node tile (a node's records side by side: one warp reads them all), the CTA's
+// top-k (value, id) list and its (max, sum) of 2^logit; then the per-node
+// global pruning threshold
 constexpr int kLmMaxK = 8;
 constexpr int kLmMaxBN = 256;
 constexpr size_t kLmVerifyOff = kWorkspaceBytes;

@@ -10,10 +10,13 @@
 //     D[vocab_row][node] accumulates in fp32 in TMEM, never in registers and
 //     never in HBM (unless the caller asks for the logits).
 //   - Warp 0 (one lane) streams W and X tiles with TMA (128B swizzle) into a
-//     STAGES-deep shared-memory ring guarded by mbarriers; warp 1 (one lane)
-//     issues tcgen05.mma.kind::f16 (bf16 x bf16 -> fp32) and commits each
-//     stage back to the producer; two TMEM accumulators let the epilogue drain
-//     tile i while tile i+1 accumulates.
+//     STAGES-deep shared-memory ring guarded by mbarriers; warp 1 walks the
+//     k-blocks and one elected lane issues tcgen05.mma.kind::f16 (bf16 x bf16 ->
+//     fp32; elected, so that the descriptors stay in uniform registers: a lane
+//     test costs a move per operand) and commits each stage back to the producer;
+//     two TMEM accumulators let the epilogue drain tile i while tile i+1
+//     accumulates.  Above 256 nodes two CTAs of a cluster share every MMA (the
+//     pair rule at the launch).
 //   - Warps 2..9 (the epilogue, two per TMEM lane quarter taking alternate
 //     16-column chunks) read the accumulator with tcgen05.ld (one TMEM lane =
 //     one vocabulary row per thread) and reduce each node's column to (max,
@@ -35,7 +38,12 @@
 //   - The producer thread issues the ring's first stages right after it
 //     initialises the barriers, before the set-up barrier.
 //   - The kernel is bound by streaming W from HBM when the node count is below
-//     the ridge point (~250), by the tensor pipe above it.
+//     the ridge point (~250), by the tensor pipe above it.  Measured: V = 152064,
+//     H = 3584, 64 nodes, tile-ordered W 166 us (6.6 TB/s); 534 nodes 353 us (1,650
+//     TFLOP/s; a CTA of its own per MMA 395 us); V = 32256, H = 7168, 128 nodes,
+//     logits kept 86.7 us.  With the verification rules (k = 5, 64 nodes) 185 us,
+//     266 before the top-K lists sat one entry a lane, the K best came from warp
+//     maxima and the log-sum-exp took one maximum a tile.
 // Every mbarrier wait is bounded (2e9 SM cycles, about 1 s); on expiry the CTA sets
 // EE_DEVERR_TIMEOUT, drains its own copies and MMAs (again bounded), frees its
 // TMEM and returns.
@@ -81,7 +89,7 @@ struct LmParams {
   int32_t* topk_ids;          // [total][K] or NULL
   int32_t* tau_out;           // [total] or NULL
   float* h_out;               // [total] or NULL
-  uint8_t* part;              // per-CTA partials (workspace), BN * (8 K + 8) bytes per CTA
+  uint8_t* part;              // partials (workspace): lm_rec_bytes(K) per node and source CTA, node by node
   unsigned long long* gthr;   // [EE_MAX_LM_NODES] best K-th key published by any CTA (workspace)
 };
 
@@ -821,7 +829,8 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
 
 // ---------------------------------------------------------------------------
 // Verification finalize (second launch of ee_lmhead_verify): one warp per node
-// merges the per-CTA partials of the LM head -- its K best (logit, id) over the
+// (bound by its scattered record loads; see nodes per CTA at the launch) merges
+// the per-CTA partials of the LM head -- its K best (logit, id) over the
 // whole vocabulary and the log-sum-exp -- computes H_norm of Eq. (entropy) and
 // top_tau, writes the ranked ids and top_tau to the workspace; the last CTA to
 // finish runs the acceptance and zeroes the pruning thresholds.
@@ -1094,7 +1103,7 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
   // M = 256) load 128 rows of W and BN / 2 rows of X each, 32 KB in the 512 cycles,
   // and the ring holds six k-blocks instead of four.  With one node tile the weight
   // stream from HBM is the bound (161 us for 64 nodes at 7B shapes) and the plain
-  // CTA reaches it.
+  // CTA reaches it.  534 nodes, V = 152064, H = 3584: 395 us alone, 353 paired.
   const bool pair = p.n_nt > 1;
   const int bn_step = pair ? 32 : 16;
   p.BN = ((total_nodes + p.n_nt - 1) / p.n_nt + bn_step - 1) / bn_step * bn_step;
