@@ -66,12 +66,13 @@ def parse_args():
 # DRAM bytes (read + write) per launch from one ncu capture of the kernel as it
 # now stands (profiles/ names the capture); a kernel changed since has no entry.
 TRAFFIC = {
-    ("tree_verify_attn", "7b"): 9062144,          # profiles/attn_tc_7b.md
-    ("tree_verify_attn", "33b"): 161879296,       # profiles/attn_tc_33b.md
-    ("tree_verify_attn", "batched"): 246827008,   # profiles/attn_tc_batched.md
-    ("lmhead_accept", "7b"): 1096552192,          # profiles/lmhead_accept_7b.md
-    ("lmhead_accept", "long"): 1107782912,        # profiles/lmhead_accept_long.md
-    ("chain_verify_attn", "long"): 30021120,      # profiles/attn_chain_long.md
+    ("tree_verify_attn", "7b"): 9063936,          # profiles/attn_tc_7b.md
+    ("tree_verify_attn", "33b"): 156175616,       # profiles/attn_tc_33b.md
+    ("tree_verify_attn", "batched"): 238391808,   # profiles/attn_tc_batched.md
+    ("lmhead_accept", "7b"): 1096135936,          # profiles/lmhead_accept_7b.md
+    ("lmhead_accept", "batched"): 1097998336,     # profiles/lmhead_accept_7b.md
+    ("lmhead_accept", "long"): 1108000000,        # profiles/lmhead_accept_long.md
+    ("chain_verify_attn", "long"): 28163328,      # profiles/attn_chain_long.md
 }
 
 
