@@ -15,7 +15,7 @@
 //     fp32; elected, so that the descriptors stay in uniform registers: a lane
 //     test costs a move per operand) and commits each stage back to the producer;
 //     two TMEM accumulators let the epilogue drain tile i while tile i+1
-//     accumulates.  Above 256 nodes two CTAs of a cluster share every MMA (the
+//     accumulates.  With many nodes two CTAs of a cluster share every MMA (the
 //     pair rule at the launch).
 //   - Warps 2..9 (the epilogue, two per TMEM lane quarter taking alternate
 //     16-column chunks) read the accumulator with tcgen05.ld (one TMEM lane =
@@ -41,7 +41,7 @@
 //     the ridge point (~250), by the tensor pipe above it.  Measured: V = 152064,
 //     H = 3584, 64 nodes, tile-ordered W 166 us (6.6 TB/s); 534 nodes 353 us (1,650
 //     TFLOP/s; a CTA of its own per MMA 395 us); V = 32256, H = 7168, 128 nodes,
-//     logits kept 86.7 us.  With the verification rules (k = 5, 64 nodes) 185 us,
+//     logits kept 83 us.  With the verification rules (k = 5, 64 nodes) 185 us,
 //     266 before the top-K lists sat one entry a lane, the K best came from warp
 //     maxima and the log-sum-exp took one maximum a tile.
 // Every mbarrier wait is bounded (2e9 SM cycles, about 1 s); on expiry the CTA sets
@@ -1096,15 +1096,22 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
   p.B = B;
   p.max_T = max_T;
   p.n_nt = (total_nodes + 255) / 256;
-  // Pair rule: with several node tiles (more than 256 nodes) the kernel is bound
-  // by the tensor pipe, but a CTA of its own loads 128 rows of W and BN rows of X
-  // per k-block, 48 KB at BN = 256, through an L2-to-SM port of 64 bytes a cycle:
-  // 768 cycles against 512 of MMA.  Two CTAs that share their MMAs (cta_group::2,
-  // M = 256) load 128 rows of W and BN / 2 rows of X each, 32 KB in the 512 cycles,
-  // and the ring holds six k-blocks instead of four.  With one node tile the weight
-  // stream from HBM is the bound (161 us for 64 nodes at 7B shapes) and the plain
-  // CTA reaches it.  534 nodes, V = 152064, H = 3584: 395 us alone, 353 paired.
-  const bool pair = p.n_nt > 1;
+  // Pair rule.  A CTA of its own loads 128 rows of W and BN rows of X per k-block
+  // (48 KB at BN = 256) through an L2-to-SM port of 64 bytes a cycle; two CTAs that
+  // share their MMAs (cta_group::2, M = 256) load 128 rows of W and BN / 2 rows of X
+  // each.  Many nodes make that port the bound (768 cycles a k-block at BN = 256
+  // against 512 of MMA or 643 of the weight stream), and the larger stages leave
+  // fewer bytes of W in flight (4 k-blocks of 128 rows instead of 6).  A pair starts
+  // about 0.8 us later and each of its tiles ends later, which a short hidden
+  // dimension does not repay.  Measured alone -> paired, us:
+  //   H = 3584, V = 152064: 64 nodes 159.0 -> 159.6, 96: 160.9 -> 160.4, 128: 164.7 ->
+  //   161.5, 192: 175.4 -> 166.5, 256: 217 -> 176 (tile-ordered W: 211 -> 172), 534:
+  //   395 -> 353; H = 7168, V = 32256: 96 nodes 77.0 -> 76.8, 128: 79.3 -> 78.0, 256:
+  //   108.8 -> 86.2;
+  //   H = 2048, V = 32256: 112 nodes 29.6 -> 30.1, 160: 31.9 -> 31.3, 224: 37.5 -> 33.6;
+  //   V = 16384: 160 nodes 21.7 -> 22.5, 224: 24.9 -> 23.6;
+  //   H = 512, V = 32256: 112 nodes 13.7 -> 14.8, 512: 30.1 -> 31.7, 1024: 52.5 -> 56.7.
+  const bool pair = hidden_dim >= 2048 && total_nodes > (hidden_dim >= 3072 ? 96 : 192);
   const int bn_step = pair ? 32 : 16;
   p.BN = ((total_nodes + p.n_nt - 1) / p.n_nt + bn_step - 1) / bn_step * bn_step;
   // vocabulary tiles: as many per CTA for every CTA (the launch's end is the

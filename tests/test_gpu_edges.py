@@ -1,8 +1,8 @@
 """GPU parity at the sizes where the attention's segments and merges and the LM
 head's CTA pairs and top-K lists can go wrong: CTAs that walk more segments than
 the published ring holds, row blocks of a few rows split over many CTAs, a row of
-NaN scores, node counts just above one node tile, odd numbers of vocabulary
-tiles, list quarters with fewer rows than k.  References and tolerances are those
+NaN scores, node counts around one node tile and the pair rule, odd numbers of
+vocabulary tiles, list quarters with fewer rows than k.  References and tolerances are those
 of the other parity tests (the fp64 oracle; parity_util)."""
 import numpy as np
 import pytest
@@ -124,11 +124,14 @@ def test_nan_scores_stay_in_their_row(ctxs):
     assert torch.equal(got[keep], clean[keep])
 
 
-@pytest.mark.parametrize("nodes,vocab,hidden,packed", [(256, 4100, 512, True), (257, 4100, 520, False),
-                                                       (288, 4097, 512, True), (513, 4224, 512, True),
-                                                       (1025, 4100, 64, False)])
-def test_lmhead_around_one_node_tile(nodes, vocab, hidden, packed):
-    """256 nodes (one tile, a CTA of its own) and just above (CTA pairs), with odd
+@pytest.mark.parametrize("nodes,vocab,hidden,packed", [(256, 4100, 512, True), (513, 4097, 520, False),
+                                                       (1025, 4100, 64, False), (96, 4100, 3584, True),
+                                                       (97, 4100, 3592, False), (192, 4097, 2048, True),
+                                                       (193, 4097, 2048, True), (256, 8320, 3584, False),
+                                                       (257, 4100, 2056, False), (513, 4224, 2048, True)])
+def test_lmhead_around_the_pair_line(nodes, vocab, hidden, packed):
+    """Node counts and hidden sizes on both sides of the lines between CTAs of
+    their own and CTA pairs, one node tile (up to 256 nodes) and several, with odd
     numbers of 128-row vocabulary tiles: argmax, longest prefix and logits."""
     import paper_2506_02780_gb300 as E
     w = W.build("long", seed=74, device="cuda", layers=1, vocab=vocab, hidden=hidden, n_q=8, n_kv=2,
@@ -158,10 +161,12 @@ def test_lmhead_around_one_node_tile(nodes, vocab, hidden, packed):
     np.testing.assert_array_equal(bonus.cpu().numpy(), rb)
 
 
-@pytest.mark.parametrize("mode,k", [("entropy", 5), ("topk", 8)])
-def test_verify_above_one_node_tile(mode, k):
-    """15 trees of 20 nodes: the verification rules on CTA pairs."""
-    w = W.build("tiny", seed=75, device="cuda", verify_plant=True, trees=[V.TREE] * 15)
+@pytest.mark.parametrize("mode,k,hidden,trees", [("entropy", 5, 3584, 6), ("entropy", 5, 2048, 15),
+                                                 ("topk", 8, 2048, 15), ("topk", 8, 512, 15)])
+def test_verify_with_many_nodes(mode, k, hidden, trees):
+    """6 or 15 trees of 20 nodes: the verification rules on CTA pairs with one and
+    with two node tiles, and on CTAs of their own with two."""
+    w = W.build("tiny", seed=75, device="cuda", hidden=hidden, verify_plant=True, trees=[V.TREE] * trees)
     V._check(w, V._run(w, mode, k), mode, k)
 
 
