@@ -41,9 +41,10 @@
 //     the ridge point (~250), by the tensor pipe above it.  Measured: V = 152064,
 //     H = 3584, 64 nodes, tile-ordered W 166 us (6.6 TB/s); 534 nodes 353 us (1,650
 //     TFLOP/s; a CTA of its own per MMA 395 us); V = 32256, H = 7168, 128 nodes,
-//     logits kept 83 us.  With the verification rules (k = 5, 64 nodes) 185 us,
-//     266 before the top-K lists sat one entry a lane, the K best came from warp
-//     maxima and the log-sum-exp took one maximum a tile.
+//     logits kept 83 us.  With the verification rules (k = 5, 64 nodes) 176 us,
+//     266 at first: the top-K lists sit one entry a lane, the first tile's lists are
+//     picked for 16 columns at once by warp maxima, one short copy of the insertion
+//     code serves all columns, and the log-sum-exp takes one maximum a tile.
 // Every mbarrier wait is bounded (2e9 SM cycles, about 1 s); on expiry the CTA sets
 // EE_DEVERR_TIMEOUT, drains its own copies and MMAs (again bounded), frees its
 // TMEM and returns.
@@ -527,15 +528,13 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
       // warp-uniform outcome: the tcgen05.ld below is warp-collective
       if (!__all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * acc, acc_phase, &s_abort))) break;
       tc_fence_after();
-      if (kVerify) {
-        // fold the other CTAs' published K-th keys into the shared threshold (a
-        // stale value only lets more rows through)
-        for (int c = threadIdx.x - 64; c < BN; c += kEpiThreads)
-          if (nt * BN + c < p.total_nodes) atomicMax(&s_thr[c], __ldcg(p.gthr + nt * BN + c));
-      }
       const int row = vt * p.BMr + q * 32 + lane;
       const bool row_ok = q * 32 + lane < p.BMr && row < p.vocab;
       for (int c0 = 16 * half; c0 < BN; c0 += 32) {
+        // the best K-th keys the other CTAs have published for the 16 columns (a
+        // stale value only lets more rows through); used after the two reductions
+        unsigned long long gkey = 0ull;
+        if (kVerify && lane < 16 && nt * BN + c0 + lane < p.total_nodes) gkey = __ldcg(p.gthr + nt * BN + c0 + lane);
         uint32_t r[16];
         tc_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + c0), r);
         float v[16];
@@ -613,25 +612,73 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
           }
           __syncwarp();
           // (2) top-K per node column: a row is a candidate when its key beats the
-          //     CTA's shared threshold.  Lane k holds entry k of the warp's sorted
-          //     list; a candidate's place is the number of better entries (one
-          //     ballot) and the worse ones move down one lane.  An empty list (the
-          //     first tile, where every row is a candidate) takes its K best by K
-          //     warp maxima, the lowest lane, i.e. row, first among equals.  (With
-          //     lane 0 inserting in shared memory and two warp reductions per pick
-          //     the first tile's epilogue outlasted two tiles' weight streams.)
+          //     CTA's shared threshold.  The 16 columns' tests go first, independent
+          //     of one another; after the first tiles almost no column has any.
+          //     Every warp folds the published keys in itself: with one warp doing it
+          //     the others tested against stale ones and inserted for nothing.
+          if (lane < 16 && gkey > s_thr[c0 + lane]) atomicMax(&s_thr[c0 + lane], gkey);
+          __syncwarp();
           const int row0 = vt * p.BMr + q * 32;
+          unsigned cand[16], cols = 0u;   // cols: bit j, column j has candidates
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const bool cand = row_ok && make_key(v0[j], row) > s_thr[c0 + j];
-            unsigned mask = __ballot_sync(0xffffffffu, cand);
-            if (mask == 0u) continue;
+            cand[j] = __ballot_sync(0xffffffffu, row_ok && make_key(v0[j], row) > s_thr[c0 + j]);
+            cols |= cand[j] != 0u ? 1u << j : 0u;
+          }
+          if (lt == 0) {
+            // the CTA's first tile: every list is empty and most rows are
+            // candidates.  K rounds of warp maxima over all 16 columns at once (a
+            // column's round alone is a chain of 100 cycles), the lowest lane, i.e.
+            // row, first among equals; lane j keeps column j's pick
+            uint32_t key[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) key[j] = (cand[j] >> lane & 1u) ? ordered(v0[j]) : 0u;
+            for (int rr = 0; rr < K; ++rr) {
+              uint32_t pick = 0u;
+              int from = 0;
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const uint32_t mx = __reduce_max_sync(0xffffffffu, key[j]);
+                const int src = __ffs(__ballot_sync(0xffffffffu, key[j] == mx)) - 1;
+                if (lane == src) key[j] = 0u;
+                if (lane == j) {
+                  pick = mx;
+                  from = src;
+                }
+              }
+              if (lane < 16 && pick != 0u) {   // (0: fewer candidates than K)
+                const size_t e = (size_t)(ew * BN + c0 + lane) * K + rr;
+                s_lv[e] = unordered(pick);
+                s_li[e] = row0 + from;
+                if (rr == K - 1) atomicMax(&s_thr[c0 + lane], make_key(unordered(pick), row0 + from));
+              }
+            }
+            __syncwarp();
+            cols = 0u;
+          }
+          // Later tiles: lane k holds entry k of the warp's sorted list; a candidate's
+          // place is the number of better entries (one ballot) and the worse ones move
+          // down one lane.  An empty list (its rows of the first tile all below the
+          // threshold) takes its K best by K warp maxima.  One copy of the code for
+          // all columns: unrolled, a CTA with two tiles first met it at its end, and
+          // fetching it took 3 us.
+          while (cols != 0u) {
+            const int j = __ffs(cols) - 1;
+            cols &= cols - 1;
+            float x = v0[0];
+            unsigned mask = cand[0];
+#pragma unroll
+            for (int k = 1; k < 16; ++k)
+              if (k == j) {
+                x = v0[k];
+                mask = cand[k];
+              }
             float* lv = s_lv + (size_t)(ew * BN + c0 + j) * K;
             int* li = s_li + (size_t)(ew * BN + c0 + j) * K;
             float av = lane < K ? lv[lane] : -INFINITY;
             int ai = lane < K ? li[lane] : 0x7fffffff;
             if (__shfl_sync(0xffffffffu, ai, 0) == 0x7fffffff) {
-              uint32_t key = cand ? ordered(v0[j]) : 0u;
+              uint32_t key = (mask >> lane & 1u) ? ordered(x) : 0u;
               for (int rr = 0; rr < K; ++rr) {
                 const uint32_t mx = __reduce_max_sync(0xffffffffu, key);
                 if (mx == 0u) break;   // fewer candidates than K
@@ -646,7 +693,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
               while (mask) {
                 const int src = __ffs(mask) - 1;
                 mask &= mask - 1;
-                const float cv = __shfl_sync(0xffffffffu, v0[j], src);
+                const float cv = __shfl_sync(0xffffffffu, x, src);
                 const int ci = row0 + src;
                 const int pos = __popc(__ballot_sync(0xffffffffu, lane < K && better(av, ai, cv, ci)));
                 const float uv = __shfl_up_sync(0xffffffffu, av, 1);

@@ -170,10 +170,11 @@ def test_verify_with_many_nodes(mode, k, hidden, trees):
     V._check(w, V._run(w, mode, k), mode, k)
 
 
-@pytest.mark.parametrize("vocab", [40, 130, 200])
+@pytest.mark.parametrize("vocab", [40, 130, 200, 29792])
 @pytest.mark.parametrize("k", [2, 8])
 def test_verify_lists_with_few_rows(vocab, k):
     """Lists that a tile fills only in part (a quarter of 32 rows holds 0, 2 or 8
-    of them): top-k ids, entropy and acceptance."""
+    of them; at 29,792 words 2 of a first tile's 98 rows, and a second tile inserts):
+    top-k ids, entropy and acceptance."""
     w = W.build("tiny", seed=76, device="cuda", vocab=vocab)
     V._check(w, V._run(w, "entropy", k), "entropy", k)
