@@ -634,16 +634,20 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
 #pragma unroll
             for (int j = 0; j < 16; ++j) key[j] = (cand[j] >> lane & 1u) ? ordered(v0[j]) : 0u;
             for (int rr = 0; rr < K; ++rr) {
-              uint32_t pick = 0u;
-              int from = 0;
+              uint32_t pick = 0u, mx[16];
+              int from = 0, src[16];
+              // (three loops: the compiler keeps warp-wide operations in order, and
+              // each column's vote would wait for its own maximum)
+#pragma unroll
+              for (int j = 0; j < 16; ++j) mx[j] = __reduce_max_sync(0xffffffffu, key[j]);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) src[j] = __ffs(__ballot_sync(0xffffffffu, key[j] == mx[j])) - 1;
 #pragma unroll
               for (int j = 0; j < 16; ++j) {
-                const uint32_t mx = __reduce_max_sync(0xffffffffu, key[j]);
-                const int src = __ffs(__ballot_sync(0xffffffffu, key[j] == mx)) - 1;
-                if (lane == src) key[j] = 0u;
+                if (lane == src[j]) key[j] = 0u;
                 if (lane == j) {
-                  pick = mx;
-                  from = src;
+                  pick = mx[j];
+                  from = src[j];
                 }
               }
               if (lane < 16 && pick != 0u) {   // (0: fewer candidates than K)
@@ -876,14 +880,18 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
 
 // ---------------------------------------------------------------------------
 // Verification finalize (second launch of ee_lmhead_verify): one warp per node
-// (bound by its scattered record loads; see nodes per CTA at the launch) merges
-// the per-CTA partials of the LM head -- its K best (logit, id) over the
+// merges the per-CTA partials of the LM head -- its K best (logit, id) over the
 // whole vocabulary and the log-sum-exp -- computes H_norm of Eq. (entropy) and
 // top_tau, writes the ranked ids and top_tau to the workspace; the last CTA to
-// finish runs the acceptance and zeroes the pruning thresholds.
+// finish runs the acceptance and zeroes the pruning thresholds.  Latency is all:
+// one round trip for a node's records and, in a kernel of a few microseconds, the
+// fetch of its own code, so the code is short (K = 8, 192 nodes, tiny shapes: 52 us
+// for the call, 65 with the records held in registers).
 // ---------------------------------------------------------------------------
 constexpr int kFinWarps = 8;   // warps of a CTA: the acceptance's
-constexpr int kSurv = 256;   // per warp: entries that can still be among a node's K best
+constexpr int kFinNodes = 4;   // nodes of a CTA at most (48 KB of records at K = 8)
+static_assert(kFinNodes * kNumSMsMax * lm_rec_bytes(kLmMaxK) + 64 <= 48 * 1024, "static shared memory");
+static_assert((EE_MAX_LM_NODES + 4 * kNumSMsMax - 1) / (4 * kNumSMsMax) <= kFinNodes, "nodes per CTA");
 
 struct FinParams {
   int total, B, max_T, n_src, K, mode;
@@ -904,55 +912,29 @@ template <int K>
 __global__ void __launch_bounds__(32 * kFinWarps, 1) lm_verify_finalize_kernel(const FinParams p) {
   ee::pdl_allow_next();
   ee::pdl_wait();   // the LM head's partials, thresholds and argmax are complete
-  __shared__ float s_sv[kFinWarps][kSurv];
-  __shared__ int s_svi[kFinWarps][kSurv];
-  __shared__ int s_svn[kFinWarps];
+  constexpr int kRecBytes = lm_rec_bytes(K);
+  __shared__ __align__(16) uint8_t s_rec[kFinNodes][kNumSMsMax * kRecBytes];
   __shared__ int s_last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int node = blockIdx.x * p.npc + warp;
   if (warp < p.npc && node < p.total) {
-    constexpr int kRec = lm_rec_bytes(K) / 16;   // 16-byte words per (CTA, node) record
-    // the best K-th key any CTA published: at most the node's true K-th best,
-    // so only entries reaching it can be among the K best
-    const unsigned long long g = __ldcg(p.gthr + node);
-    constexpr int kMaxU = (kNumSMsMax + 31) / 32;
-    float cv[kMaxU][K];
-    int ci[kMaxU][K];
+    // the node's records, side by side, into shared memory: all copies in flight,
+    // then short loops over them (held in registers, five sources a lane, the
+    // unrolled code was 10 KB that every launch fetched anew)
+    const uint8_t* rec = s_rec[warp];
+    const char* src = reinterpret_cast<const char*>(p.part + (size_t)node * p.n_src * kRecBytes);
+    for (int i = lane; i < p.n_src * (kRecBytes / 16); i += 32)
+      cp_async16(smem_u32(rec) + 16 * i, src + 16 * (size_t)i, 16u);
+    cp_async_wait_all();
+    __syncwarp();
+    constexpr int kMaxU = (kNumSMsMax + 31) / 32;   // lane l takes source CTAs l, l + 32, ...
     float2 xs[kMaxU];
-    // every record of the node: lane l takes source CTAs l, l + 32, ...; all
-    // loads are unconditional (source 0 stands in for absent ones) and in flight
-    // together, the absent ones masked afterwards
-    uint4 w[kMaxU][kRec];
-#pragma unroll
-    for (int u = 0; u < kMaxU; ++u) {
-      const int q2 = lane + 32 * u;
-      const uint4* rec = reinterpret_cast<const uint4*>(
-          p.part + ((size_t)node * p.n_src + (q2 < p.n_src ? q2 : 0)) * lm_rec_bytes(K));
-#pragma unroll
-      for (int t = 0; t < kRec; ++t) w[u][t] = __ldcg(rec + t);
-    }
-#pragma unroll
-    for (int u = 0; u < kMaxU; ++u) {
-      const uint32_t* ww = reinterpret_cast<const uint32_t*>(w[u]);
-#pragma unroll
-      for (int rr = 0; rr < K; ++rr) {
-        cv[u][rr] = __uint_as_float(ww[rr]);
-        ci[u][rr] = (int)ww[K + rr];
-      }
-      xs[u] = make_float2(__uint_as_float(ww[2 * K]), __uint_as_float(ww[2 * K + 1]));
-    }
     float m = -INFINITY, sm = 0.f;
 #pragma unroll
     for (int u = 0; u < kMaxU; ++u) {
-      const bool valid = lane + 32 * u < p.n_src;
-      if (!valid) xs[u] = make_float2(-INFINITY, 0.f);
+      const int q = lane + 32 * u;
+      xs[u] = q < p.n_src ? *reinterpret_cast<const float2*>(rec + q * kRecBytes + 8 * K) : make_float2(-INFINITY, 0.f);
       m = fmaxf(m, xs[u].x);
-#pragma unroll
-      for (int rr = 0; rr < K; ++rr)
-        if (!valid) {
-          cv[u][rr] = -INFINITY;
-          ci[u][rr] = 0x7fffffff;
-        }
     }
     m = unordered(__reduce_max_sync(0xffffffffu, ordered(m)));
 #pragma unroll
@@ -960,93 +942,33 @@ __global__ void __launch_bounds__(32 * kFinWarps, 1) lm_verify_finalize_kernel(c
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) sm += __shfl_xor_sync(0xffffffffu, sm, d);
     const float lse = m + logf(sm);
-    // survivors into the warp's buffer
-    float* sv = s_sv[warp];
-    int* svi = s_svi[warp];
-    if (lane == 0) s_svn[warp] = 0;
-    __syncwarp();
-#pragma unroll
-    for (int u = 0; u < kMaxU; ++u)
-#pragma unroll
-      for (int rr = 0; rr < K; ++rr)
-        if (ci[u][rr] != 0x7fffffff && make_key(cv[u][rr], ci[u][rr]) >= g) {
-          const int pos = atomicAdd(&s_svn[warp], 1);
-          if (pos < kSurv) {
-            sv[pos] = cv[u][rr];
-            svi[pos] = ci[u][rr];
-          }
-        }
-    __syncwarp();
-    const int n_sv = s_svn[warp];
-    const bool few = n_sv <= kSurv;
-    // overflow (not seen with a published threshold): each lane merges its own
-    // sorted source lists, then the warp takes the K best of the lane heads
-    float lv[K];
-    int li[K];
-#pragma unroll
-    for (int t = 0; t < K; ++t) {
-      lv[t] = -INFINITY;
-      li[t] = 0x7fffffff;
-    }
-    if (!few) {
-#pragma unroll
-      for (int rr = 0; rr < K; ++rr) {
-        int wu = 0;
-        float bv = cv[0][0];
-        int bi = ci[0][0];
-#pragma unroll
-        for (int u = 1; u < kMaxU; ++u)
-          if (better(cv[u][0], ci[u][0], bv, bi)) {
-            wu = u;
-            bv = cv[u][0];
-            bi = ci[u][0];
-          }
-        lv[rr] = bv;
-        li[rr] = bi;
-#pragma unroll
-        for (int u = 0; u < kMaxU; ++u) {
-          if (u != wu) continue;
-#pragma unroll
-          for (int t = 0; t < K - 1; ++t) {
-            cv[u][t] = cv[u][t + 1];
-            ci[u][t] = ci[u][t + 1];
-          }
-          cv[u][K - 1] = -INFINITY;
-          ci[u][K - 1] = 0x7fffffff;
-        }
-      }
-    }
+    // K rounds: each lane offers the best head of its sources' sorted lists, the
+    // warp takes the best of the lanes (4 bits of `heads` per source)
+    uint32_t heads = 0u;
     float hsum = 0.f;   // -sum p ln p over the K best, with ln p = logit - lse
+#pragma unroll 1
     for (int rr = 0; rr < K; ++rr) {
-      float xv;
-      int xi;
-      if (few) {
-        float bv = -INFINITY;
-        int bi = 0x7fffffff, bpos = -1;
-        for (int pos = lane; pos < n_sv; pos += 32)
-          if (better(sv[pos], svi[pos], bv, bi)) {
-            bv = sv[pos];
-            bi = svi[pos];
-            bpos = pos;
-          }
-        warp_best(bv, bi, &xv, &xi);
-        if (bpos >= 0 && bi == xi && bv == xv) {
-          sv[bpos] = -INFINITY;
-          svi[bpos] = 0x7fffffff;
-        }
-        __syncwarp();
-      } else {
-        warp_best(lv[0], li[0], &xv, &xi);
-        if (xi != 0x7fffffff && li[0] == xi && lv[0] == xv) {   // this lane held it: next one up
+      float bv = -INFINITY, xv;
+      int bi = 0x7fffffff, bu = -1, xi;
 #pragma unroll
-          for (int t = 0; t < K - 1; ++t) {
-            lv[t] = lv[t + 1];
-            li[t] = li[t + 1];
-          }
-          lv[K - 1] = -INFINITY;
-          li[K - 1] = 0x7fffffff;
+      for (int u = 0; u < kMaxU; ++u) {
+        const int q = lane + 32 * u;
+        if (q >= p.n_src) continue;
+        const float* lv = reinterpret_cast<const float*>(rec + q * kRecBytes);
+        const int* li = reinterpret_cast<const int*>(lv + K);
+        int h = (int)(heads >> (4 * u) & 15u);
+        while (h < K && lv[h] != lv[h]) {   // a NaN is never ranked
+          ++h;
+          heads += 1u << (4 * u);
+        }
+        if (h < K && better(lv[h], li[h], bv, bi)) {
+          bv = lv[h];
+          bi = li[h];
+          bu = u;
         }
       }
+      warp_best(bv, bi, &xv, &xi);
+      if (bu >= 0 && bi == xi && bv == xv) heads += 1u << (4 * bu);   // this lane held it
       const float pr = ex2f((xv - lse) * kLog2e);
       if (pr > 0.f) hsum += pr * (lse - xv);
       if (lane == 0) {
@@ -1272,7 +1194,7 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
     // nodes per CTA (one warp each): one while the CTAs fit on the GPU a few at a
     // time -- a node's 152 records are scattered loads, and eight warps of them on
     // one SM took 9 us longer than one (64 nodes, k = 5: 195.5 us against 184.9)
-    fp.npc = std::max(1, std::min(kFinWarps, (total_nodes + 4 * ee::kNumSMs - 1) / (4 * ee::kNumSMs)));
+    fp.npc = std::max(1, std::min(kFinNodes, (total_nodes + 4 * ee::kNumSMs - 1) / (4 * ee::kNumSMs)));
     const dim3 fg((total_nodes + fp.npc - 1) / fp.npc), fb(32 * kFinWarps);
     cudaError_t fe = cudaErrorInvalidValue;
     switch (K) {
