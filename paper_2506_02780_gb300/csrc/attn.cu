@@ -478,21 +478,23 @@ __device__ __forceinline__ void load_q(const AttnParams& p, const Seg& s, uint32
   int h = rr - nd * g;
   const char* base =
       reinterpret_cast<const char*>(p.q + ((size_t)s.o * p.n_q + s.hk * g) * kD + 8 * j);
-  uint32_t off = ((uint32_t)nd * p.n_q + h) * (kD * 2);   // bytes; below 2048 * n_q * 256
+  // (node, head) as a row number, scaled to bytes in 64 bits: 2048 nodes of more than
+  // 8192 heads pass 4 GiB (2^32 rows would be 1 TB)
+  uint32_t row = (uint32_t)nd * p.n_q + h;
   const int dn = kStep / g, dh = kStep - dn * g;          // kStep rows = dn nodes and dh heads
-  const uint32_t step = ((uint32_t)dn * p.n_q + dh) * (kD * 2), wrap = (uint32_t)(p.n_q - g) * (kD * 2);
+  const uint32_t step = (uint32_t)dn * p.n_q + dh, wrap = (uint32_t)(p.n_q - g);
   const uint32_t dst = sQ + (j >> 3) * kKVHalf;
-#pragma unroll
+#pragma unroll 16   // (all 64 rows of a later row block: the balanced kernels spill)
   for (int k = 0; k < kCount; ++k) {
     const bool in = rq < left;
-    cp_async16(dst + (rq >> 3) * 1024 + (rq & 7) * 128 + (((j & 7) ^ (rq & 7)) << 4), base + (in ? off : 0u),
-               in ? 16u : 0u);
+    cp_async16(dst + (rq >> 3) * 1024 + (rq & 7) * 128 + (((j & 7) ^ (rq & 7)) << 4),
+               base + (size_t)(in ? row : 0u) * (kD * 2), in ? 16u : 0u);
     rq += kStep;
-    off += step;
+    row += step;
     h += dh;
     if (h >= g) {
       h -= g;
-      off += wrap;
+      row += wrap;
     }
   }
   cp_async_wait_all();

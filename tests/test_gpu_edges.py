@@ -124,6 +124,31 @@ def test_nan_scores_stay_in_their_row(ctxs):
     assert torch.equal(got[keep], clean[keep])
 
 
+def test_query_offsets_beyond_four_gib():
+    """A causal draft of 2,048 nodes with 8,320 query heads: the byte offset of a
+    node's query rows passes 2^32 from node 2,017 on.  Sampled rows on both sides
+    against fp64."""
+    import paper_2506_02780_gb300 as E
+    T, n_q, n_kv = 2048, 8320, 65
+    gen = torch.Generator(device="cuda").manual_seed(77)
+    bf = dict(dtype=torch.bfloat16, device="cuda")
+    q = torch.empty((T, n_q, 128), **bf).normal_(generator=gen)
+    assert 2016 * n_q * 256 < 2**32 <= 2017 * n_q * 256
+    kc, vc = (torch.empty((T // 16, n_kv, 16, 128), **bf).normal_(generator=gen) for _ in range(2))
+    i32 = dict(dtype=torch.int32, device="cuda")
+    bt = torch.arange(T // 16, **i32).view(1, -1)
+    out = torch.full((T, n_q, 128), float("nan"), device="cuda")
+    ws = E.new_workspace(1, T, 1, 0)      # no partial slots: one CTA per row block
+    E.ee_chain_verify_attn(q, kc, vc, bt, torch.zeros(1, **i32), 0, torch.tensor([0, T], **i32), T, 128**-0.5, out, ws)
+    torch.cuda.synchronize()
+    assert E.ee_read_errors(ws) == 0
+    for node in (0, 1000, 2016, 2017, 2047):
+        for head in (0, 4099, n_q - 1):
+            k, v = (c[:, head * n_kv // n_q].reshape(T, 128)[:node + 1].double() for c in (kc, vc))
+            ref = torch.softmax(k @ q[node, head].double() * 128**-0.5, 0) @ v
+            U.assert_close(out[node, head].cpu().numpy(), ref.cpu().numpy(), f"node {node} head {head}")
+
+
 @pytest.mark.parametrize("nodes,vocab,hidden,packed", [(256, 4100, 512, True), (513, 4097, 520, False),
                                                        (1025, 4100, 64, False), (96, 4100, 3584, True),
                                                        (97, 4100, 3592, False), (192, 4097, 2048, True),
