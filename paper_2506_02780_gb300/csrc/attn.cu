@@ -745,6 +745,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
       return false;
     }
   };
+  // the same without a wait: segment nseg + 1 is known to be published
+  auto next_published = [&]() -> bool {
+    if constexpr (kBal) {
+      tb += sg.n_tiles;
+      ++nseg;
+      sg = s_seg[nseg % kSegRing];
+      return sg.n_tiles > 0;
+    } else {
+      return false;
+    }
+  };
 
   // Uniform launches: the merge keeps 32 loads a thread in flight, so the softmax
   // warps, which run it, take registers from the others (the shares add up to the
@@ -876,14 +887,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
             }
           }
         }
-        if (kBal && isK) {
-          tb += sg.n_tiles;
-          ++nseg;
-          sg = s_seg[kBal ? nseg % kSegRing : 0];
-          more = sg.n_tiles > 0;
-        } else {
-          more = next();
-        }
+        more = kBal && isK ? next_published() : next();
       }
     } else if (warp == kWarpQk) {
       // ---------------- S = Q K^T, up to kSB tiles ahead of P.V ----------------
@@ -1000,8 +1004,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   // shared memory at a 64-thread named barrier, so both halves take the same
   // rescale decisions; each keeps the sum over its own keys, and the two sums
   // are added (half 0 first) at the end.  Two warps per sub-partition hide
-  // each other's latencies.  Every exit from the tile loop happens right
-  // after the pair barrier and on a decision both warps share.
+  // each other's latencies.  Every exit, from the tile loop and from the walk
+  // of the segments, happens right after the pair barrier and on a decision both
+  // warps share: a bounded wait can end differently in the two (one sees the
+  // abort flag, the other its barrier complete), and a warp that left alone
+  // would leave its partner at the pair barrier for good.
   const int qd = warp & 3;
   const int hf = (warp - kWarpSoft0) >> 2;
   const uint32_t pair_bar = 2 + qd;
@@ -1010,7 +1017,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
   const float sl2 = p.scale_log2;
   bool ok = true;
   bool loaded = false;
-  for (bool more = first(false); more && ok; more = next()) {
+  for (bool more = first(false); more && ok; more = next_published()) {
     const int R = sg.T * g;
     const int rr = sg.rb * kRows + r;
     const bool vrow = rr < R;
@@ -1192,7 +1199,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
     // columns out: O / l itself when the segment is a whole row block, else the
     // partial (O, m, l) to the segment's slot
     const int tl_g = tb + sg.n_tiles - 1;
-    const bool have = ok && sg.n_tiles > 0 && wait(pv_done + 8 * (tl_g % kSB), tl_g / kSB);
+    // (balanced: with the next segment received, or an exit both share)
+    const bool have = ok && sg.n_tiles > 0 && wait(pv_done + 8 * (tl_g % kSB), tl_g / kSB) &&
+                      (!kBal || wait(seg_full + 8 * ((nseg + 1) % kSegRing), (nseg + 1) / kSegRing));
     s_xl[hf][r] = l;
     if (lane == 0) s_xok[nseg & 1][qd][hf] = have;
     asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
