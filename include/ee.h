@@ -270,10 +270,12 @@ ee_status ee_tree_verify_attn_inplace(const ee_bf16* q, const ee_bf16* k_cache, 
  * Optional outputs (NULL to skip): topk_ids int32 [total_nodes][k] ranked
  * token ids; top_tau int32 [total_nodes] the number of leading ranks an edit
  * child may hold (greedy 1, top-k k, entropy top_tau, direct 0 = any);
- * h_norm fp32 [total_nodes] (0 when k = 1).  Logits, the log-sum-exp and
- * H_norm are fp32.  The workspace must hold ee_workspace_size(...) bytes
- * (per-CTA partials of the top-k lists live there).  EE_ERR_INVALID_ARG for a
- * bad mode or k; otherwise as ee_lmhead_accept.
+ * h_norm fp32 [total_nodes] (0 when k = 1).  A rank without a token (fewer
+ * than k logits that are numbers) holds INT32_MAX; a node with a NaN logit has
+ * h_norm 0, hence top_tau 1.  Logits, the log-sum-exp and H_norm are fp32.  The
+ * workspace must hold ee_workspace_size(...) bytes (per-CTA partials of the
+ * top-k lists live there).  EE_ERR_INVALID_ARG for a bad mode or k; otherwise
+ * as ee_lmhead_accept.
  */
 typedef enum {
   EE_VERIFY_GREEDY = 0,
@@ -313,7 +315,8 @@ ee_status ee_attn_plan(int32_t B, int32_t max_T, int32_t n_q, int32_t n_kv, int3
  * ee_lmhead_accept -- LM head fused with greedy decode and acceptance
  * (Eq. (piecewise)).  logits[i][v] = hidden[i] . lm_w[v] (fp32 accumulate of
  * bf16 products, never stored unless logits_or_null is given);
- * argmax[i] = the highest logit, lowest token id on ties.  Node i (i > 0) is
+ * argmax[i] = the highest logit, lowest token id on ties; a NaN logit is never
+ * chosen or ranked (-1 when all of a node's are NaN).  Node i (i > 0) is
  * accepted when every edge a -> b on its root path has draft_tok[b] ==
  * argmax[a]; the deepest accepted node u* wins (lowest local id among equally
  * deep ones):

@@ -128,6 +128,10 @@ __device__ __forceinline__ unsigned long long make_key(float v, int idx) {
 __device__ __forceinline__ bool better(float v, int i, float w, int j) {
   return v > w || (v == w && i < j);
 }
+// the same where either value can be NaN: a NaN loses to every number
+__device__ __forceinline__ bool better_or_nan(float v, int i, float w, int j) {
+  return better(v, i, w, j) || w != w;
+}
 
 __device__ __forceinline__ float unordered(uint32_t k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
@@ -530,6 +534,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
       tc_fence_after();
       const int row = vt * p.BMr + q * 32 + lane;
       const bool row_ok = q * 32 + lane < p.BMr && row < p.vocab;
+      const int row_id = row_ok ? row : 0x7fffffff;   // a dropped row is never chosen
       for (int c0 = 16 * half; c0 < BN; c0 += 32) {
         // the best K-th keys the other CTAs have published for the 16 columns (a
         // stale value only lets more rows through); used after the two reductions
@@ -544,7 +549,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
         for (int j = 0; j < 16; ++j) {
           v[j] = row_ok ? __uint_as_float(r[j]) : -INFINITY;
           v0[j] = v[j];
-          id[j] = row;
+          id[j] = row_id;
         }
         if (p.logits != nullptr && row_ok) {
 #pragma unroll
@@ -565,7 +570,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
             const int give_i = upper ? id[j] : id[j + half];
             const float ov = __shfl_xor_sync(0xffffffffu, give_v, bit);
             const int oi = __shfl_xor_sync(0xffffffffu, give_i, bit);
-            const bool take = better(ov, oi, keep_v, keep_i);
+            const bool take = better_or_nan(ov, oi, keep_v, keep_i);
             v[j] = take ? ov : keep_v;
             id[j] = take ? oi : keep_i;
           }
@@ -573,7 +578,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
         {
           const float ov = __shfl_xor_sync(0xffffffffu, v[0], 1);
           const int oi = __shfl_xor_sync(0xffffffffu, id[0], 1);
-          if (better(ov, oi, v[0], id[0])) {
+          if (better_or_nan(ov, oi, v[0], id[0])) {
             v[0] = ov;
             id[0] = oi;
           }
@@ -592,7 +597,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const float cm = __shfl_sync(0xffffffffu, v[0], lane_of_col(j));
-            e[j] = cm == -INFINITY ? 0.f : ex2f((v0[j] - cm) * kLog2e);
+            e[j] = v0[j] == -INFINITY ? 0.f : ex2f((v0[j] - cm) * kLog2e);
           }
 #pragma unroll
           for (int half = 8, bit = 16; half >= 1; half >>= 1, bit >>= 1) {
@@ -607,22 +612,23 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
           e[0] += __shfl_xor_sync(0xffffffffu, e[0], 1);
           if ((lane & 1) == 0) {
             float2 cur = s_lse[ew * BN + c0 + col];
-            lse_add(cur.x, cur.y, v[0], e[0]);
+            lse_add(cur.x, cur.y, e[0] == e[0] ? v[0] : e[0], e[0]);   // a NaN logit makes the sum NaN
             s_lse[ew * BN + c0 + col] = cur;
           }
           __syncwarp();
-          // (2) top-K per node column: a row is a candidate when its key beats the
-          //     CTA's shared threshold.  The 16 columns' tests go first, independent
-          //     of one another; after the first tiles almost no column has any.
-          //     Every warp folds the published keys in itself: with one warp doing it
-          //     the others tested against stale ones and inserted for nothing.
+          // (2) top-K per node column: a row is a candidate when its logit is a number
+          //     (a NaN's key would beat all) and its key beats the CTA's shared
+          //     threshold.  The 16 columns' tests go first, independent of one another;
+          //     after the first tiles almost no column has any.  Every warp folds the
+          //     published keys in itself: with one warp doing it the others tested
+          //     against stale ones and inserted for nothing.
           if (lane < 16 && gkey > s_thr[c0 + lane]) atomicMax(&s_thr[c0 + lane], gkey);
           __syncwarp();
           const int row0 = vt * p.BMr + q * 32;
           unsigned cand[16], cols = 0u;   // cols: bit j, column j has candidates
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            cand[j] = __ballot_sync(0xffffffffu, row_ok && make_key(v0[j], row) > s_thr[c0 + j]);
+            cand[j] = __ballot_sync(0xffffffffu, row_ok && v0[j] == v0[j] && make_key(v0[j], row) > s_thr[c0 + j]);
             cols |= cand[j] != 0u ? 1u << j : 0u;
           }
           if (lt == 0) {
@@ -956,11 +962,7 @@ __global__ void __launch_bounds__(32 * kFinWarps, 1) lm_verify_finalize_kernel(c
         if (q >= p.n_src) continue;
         const float* lv = reinterpret_cast<const float*>(rec + q * kRecBytes);
         const int* li = reinterpret_cast<const int*>(lv + K);
-        int h = (int)(heads >> (4 * u) & 15u);
-        while (h < K && lv[h] != lv[h]) {   // a NaN is never ranked
-          ++h;
-          heads += 1u << (4 * u);
-        }
+        const int h = (int)(heads >> (4 * u) & 15u);
         if (h < K && better(lv[h], li[h], bv, bi)) {
           bv = lv[h];
           bi = li[h];

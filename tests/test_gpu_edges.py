@@ -203,3 +203,33 @@ def test_verify_lists_with_few_rows(vocab, k):
     top-k ids, entropy and acceptance."""
     w = W.build("tiny", seed=76, device="cuda", vocab=vocab)
     V._check(w, V._run(w, "entropy", k), "entropy", k)
+
+
+@pytest.mark.parametrize("vocab", [4096, 4100, 29792])
+@pytest.mark.parametrize("mode,k", [("topk", 1), ("topk", 8), ("entropy", 5)])
+def test_verify_with_nan_words(vocab, mode, k):
+    """Vocabulary rows of NaN -- beside node 0's best word, in every quarter of a
+    tile, nine in a row (more than a list holds); at 4,100 words the last tile's only
+    four -- and a node whose logits are all NaN (one and two tiles a CTA): no NaN word
+    is chosen or ranked, the other words rank as without them, H_norm is 0 and top_tau 1."""
+    w = W.build("tiny", seed=78, device="cuda", verify_plant=True, trees=[V.TREE], vocab=vocab)
+    lg, err = O.lm_head_logits(w.hidden_states, w.lm_w)
+    best = O.node_ranking(lg[0], 3).tolist()
+    words = {best[0] ^ 1, 3, 40, 70, 100, 161} | set(range(600, 609)) if vocab % 128 != 4 else set(range(4096, 4100))
+    words = sorted(words - set(best))
+    w.lm_w[words] = float("nan")
+    w.hidden_states[5] = float("nan")
+    r = V._run(w, mode, k)
+    assert r["argmax"][5] == -1 and (r["topk"][5] == 2**31 - 1).all()
+    lg[:, words] = -np.inf
+    for a in range(w.total_nodes):
+        if a == 5:
+            continue
+        ids = r["topk"][a]
+        assert r["argmax"][a] == ids[0] and len(set(ids.tolist())) == k and not set(ids.tolist()) & set(words), a
+        e = 2.0 * err[a].max()      # fp32 accumulation: closer words may change places
+        np.testing.assert_allclose(lg[a][ids], lg[a][O.node_ranking(lg[a], k)], atol=e, rtol=0)
+    if mode == "entropy":
+        assert (r["h"] == 0).all() and (r["tau"] == 1).all()
+    g = V._run(w, "greedy", 1, verify=False)
+    np.testing.assert_array_equal(g["argmax"], r["argmax"])
