@@ -41,7 +41,9 @@
 //     operand; V is read straight from shared memory (MN-major).  P is carried
 //     to about 2^-17 relative (fp16 would give 2^-11) and V needs no
 //     conversion.  Per column pair the split is two packing conversions and two
-//     mixed-type subtractions head - p; the MMA negates the tail back.
+//     mixed-type subtractions head - p; the MMA negates the tail back.  The tail's
+//     MMAs go first: each MMA cuts O's lowest bits off, which is the error of long
+//     sums, and before the head's the segment's O is one tile smaller.
 //   - Warps 4-11 own one query row per thread (its TMEM lane), two warps per
 //     lane quarter splitting each tile's keys: they read S, mask, keep the
 //     running max/sum, write P, and rescale O in TMEM only when a row's max
@@ -953,12 +955,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
             const uint32_t pa = tmem + sb * kKT;       // bf16 P head: cols 0..63, tail: 64..127
             const uint64_t dv = dv0 + (uint64_t)(st * (kKVBytes >> 4));
 #pragma unroll
-            for (int part = 0; part < 2; ++part)
+            for (int part = 1; part >= 0; --part)    // the tail first
 #pragma unroll
               for (int j = 0; j < kKT / 16; ++j)
                 tc_mma_ts(tmem + kColO, pa + 64 * part + 8 * j, dv + (uint64_t)(j * (2048 >> 4)),
                           part ? (id_pv | kIdescNegA) : id_pv,
-                          (t > 0 || part > 0 || j > 0) ? 1u : 0u);
+                          (t > 0 || part == 0 || j > 0) ? 1u : 0u);
             tc_commit(pv_done + 8 * sb);
             tc_commit(v_empty + 8 * st);
           }

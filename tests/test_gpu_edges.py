@@ -101,6 +101,28 @@ def test_uniform_plans_beside_the_balanced_line(B, ctx, T, n_q, n_kv, kind):
         U.assert_close(st.attn_out[0].cpu().numpy(), ref, "tree attention")
 
 
+@pytest.mark.parametrize("seed,first,last", [(81, 3.505e-6, 3.685e-6), (82, 3.329e-6, 3.504e-6),
+                                             (83, 3.398e-6, 3.573e-6)])
+def test_long_sums_add_the_tails_first(seed, first, last):
+    """1,500 keys in one CTA, whose accumulator each P.V MMA cuts at its lowest bits: the
+    relative error (2-norm) against fp64 with a tile's tails added before its heads
+    (`first`), not the 5 % larger one of the other order (`last`).  Seeded inputs, sums in
+    a fixed order: the bound is half way between the two."""
+    import paper_2506_02780_gb300 as E
+    from paper_2506_02780_gb300 import step as S
+    w = W.build("tiny", seed=seed, device="cuda", vocab=512, hidden=64, trees=[W.TreeSpec(64, [], [0])], ctxs=[1500])
+    kc, vc = (torch.from_numpy(U.raw16(t).copy()).view(torch.bfloat16) for t in (w.k_cache, w.v_cache))
+    st = S.from_workload(w)
+    st.ws = E.new_workspace(1, 64, 1, 0)      # no partial slots: one CTA per row block
+    st.run()
+    torch.cuda.synchronize()
+    assert E.ee_read_errors(st.ws) == 0
+    anc = O.tree_prepare(w.parent, w.node_off)[1]
+    ref = O.tree_attention(w.q[0], w.k_tree[0], w.v_tree[0], kc[0], vc[0], w.block_table, w.ctx_len, w.node_off, anc)
+    err = np.linalg.norm(st.attn_out[0].cpu().numpy() - ref) / np.linalg.norm(ref)
+    assert err < (first + last) / 2
+
+
 @pytest.mark.parametrize("ctxs", [[512], [2900] * 40])
 def test_nan_scores_stay_in_their_row(ctxs):
     """A query row of NaN (split and balanced launches): its output is NaN, every
