@@ -143,7 +143,7 @@ struct AttnParams {
   float* out;
   uint8_t* part;               // per-CTA partial slots (ee::kAttnPartBytes each), S > 1 only
   int32_t* err;
-  int num_pages, max_pages, max_ctx, n_q, n_kv, g, total_nodes, max_T, nrb, chunk, S;
+  int num_pages, max_pages, max_ctx, n_q, n_kv, g, total_nodes, max_T, chunk, S;
   int coop;                    // 1: cooperative launch, counters; 0: cluster barrier
   int B;                       // sequences (the balanced mode's work list)
   uint32_t g_inv;              // ceil(2^32 / g) for g > 1 (row -> node without a division), 0 for g = 1
@@ -1594,7 +1594,6 @@ ee_status verify_attn(const ee_bf16* q, const ee_bf16* k_tree, const ee_bf16* v_
   p.g = g;
   p.total_nodes = total_nodes;
   p.max_T = max_T;
-  p.nrb = nrb;
   p.chunk = chunk;
   p.S = S;
   p.coop = (S > 1 && sp.coop) || sp.bal ? 1 : 0;

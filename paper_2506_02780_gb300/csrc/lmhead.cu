@@ -67,7 +67,7 @@ constexpr int kEpiThreads = 32 * kEpiWarps;
 constexpr int kABytes = BM * BK * 2;
 
 struct LmParams {
-  int vocab, hidden, total_nodes, B, max_T;
+  int vocab, total_nodes, B, max_T;
   int BN, n_nt, n_vt, nkb, stages, tmem_cols;
   int BMr;                    // vocabulary rows per tile (<= BM; the MMA's other rows are not used)
   int packed;                 // W in tile order ([V/128][H/64][128][64], ee_lmhead_pack_weights): BMr = BM
@@ -85,11 +85,7 @@ struct LmParams {
   unsigned int* ticket;       // CTAs finished (workspace)
   int32_t* err;
   // verification rules (ee_lmhead_verify only)
-  int mode, K;                // EE_VERIFY_*, list length k
-  const uint8_t* gen_mask;    // 1 = edit content (the mode's rule), 0 = reused (greedy); NULL = all 1
-  int32_t* topk_ids;          // [total][K] or NULL
-  int32_t* tau_out;           // [total] or NULL
-  float* h_out;               // [total] or NULL
+  int K;                      // list length k
   uint8_t* part;              // partials (workspace): lm_rec_bytes(K) per node and source CTA, node by node
   unsigned long long* gthr;   // [EE_MAX_LM_NODES] best K-th key published by any CTA (workspace)
 };
@@ -1062,7 +1058,6 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
   LmParams p;
   p.packed = packed ? 1 : 0;
   p.vocab = vocab;
-  p.hidden = hidden_dim;
   p.total_nodes = total_nodes;
   p.B = B;
   p.max_T = max_T;
@@ -1125,12 +1120,7 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
   p.keys = keys;
   p.ticket = ticket;
   p.err = err;
-  p.mode = va ? va->mode : EE_VERIFY_GREEDY;
   p.K = K;
-  p.gen_mask = va ? va->gen_mask : nullptr;
-  p.topk_ids = va ? va->topk_ids : nullptr;
-  p.tau_out = va ? va->tau : nullptr;
-  p.h_out = va ? va->h_norm : nullptr;
   p.part = va ? va->part : nullptr;
   p.gthr = va ? reinterpret_cast<unsigned long long*>(va->part + ee::kLmGthrOff) : nullptr;
 
