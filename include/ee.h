@@ -91,7 +91,8 @@ typedef enum {
 #define EE_DEVERR_PAGE         0x04  /* block_table entry outside [0, num_pages) for a needed slot */
 #define EE_DEVERR_CTX          0x08  /* ctx_len < 0 or above the max_ctx passed by the host */
 #define EE_DEVERR_FP16_RANGE   0x10  /* reserved (no current kernel sets it) */
-#define EE_DEVERR_TIMEOUT      0x20  /* a bounded device wait gave up */
+#define EE_DEVERR_TIMEOUT      0x20  /* a bounded device wait gave up: arrival counts may be left part-way, so the
+                                        next call needs ee_workspace_init first */
 #define EE_DEVERR_PATH         0x40  /* path / accept_len inconsistent with the tree */
 #define EE_DEVERR_OVERFLOW     0x80  /* ee_advance: the committed-token buffer is full */
 
@@ -116,7 +117,8 @@ ee_status ee_workspace_init(void* ws, size_t ws_bytes, ee_stream_t stream);
 
 /*
  * Synchronise `stream`, copy the device error word to *bits (host pointer),
- * clear it on the device.  Returns EE_ERR_DEVICE when any bit was set.
+ * clear it on the device.  Returns EE_ERR_DEVICE when any bit was set.  Only the
+ * error word is cleared: re-initialise the workspace after an error.
  */
 ee_status ee_read_errors(void* ws, ee_stream_t stream, int32_t* bits);
 

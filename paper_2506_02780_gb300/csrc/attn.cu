@@ -106,7 +106,11 @@ constexpr int kVST = 2;                          // V ring depth
 constexpr int kSB = 3;                           // S buffers in TMEM (Q.K^T runs kSB tiles ahead)
 constexpr uint32_t kKVHalf = kKT * 128;          // 16 KB: one 64-dim half of a K or V tile
 constexpr uint32_t kKVBytes = 2 * kKVHalf;       // 32 KB
-constexpr int kMaxCtaPages = 2048;               // context pages of one CTA's share at most (32768 keys)
+// Context pages of one CTA's share at most: 32,768 keys, 256 tiles.  Nothing in shared
+// memory needs the limit; it bounds what one accumulator adds up (the error grows with
+// its tiles) and, with kMaxCluster chunks, sets the 262,144 positions the calls accept.
+// No longer share has been measured.
+constexpr int kMaxCtaPages = 2048;
 constexpr int kUnitCost = 3;                      // balanced: a unit's weight beyond its tiles (see the work list)
 constexpr int kSegRing = 16;                     // published segments (K runs at most 8 ahead of the softmax)
 constexpr int kMaskRing = 8;                     // page-validity masks in flight (K runs at most 6 tiles ahead)
@@ -1151,8 +1155,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
       // p = 2^(s*scale_log2 - m); P = head + tail, both bf16: this
       // half's head pairs go to columns 32 hf.. of the S buffer, its tail pairs
       // to 64 + 32 hf..
-      // (pairs of columns run on packed fp32x2 arithmetic: the scale-and-shift,
-      // the running sums and the tail subtraction take one instruction per pair)
+      // (the scale-and-shift and the running sums take one packed fp32x2
+      // instruction per pair of columns)
       const uint64_t sl2x2 = f2_pack(__float_as_uint(sl2), __float_as_uint(sl2));
       const uint64_t nmsx2 = f2_pack(__float_as_uint(nms), __float_as_uint(nms));
       uint64_t ls2[4];
@@ -1170,8 +1174,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmKc, const __grid_constant__
           const uint32_t p1 = __float_as_uint(ex2(__uint_as_float(y1)));
           const uint64_t pp = f2_pack(p0, p1);
           ls2[e & 3] = e < 4 ? pp : f2_add(ls2[e & 3], pp);
-          // head = p rounded to bf16; tail = the remainder p - head (exact
-          // in fp32) rounded to bf16
+          // head = p rounded to bf16; the negated tail = head - p (exact in fp32)
+          // rounded to bf16, two mixed-type subtractions; the MMA negates it back
           const uint32_t hb = bf16x2_rn(__uint_as_float(p1), __uint_as_float(p0));
           float t0, t1;
           sub_bf16x2(hb, __uint_as_float(p0), __uint_as_float(p1), t0, t1);

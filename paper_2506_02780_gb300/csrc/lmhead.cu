@@ -39,12 +39,13 @@
 //     initialises the barriers, before the set-up barrier.
 //   - The kernel is bound by streaming W from HBM when the node count is below
 //     the ridge point (~250), by the tensor pipe above it.  Measured: V = 152064,
-//     H = 3584, 64 nodes, tile-ordered W 166 us (6.6 TB/s); 534 nodes 353 us (1,650
-//     TFLOP/s; a CTA of its own per MMA 395 us); V = 32256, H = 7168, 128 nodes,
-//     logits kept 83 us.  With the verification rules (k = 5, 64 nodes) 176 us,
-//     266 at first: the top-K lists sit one entry a lane, the first tile's lists are
-//     picked for 16 columns at once by warp maxima, one short copy of the insertion
-//     code serves all columns, and the log-sum-exp takes one maximum a tile.
+//     H = 3584, 64 nodes, tile-ordered W 166 us (6.6 TB/s); 534 nodes 353 us, 345 to
+//     363 over ten runs (1,530 to 1,605 TFLOP/s; a CTA of its own per MMA 395 us); V =
+//     32256, H = 7168, 128 nodes, logits kept 85 us.  With the verification rules
+//     (k = 5, 64 nodes) 177 us: the top-K lists sit one entry a lane, the first
+//     tile's lists are picked for 16 columns at once by warp maxima, one short copy
+//     of the insertion code serves all columns, and the log-sum-exp takes one maximum
+//     a tile.
 // Every mbarrier wait is bounded (2e9 SM cycles, about 1 s); on expiry the CTA sets
 // EE_DEVERR_TIMEOUT, drains its own copies and MMAs (again bounded), frees its
 // TMEM and returns.
@@ -887,8 +888,8 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
 // top_tau, writes the ranked ids and top_tau to the workspace; the last CTA to
 // finish runs the acceptance and zeroes the pruning thresholds.  Latency is all:
 // one round trip for a node's records and, in a kernel of a few microseconds, the
-// fetch of its own code, so the code is short (K = 8, 192 nodes, tiny shapes: 52 us
-// for the call, 65 with the records held in registers).
+// fetch of its own code, so the code is short (K = 8, 192 nodes, 4,096 words x 512: 52 us
+// for the call; with the records in registers, unrolled, it takes 65).
 // ---------------------------------------------------------------------------
 constexpr int kFinWarps = 8;   // warps of a CTA: the acceptance's
 constexpr int kFinNodes = 4;   // nodes of a CTA at most (48 KB of records at K = 8)
@@ -921,8 +922,8 @@ __global__ void __launch_bounds__(32 * kFinWarps, 1) lm_verify_finalize_kernel(c
   const int node = blockIdx.x * p.npc + warp;
   if (warp < p.npc && node < p.total) {
     // the node's records, side by side, into shared memory: all copies in flight,
-    // then short loops over them (held in registers, five sources a lane, the
-    // unrolled code was 10 KB that every launch fetched anew)
+    // then short loops over them (five sources a lane in registers make 10 KB of
+    // unrolled code that every launch fetches anew)
     const uint8_t* rec = s_rec[warp];
     const char* src = reinterpret_cast<const char*>(p.part + (size_t)node * p.n_src * kRecBytes);
     for (int i = lane; i < p.n_src * (kRecBytes / 16); i += 32)
@@ -1135,8 +1136,7 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
     return EE_ERR_CUDA;
 
   const size_t smem = 1024 + (size_t)p.stages * stage_bytes + 8 * (2 * p.stages + 5) + 8 + epi;
-  // the last CTA reuses the pipeline buffers: argmax (+ ranked ids and top_tau) per node
-  // the last CTA: argmax per node and the node offsets
+  // the last CTA keeps the argmax per node and the node offsets in the pipeline buffers
   const size_t last = 1024 + (size_t)(2 * EE_MAX_LM_NODES + 5) * 4;
   const size_t smem_acc = std::max(smem, last);
   if (smem_acc > 227 * 1024) return EE_ERR_UNSUPPORTED;
@@ -1183,9 +1183,11 @@ ee_status launch_lmhead(const ee_bf16* hidden, const ee_bf16* lm_w, int32_t hidd
     fp.ticket = va->fin_ticket;
     fp.acc = AcceptArgs{B, max_T, total_nodes, va->mode, K, node_off, parent, draft_tok, depth, anc,
                         va->gen_mask, accept_len, path, bonus, err};
-    // nodes per CTA (one warp each): one while the CTAs fit on the GPU a few at a
-    // time -- a node's 152 records are scattered loads, and eight warps of them on
-    // one SM took 9 us longer than one (64 nodes, k = 5: 195.5 us against 184.9)
+    // nodes per CTA (one warp each; the other warps are the acceptance's): one while
+    // the CTAs fit on the GPU a few at a time.  One, two or four a CTA are the same at
+    // 64 nodes (V = 152064, k = 5: 175.9, 175.9, 176.1 us for the call); many nodes want
+    // fewer CTAs (V = 4096, H = 512: 576 nodes 47.2, 44.0, 44.0; 1,920: 140.5, 132.9,
+    // 128.8), and four nodes' records are the 48 KB of kFinNodes
     fp.npc = std::max(1, std::min(kFinNodes, (total_nodes + 4 * ee::kNumSMs - 1) / (4 * ee::kNumSMs)));
     const dim3 fg((total_nodes + fp.npc - 1) / fp.npc), fb(32 * kFinWarps);
     cudaError_t fe = cudaErrorInvalidValue;
