@@ -490,7 +490,7 @@ __device__ __forceinline__ void load_q(const AttnParams& p, const Seg& s, uint32
   const int dn = kStep / g, dh = kStep - dn * g;          // kStep rows = dn nodes and dh heads
   const uint32_t step = (uint32_t)dn * p.n_q + dh, wrap = (uint32_t)(p.n_q - g);
   const uint32_t dst = sQ + (j >> 3) * kKVHalf;
-#pragma unroll 16   // (all 64 rows of a later row block: the balanced kernels spill)
+#pragma unroll 8   // (all 64 rows of a later row block: the balanced kernels spill)
   for (int k = 0; k < kCount; ++k) {
     const bool in = rq < left;
     cp_async16(dst + (rq >> 3) * 1024 + (rq & 7) * 128 + (((j & 7) ^ (rq & 7)) << 4),
