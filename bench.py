@@ -67,12 +67,12 @@ def parse_args():
 # now stands (profiles/ names the capture); a kernel changed since has no entry.
 TRAFFIC = {
     ("tree_verify_attn", "7b"): 9063936,          # profiles/attn_tc_7b.md
-    ("tree_verify_attn", "33b"): 156175616,       # profiles/attn_tc_33b.md
-    ("tree_verify_attn", "batched"): 238391808,   # profiles/attn_tc_batched.md
-    ("lmhead_accept", "7b"): 1096135936,          # profiles/lmhead_accept_7b.md
-    ("lmhead_accept", "batched"): 1097998336,     # profiles/lmhead_accept_7b.md
-    ("lmhead_accept", "long"): 1108000000,        # profiles/lmhead_accept_long.md
-    ("chain_verify_attn", "long"): 28163328,      # profiles/attn_chain_long.md
+    ("tree_verify_attn", "33b"): 158343168,       # profiles/attn_tc_33b.md
+    ("tree_verify_attn", "batched"): 238981376,   # profiles/attn_tc_batched.md
+    ("lmhead_accept", "7b"): 1096489984,          # profiles/lmhead_accept_7b.md
+    ("lmhead_accept", "batched"): 1098163456,     # profiles/lmhead_accept_7b.md
+    ("lmhead_accept", "long"): 1108240128,        # profiles/lmhead_accept_long.md
+    ("chain_verify_attn", "long"): 28699904,      # profiles/attn_chain_long.md
 }
 
 

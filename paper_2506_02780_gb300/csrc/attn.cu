@@ -79,11 +79,11 @@
 //     once every CTA has drained its pipeline; triggering earlier lets its
 //     CTAs hold SMs that a later wave of this grid still needs.
 //
-// What bounds it (SM cycles at 2.07 GHz).  Long work: the tile period, 2,000 to
-// 2,040.  A tile's MMAs take 1,536 (24 of 128 x 128 x 16) and about 1,700 with
+// What bounds it (SM cycles at 2.07 GHz).  Long work: the tile period, about
+// 2,000.  A tile's MMAs take 1,536 (24 of 128 x 128 x 16) and about 1,700 with
 // their operand waits; the softmax warps, two per sub-partition, walk the rest:
 // wait for S 140, load and maxima 400, the pair's exchange 165, exponentials,
-// split and stores 1,050 to 1,150, sums and arrival 200.  Tensor pipe 65 % active
+// split and stores 1,050 to 1,150, sums and arrival 200.  Tensor pipe 69 % active
 // (56 heads, 128 nodes, 32,768 keys, one layer: 148 -> 125 us).  A segment switch
 // costs 5,700 more.  Short work: latency.  28 heads, 64 nodes, 4,096 keys, 4 tiles
 // a CTA: 13.3 us, of which 2.8 until the first scores, 4 x 1 for the tiles, 1.3 to
